@@ -25,7 +25,8 @@ constexpr uint32_t kSmemHistMax = 12288;  // items counted in shared memory (48 
 // items).  Only items[0, off[D]) is ever read, whatever the offsets: a
 // transaction whose range is reversed or leaves [0, off[D]] is reported and
 // skipped, and so is every transaction when off[0] != 0.
-// flags = [error bits, longest transaction, off[0], off[D]].
+// flags = [error bits (and DEV_NOTE_REPEATS), longest transaction, off[0], off[D], pairs (u64)], pairs = the sum
+// of len (len - 1) / 2 over the transactions of len distinct items (what counting pairs from the transactions costs).
 constexpr uint32_t kShortTx = 64;
 
 __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* __restrict__ items, uint32_t D,
@@ -43,6 +44,7 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
     flags[3] = nnz;
   }
   uint32_t local_max = 0, local_err = first != 0 ? DEV_ERR_OFFSETS : 0u;
+  uint64_t local_pairs = 0;
   auto bump = [&](uint32_t it) {
     if (use_smem) atomicAdd(&hist[it], 1u);
     else atomicAdd(&cnt[it], 1u);
@@ -76,6 +78,7 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
           if (k > b && !(asc && it > prev)) {
             asc = false;
             for (uint32_t q = b; q < k && !dup; ++q) dup = items[q] == it;
+            if (dup) local_err |= DEV_NOTE_REPEATS;
           }
           prev = it;
           if (it >= N) {
@@ -87,6 +90,7 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
         }
       }
       local_max = max(local_max, distinct);
+      local_pairs += (uint64_t)distinct * (distinct - 1) / 2;
     }
     for (uint32_t pend = __ballot_sync(0xffffffffu, wide); pend; pend &= pend - 1) {
       const uint32_t src = __ffs(pend) - 1;
@@ -107,15 +111,21 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
           for (uint32_t q = 0; q < 32; ++q) dup |= __shfl_sync(0xffffffffu, prv, q) == it;
         }
         const bool count = ok && !dup;
+        if (ok && dup) local_err |= DEV_NOTE_REPEATS;
         distinct += __popc(__ballot_sync(0xffffffffu, count));
         if (count) bump(it);
       }
       local_max = max(local_max, distinct);
+      if (lane == 0) local_pairs += (uint64_t)distinct * (distinct - 1) / 2;
     }
   }
   if (local_err) atomicOr(&flags[0], local_err);
   local_max = __reduce_max_sync(0xffffffffu, local_max);
   if (lane == 0 && local_max) atomicMax(&flags[1], local_max);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) local_pairs += __shfl_xor_sync(0xffffffffu, local_pairs, o);
+  if (lane == 0 && local_pairs)
+    atomicAdd(reinterpret_cast<unsigned long long*>(flags + 4), (unsigned long long)local_pairs);
   if (use_smem) {
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < N; i += blockDim.x)
@@ -156,14 +166,6 @@ __global__ void k_bitmap_build(const uint32_t* __restrict__ off, const uint32_t*
   }
 }
 
-__device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t k) {
-  // k-th output of SplitMix64 (Steele, Lea, Flood 2014) started at state `seed`
-  uint64_t z = seed + (k + 1) * 0x9E3779B97F4A7C15ULL;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
-  return z ^ (z >> 31);
-}
-
 // Database sample D_s drawn with replacement (Sec. 6.1): sample row k is
 // transaction ((x_k >> 32) * D) >> 32; its kept items are set in bit k of the
 // sample bitmap rows (same row order as the full database).
@@ -171,8 +173,7 @@ __global__ void k_sample_build(const uint32_t* __restrict__ off, const uint32_t*
                                const int32_t* __restrict__ item_rank, uint64_t seed, uint32_t m,
                                uint32_t* __restrict__ sbits, uint32_t sstride) {
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < m; k += gridDim.x * blockDim.x) {
-    uint64_t x = splitmix64_at(seed, k);
-    uint32_t t = (uint32_t)(((x >> 32) * (uint64_t)D) >> 32);
+    const uint32_t t = sample_draw(seed, k, D);
     const uint32_t bit = 1u << (k & 31), word = k >> 5;
     for (uint32_t q = off[t]; q < off[t + 1]; ++q) {
       int32_t r = item_rank[items[q]];

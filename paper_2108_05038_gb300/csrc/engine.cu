@@ -98,17 +98,43 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     const uint64_t xb = pair_mma_buffer_bytes(n1, in.stride, ep->pair_e2m1);
     const bool coords_ok = (uint64_t)in.stride * 32 < (1ull << 31);
     const double cores_us = pair_cores_cost_us(n1, in.stride, db->num_sms);
+    double rows_us = cores_us;  // the better of the kernels that read the bitmap rows (automatic choice)
     if (cfg.pair_kernel == FIM_PAIR_TENSOR_FUSED) {
       if (!consecutive) return fail(FIM_ERR_INVALID, "the fused tensor-core pair kernel needs consecutive rows");
       ep->pair_mma = ep->pair_fused = true;
     } else if (cfg.pair_kernel >= FIM_PAIR_TENSOR) {
       ep->pair_mma = coords_ok;
     } else if (cfg.pair_kernel == FIM_PAIR_AUTO) {
-      if (consecutive)
-        ep->pair_mma = ep->pair_fused = pair_mma_cost_us(n1, in.stride, db->num_sms, false, true) < cores_us;
-      else
-        ep->pair_mma = coords_ok && xb <= db->total_mem / 16 &&
-                       pair_mma_cost_us(n1, in.stride, db->num_sms, ep->pair_e2m1) < cores_us;
+      if (consecutive) {
+        const double us = pair_mma_cost_us(n1, in.stride, db->num_sms, false, true);
+        ep->pair_mma = ep->pair_fused = us < cores_us;
+        rows_us = std::min(us, cores_us);
+      } else if (coords_ok && xb <= db->total_mem / 16) {
+        const double us = pair_mma_cost_us(n1, in.stride, db->num_sms, ep->pair_e2m1);
+        ep->pair_mma = us < cores_us;
+        rows_us = std::min(us, cores_us);
+      }
+      // the transactions instead of the rows, for all rows or (consecutive ones) for all but the most frequent,
+      // whose pairs a block of the product counts
+      if (in.tx.n) {
+        const double all_us = pair_tx_cost_us(db, in.tx, in.frows.data(), 0, n1, n1);
+        const double part_us = consecutive && n1 >= 2 * kTxDenseRows
+                                   ? pair_tx_cost_us(db, in.tx, in.frows.data(), 0, n1, n1 - kTxDenseRows) +
+                                         pair_mma_block_cost_us(n1, in.stride, db->num_sms)
+                                   : 1e300;
+        if (std::min(all_us, part_us) < rows_us) {
+          ep->pair_tx = true;
+          ep->tx_lim = all_us <= part_us ? n1 : n1 - kTxDenseRows;
+          ep->pair_mma = ep->pair_fused = ep->tx_lim < n1;
+          ep->tx = in.tx;
+          if (!in.tx.map) {
+            FIM_TRY(ws_get(ws, WS_TX_MAP, db->N, &ep->d_tx_map));
+            ep->tx.map = ep->d_tx_map;
+            ep->d_item_rank = db->d_item_rank;
+            ep->n_items = db->N;
+          }
+        }
+      }
     }
     if (ep->pair_mma && !ep->pair_fused) FIM_TRY(ws_get(ws, WS_PAIR_X, xb, &ep->d_X));
     ep->pair_extra_tx = cfg.fault_pair_wait ? 16u : 0u;
@@ -258,7 +284,17 @@ cudaError_t engine_launch_front(const EnginePlan& ep, cudaStream_t st, bool pair
   if (pairs) {
     uint32_t ksplit = 0;
     PairLaunch pl{ep.bits, ep.stride, ep.d_frows, ep.n1, ep.d_C2, 0, ep.rows_base};
+    if (ep.pair_tx) {
+      ce = cudaMemsetAsync(ep.d_C2, 0, (size_t)ep.n1 * ep.n1 * sizeof(uint32_t), st);
+      if (ce == cudaSuccess && ep.d_tx_map)
+        ce = launch_tx_map(ep.d_item_rank, ep.n_items, ep.d_frows, ep.n1, ep.d_tx_map, st);
+      if (ce == cudaSuccess) ce = launch_pair_tx(ep.tx, ep.n1, ep.tx_lim, ep.d_C2, ep.num_sms, st);
+      if (ce != cudaSuccess) return ce;
+      pl.cleared = true;
+      if (ep.tx_lim < ep.n1) pl.col0 = ep.tx_lim;
+    }
     ce = ep.pair_fused ? launch_pair_mma_fused(pl, &ep.d_ctrl->err, ep.num_sms, st, &ksplit, ep.pair_extra_tx)
+         : ep.pair_tx  ? cudaSuccess
          : ep.pair_mma ? launch_pair_mma(pl, ep.d_X, ep.pair_e2m1, &ep.d_ctrl->err, ep.num_sms, st, &ksplit,
                                          ep.pair_extra_tx)
                        : launch_pair_counts(pl, ep.num_sms, st, &ksplit);

@@ -276,13 +276,14 @@ static fim_status db_build_rows(fim_db* db, const uint32_t* src_off, const uint3
   cudaStream_t st = db->stream;
   const uint32_t N = db->N, D = db->D;
   uint32_t *d_cnt = nullptr, *d_flags = nullptr;
-  FIM_TRY(ws_get(db->ws, WS_TALLY, (size_t)N + 4, &d_cnt));
-  d_flags = d_cnt + N;  // [err, max_len, off[0], off[D]]
-  FIM_CUDA(cudaMemsetAsync(d_cnt, 0, ((size_t)N + 4) * 4, st));
+  const size_t fl = ((size_t)N + 1) & ~(size_t)1, cnt_words = fl + 6;  // (the 64-bit flag on 8 bytes)
+  FIM_TRY(ws_get(db->ws, WS_TALLY, cnt_words, &d_cnt));
+  d_flags = d_cnt + fl;  // [err, max_len, off[0], off[D], pairs (u64)]
+  FIM_CUDA(cudaMemsetAsync(d_cnt, 0, cnt_words * 4, st));
   FIM_CUDA(launch_item_count(src_off, src_items, D, N, d_cnt, d_flags, st));
   void* hcnt = nullptr;
-  FIM_TRY(stage_get(db, ((size_t)N + 4) * 4, &hcnt));
-  FIM_CUDA(cudaMemcpyAsync(hcnt, d_cnt, ((size_t)N + 4) * 4, cudaMemcpyDeviceToHost, st));
+  FIM_TRY(stage_get(db, cnt_words * 4, &hcnt));
+  FIM_CUDA(cudaMemcpyAsync(hcnt, d_cnt, cnt_words * 4, cudaMemcpyDeviceToHost, st));
   // Without a prefilter every item gets a row (n_rows = N), so the bitmap block is known before the counts:
   // it is cleared behind the counts' copy, while the host waits for that copy alone and relabels the rows.
   const bool early_bits = db->prefilter == 0 && (size_t)N * db->stride > 0;
@@ -296,14 +297,18 @@ static fim_status db_build_rows(fim_db* db, const uint32_t* src_off, const uint3
   } else {
     FIM_TRY(stream_sync(db));
   }
-  std::vector<uint32_t> cnt(static_cast<uint32_t*>(hcnt), static_cast<uint32_t*>(hcnt) + N + 4);
-  const uint32_t err = cnt[N];
-  if (cnt[N + 2] != 0) return fail(FIM_ERR_INVALID, "tx_offsets[0] must be 0");
+  std::vector<uint32_t> cnt(static_cast<uint32_t*>(hcnt), static_cast<uint32_t*>(hcnt) + cnt_words);
+  const uint32_t* const flags = cnt.data() + fl;
+  const uint32_t err = flags[0];
+  if (flags[2] != 0) return fail(FIM_ERR_INVALID, "tx_offsets[0] must be 0");
   if (err & DEV_ERR_OFFSETS) return fail(FIM_ERR_INVALID, "tx_offsets is not non-decreasing");
   if (err & DEV_ERR_ITEM_RANGE) return fail(FIM_ERR_INVALID, "an item id is >= N");
-  db->max_tx_len = cnt[N + 1];
+  db->max_tx_len = flags[1];
+  db->tx_repeats = (err & DEV_NOTE_REPEATS) != 0;
+  db->tx_pairs = flags[4] | (uint64_t)flags[5] << 32;
+  db->tx_distinct = std::accumulate(cnt.begin(), cnt.begin() + N, (uint64_t)0);
   if (device_input) {  // the offsets are valid: keep a copy of the CSR (the sample draw reads it)
-    db->nnz = cnt[N + 3];
+    db->nnz = flags[3];
     FIM_TRY(ws_get(db->ws, WS_DB_TXOFF, (size_t)D + 1, &db->d_tx_off));
     FIM_TRY(ws_get(db->ws, WS_DB_TXITEMS, std::max<uint64_t>(1, db->nnz), &db->d_tx_items));
     FIM_CUDA(cudaMemcpyAsync(db->d_tx_off, src_off, ((size_t)D + 1) * 4, cudaMemcpyDeviceToDevice, st));
@@ -404,6 +409,21 @@ static void rows_for_minsup(const fim_db* db, uint32_t minsup, EngineInput* in) 
   }
 }
 
+// the transactions a mine of rows r0 .. n_rows - 1 (sample = false) or a sample of m draws stands for
+static TxPairs tx_pairs(const fim_db* db, bool sample, uint32_t m, uint64_t seed, int32_t base) {
+  TxPairs t;
+  if (db->tx_repeats) return t;
+  t.off = db->d_tx_off;
+  t.items = db->d_tx_items;
+  t.map = db->d_item_rank;
+  t.base = base;
+  t.n = sample ? m : db->D;
+  t.D = db->D;
+  t.seed = seed;
+  t.sample = sample ? 1u : 0u;
+  return t;
+}
+
 static void engine_config_from_opts(const fim_mine_opts* o, EngineConfig* c) {
   fim_mine_opts d;
   fim_mine_opts_init(&d);
@@ -460,6 +480,7 @@ fim_status mine_input(fim_db* db, uint32_t minsup_abs, const fim_mine_opts* opts
   in->d_rank_item = db->d_rank_item;
   in->minsup = minsup_abs;
   in->max_len_bound = db->max_tx_len;
+  in->tx = tx_pairs(db, false, 0, 0, (int32_t)(db->n_rows - in->n1));
   if (in->n1) {
     in->d_frows = db->d_iota + (db->n_rows - in->n1);  // frequent rows are the suffix
     in->d_row_supp = db->d_supp + (db->n_rows - in->n1);
@@ -706,6 +727,7 @@ fim_status estimate_impl(fim_db* db, double sample_rate, double rel_minsup, uint
       in.d_rank_item = db->d_rank_item;
       in.minsup = minsup_s;
       in.max_len_bound = db->max_tx_len;
+      in.tx = tx_pairs(db, true, m, seed, 0);
       EngineConfig cfg;
       cfg.donate = 0;
       unsigned long long* d_work = nullptr;
@@ -804,6 +826,8 @@ fim_status estimate_impl(fim_db* db, double sample_rate, double rel_minsup, uint
     in.d_rank_item = db->d_rank_item;
     in.minsup = minsup_s;
     in.max_len_bound = db->max_tx_len;
+    in.tx = tx_pairs(db, true, m, seed, 0);
+    if (!all_rows) in.tx.map = nullptr;  // (rows of a choice: their map is built)
     EngineConfig cfg;
     cfg.donate = 0;
     cfg.max_sets = max_sample_itemsets;

@@ -53,7 +53,17 @@ enum : uint32_t {
   DEV_ERR_POOL = 1u << 5,         // donation pool protocol violated
   DEV_ERR_ABORTED = 1u << 6,      // more itemsets than the caller's limit: mining stopped early
   DEV_ERR_PSTACK = 1u << 7,       // projected DFS: a warp's stack was too small (grown and repeated)
+  DEV_NOTE_REPEATS = 1u << 8,     // (not an error) a transaction holds an item twice
 };
+
+// the k-th draw of the estimate's sample (with replacement, Sec. 6.1): transaction ((x_k >> 32) * D) >> 32, x_k the
+// k-th output of SplitMix64 (Steele, Lea, Flood 2014) started at state `seed`
+__device__ __forceinline__ uint32_t sample_draw(uint64_t seed, uint64_t k, uint32_t D) {
+  uint64_t z = seed + (k + 1) * 0x9E3779B97F4A7C15ULL;
+  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
+  z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
+  return (uint32_t)((((z ^ (z >> 31)) >> 32) * (uint64_t)D) >> 32);
+}
 
 // ---------------------------------------------------------------------------
 // stream-ordered device buffers, grown on demand and reused across calls
@@ -103,6 +113,7 @@ enum WsSlot {
   WS_EST,  // a deferred estimate's class costs (u64) and order (u32)
   WS_CTATIME,
   WS_PAIR_X,        // rows widened to bytes for the tensor-core pair kernel
+  WS_TX_MAP,        // item -> index of its row among a sample's rows (pair counts from the transactions)
   WS_QUERY_ROWS,    // fim_extension_supports: prefix rows | candidate rows
   WS_QUERY_OUT,     // fim_extension_supports: one count per candidate
   WS_QUERY_PREFIX,  // fim_extension_supports: t(P) of a prefix of two or more items
@@ -188,6 +199,9 @@ struct fim_db {
   uint32_t prefilter = 0;
   uint32_t max_tx_len = 0;  // longest transaction (distinct kept items)
   uint64_t nnz = 0;
+  uint64_t tx_pairs = 0;    // sum of len (len - 1) / 2 over the transactions (distinct items)
+  uint64_t tx_distinct = 0; // sum of len
+  bool tx_repeats = false;  // a transaction holds an item twice (its pairs cannot be counted from the list)
   cudaStream_t stream = nullptr;
   int device = 0;
   int num_sms = 0;
@@ -261,6 +275,20 @@ namespace fim {
 // ---------------------------------------------------------------------------
 // mining engine (shared by fim_mine and the sample mining of the estimate)
 
+// The same counts from the transactions (pair_tx.cu): C2 (cleared by the caller) gets 1 per transaction and pair of
+// its rows below `lim`.  A transaction is one of the database (sample = false: 0 .. n - 1) or the k-th of n draws
+// of the estimate's sample (sample = true, seed, D transactions to draw from); an item's row is map[item] - base,
+// and items whose row is negative or >= lim take no part.  No transaction may hold an item twice.
+struct TxPairs {
+  const uint32_t *off = nullptr, *items = nullptr;
+  const int32_t* map = nullptr;
+  int32_t base = 0;
+  uint32_t n = 0, D = 0;
+  uint64_t seed = 0;
+  uint32_t sample = 0;
+};
+constexpr uint32_t kTxDenseRows = 256;  // the most frequent rows, left to the tensor-core product
+
 struct EngineInput {
   const uint32_t* bits = nullptr;  // rows of `stride` words
   const uint32_t* d_frows = nullptr;     // optional device copy of frows (else uploaded)
@@ -276,6 +304,8 @@ struct EngineInput {
   const uint32_t* d_rank_item = nullptr;  // row -> original item id
   uint32_t minsup = 1;
   uint32_t max_len_bound = 2;      // upper bound on the length of a frequent itemset
+  // the transactions the rows stand for (n = 0: not to be used; map NULL: the rows are not consecutive, a map is built)
+  TxPairs tx;
 };
 
 struct EngineOutput {
@@ -341,6 +371,12 @@ struct EnginePlan {
   bool pair_e2m1 = true;    // tensor-core operands packed as e2m1 (else e4m3)
   bool pair_fused = false;  // widening fused into the tensor-core product (consecutive rows, no widened copy)
   const uint32_t* rows_base = nullptr;  // the frequent rows when consecutive
+  bool pair_tx = false;     // level 2 from the transactions, for the rows below tx_lim (the others: fused product)
+  uint32_t tx_lim = 0;
+  TxPairs tx;
+  int32_t* d_tx_map = nullptr;          // item -> row index, built by the launch (rows not consecutive)
+  const int32_t* d_item_rank = nullptr;
+  uint32_t n_items = 0;
   uint32_t pair_extra_tx = 0;  // test: bytes a stage waits for beyond its copies (0 normally)
   uint8_t* d_X = nullptr;   // widened rows (pair_mma only)
   // projected DFS (mode 5): budgets, geometry and buffers; the fallback runs the sparse node mode with
@@ -444,6 +480,8 @@ struct PairLaunch {
   uint32_t* C2;  // n1 * n1
   uint32_t ksplit;
   const uint32_t* rows_base = nullptr;  // the frequent rows when they are consecutive rows of `bits` (else NULL)
+  uint32_t col0 = 0;     // fused kernel: nonzero = n1 - kTxDenseRows: only the pairs with j >= col0
+  bool cleared = false;  // C2 is cleared already (fused kernel)
 };
 cudaError_t launch_pair_counts(const PairLaunch& p, int num_sms, cudaStream_t st, uint32_t* ksplit_used);
 // the same counts on the tensor cores: rows widened into X (pair_mma_buffer_bytes), then C2 = X X^T;
@@ -456,9 +494,19 @@ uint64_t pair_mma_buffer_bytes(uint32_t n1, uint32_t stride, bool e2m1);
 // bits, no widened copy); needs p.rows_base
 cudaError_t launch_pair_mma_fused(const PairLaunch& p, uint32_t* err, int num_sms, cudaStream_t st,
                                   uint32_t* ksplit_used, uint32_t extra_tx = 0);
+// (pair_tx.cu)
+cudaError_t launch_pair_tx(const TxPairs& p, uint32_t n1, uint32_t lim, uint32_t* C2, int num_sms, cudaStream_t st);
+// map[item] = index of its row among the n1 ascending rows, or -1
+cudaError_t launch_tx_map(const int32_t* item_rank, uint32_t N, const uint32_t* frows, uint32_t n1, int32_t* map,
+                          cudaStream_t st);
 // modelled device time (µs) of each pair kernel, for the automatic choice
 double pair_mma_cost_us(uint32_t n1, uint32_t stride, int num_sms, bool e2m1, bool fused = false);
 double pair_cores_cost_us(uint32_t n1, uint32_t stride, int num_sms);
+// (the product's block of the last kTxDenseRows columns only)
+double pair_mma_block_cost_us(uint32_t n1, uint32_t stride, int num_sms);
+// counting the pairs of the n1 rows (ids frows, ascending, or r0 .. when NULL) below lim from p's transactions
+double pair_tx_cost_us(const fim_db* db, const TxPairs& p, const uint32_t* frows, uint32_t r0, uint32_t n1,
+                       uint32_t lim);
 
 struct LevelLaunch {
   const uint32_t* C2;

@@ -109,8 +109,20 @@ extern "C" fim_status fim_mine_pairs_noalloc(const fim_db* db, uint32_t minsup_a
   note_launch();
   FIM_CUDA(cudaGetLastError());
   uint32_t ksplit = 0;
-  PairLaunch pl{db->d_bits, db->stride, frows, n1, C2, 0};
-  FIM_CUDA(launch_pair_counts(pl, db->num_sms, st, &ksplit));  // clears C2 itself when it splits rows
+  // from the transactions or from the rows, whichever is modelled faster
+  TxPairs tx;
+  tx.off = db->d_tx_off;
+  tx.items = db->d_tx_items;
+  tx.map = db->d_item_rank;
+  tx.base = (int32_t)r0;
+  tx.n = tx.D = db->D;
+  if (!db->tx_repeats && pair_tx_cost_us(db, tx, nullptr, r0, n1, n1) < pair_cores_cost_us(n1, db->stride, db->num_sms)) {
+    FIM_CUDA(cudaMemsetAsync(C2, 0, (size_t)n1 * n1 * 4, st));
+    FIM_CUDA(launch_pair_tx(tx, n1, n1, C2, db->num_sms, st));
+  } else {
+    PairLaunch pl{db->d_bits, db->stride, frows, n1, C2, 0};
+    FIM_CUDA(launch_pair_counts(pl, db->num_sms, st, &ksplit));  // clears C2 itself when it splits rows
+  }
   k_pairs_emit<<<n1, 256, 0, st>>>(C2, n1, minsup_abs, r0, db->d_rank_item, d_pairs, d_supports, capacity, counter);
   note_launch();
   FIM_CUDA(cudaGetLastError());

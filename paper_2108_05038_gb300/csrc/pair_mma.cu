@@ -437,6 +437,7 @@ constexpr size_t kFSmemBytes =
 static_assert(kFSmemBytes <= 227u * 1024u, "shared memory per CTA");
 static_assert(kFThreads <= 1024 && kRawRows % kGroupThreads == 0, "whole rows per expander thread");
 static_assert(kRStages == kExpGroups && kFStages == kExpGroups, "group g owns raw stage g and operand stage g");
+static_assert(kFN == kTxDenseRows, "one column block holds the rows left to the product");
 static_assert(kBK == 128 && kFM == 2 * kBM && 2 * kBN == kTmemCols, "128-byte operand rows; two accumulators");
 
 // the 32 transactions of raw word w as output words t = 0..7 (two 16-byte chunks): (w << (6 - t)) & keep,
@@ -454,7 +455,7 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 }
 
 __global__ void __launch_bounds__(kFThreads, 1)
-    k_pair_mma_fused(const __grid_constant__ CUtensorMap rmap, uint32_t n1, uint32_t nb, uint32_t n_tiles,
+    k_pair_mma_fused(const __grid_constant__ CUtensorMap rmap, uint32_t n1, uint32_t nb, uint32_t col0, uint32_t n_tiles,
                      uint32_t nsteps, uint32_t steps_per_item, uint32_t ksplit, uint32_t* __restrict__ C2,
                      uint32_t* __restrict__ err, uint32_t extra_tx, uint32_t unit) {
   extern __shared__ uint8_t smem_raw[];
@@ -508,34 +509,36 @@ __global__ void __launch_bounds__(kFThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem_raw + (tslot - raw));
 
-  // item -> (row block bi, column block bj >= bi, first K slice, slices); items of one K range are
-  // consecutive, so the CTAs of a round read the same K slices of the rows (L2 reuse)
+  // item -> (first row i0, first column row j0, first K slice, slices); items of one K range are
+  // consecutive, so the CTAs of a round read the same K slices of the rows (L2 reuse).  With col0 the tiles are
+  // the row blocks against the one column block that starts there
   const uint32_t n_items = n_tiles * ksplit;
-  auto decode = [&](uint32_t item, uint32_t& bi, uint32_t& bj, uint32_t& k0, uint32_t& ns) {
+  auto decode = [&](uint32_t item, uint32_t& i0, uint32_t& j0, uint32_t& k0, uint32_t& ns) {
     const uint32_t split = item / n_tiles;
     uint32_t t = item % n_tiles;
-    bi = 0;
-    while (t >= nb - bi) {  // row block bi pairs with the column blocks bj >= bi
+    uint32_t bi = 0;
+    while (!col0 && t >= nb - bi) {  // row block bi pairs with the column blocks bj >= bi
       t -= nb - bi;
       ++bi;
     }
-    bj = bi + t;
+    i0 = (col0 ? t : bi) * kFM;
+    j0 = col0 ? col0 : (bi + t) * kFN;
     k0 = split * steps_per_item;
     ns = min(nsteps, k0 + steps_per_item) - k0;
   };
 
-  // read-back round rd (0-31) of tile (bi, bj) by one warp for TMEM lane quarter `quarter`: half rd / 16, 16
+  // read-back round rd (0-31) of the tile at (i0, j0) by one warp for TMEM lane quarter `quarter`: half rd / 16, 16
   // columns from (rd mod 16) x 16, through the warp's staging area sw (32 x kFPitch words)
-  auto readback_round = [&](uint32_t rd, uint32_t* sw, uint32_t bi, uint32_t bj, uint32_t quarter) {
+  auto readback_round = [&](uint32_t rd, uint32_t* sw, uint32_t i0, uint32_t j0, uint32_t quarter) {
     const uint32_t h = rd / (kFN / kFChunk), c0 = (rd % (kFN / kFChunk)) * kFChunk;
-    const uint32_t row0 = bi * kFM + h * kBM + quarter * 32;
+    const uint32_t row0 = i0 + h * kBM + quarter * 32;
     uint32_t r[16];
     tmem_ld16(tmem + ((quarter * 32u) << 16) + h * kBN + c0, r);
 #pragma unroll
     for (uint32_t c = 0; c < 16; ++c)
       sw[lane * kFPitch + c] = __float2uint_rn(__uint_as_float(r[c]) * 0.25f);  // exact: a power of 2
     __syncwarp();
-    const uint32_t j = bj * kFN + c0 + (lane & 15u);
+    const uint32_t j = j0 + c0 + (lane & 15u);
 #pragma unroll 4
     for (uint32_t rr = 0; rr < 16; ++rr) {
       const uint32_t rl = rr + (lane >> 4) * 16u, i = row0 + rl;
@@ -553,8 +556,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
   if (warp == 0) {
     if (lane == 0) {
       for (uint32_t item = blockIdx.x; item < n_items && !*abort_flag; item += gridDim.x) {
-        uint32_t bi, bj, k0, ns;
-        decode(item, bi, bj, k0, ns);
+        uint32_t i0, j0, k0, ns;
+        decode(item, i0, j0, k0, ns);
         bool ok = true;
         for (uint32_t s = 0; s < ns; ++s, ++issued) {
           const uint32_t st = issued % kRStages;
@@ -567,10 +570,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
           mbar_expect_tx(rfull(st), kRawStageBytes + extra_tx);
           const int32_t x = (int32_t)((k0 + s) * 4);  // words: x * 4 bytes is a multiple of 16
           const uint32_t d = raw_st + st * kRawStageBytes;
-          tma_load(d, &rmap, x, (int32_t)(bi * kFM), rfull(st));
-          tma_load(d + kBM * 16, &rmap, x, (int32_t)(bi * kFM + kBM), rfull(st));
-          tma_load(d + 2 * kBM * 16, &rmap, x, (int32_t)(bj * kFN), rfull(st));
-          tma_load(d + 3 * kBM * 16, &rmap, x, (int32_t)(bj * kFN + kBM), rfull(st));
+          tma_load(d, &rmap, x, (int32_t)i0, rfull(st));
+          tma_load(d + kBM * 16, &rmap, x, (int32_t)(i0 + kBM), rfull(st));
+          tma_load(d + 2 * kBM * 16, &rmap, x, (int32_t)j0, rfull(st));
+          tma_load(d + 3 * kBM * 16, &rmap, x, (int32_t)(j0 + kBM), rfull(st));
         }
         if (!ok) break;
       }
@@ -580,8 +583,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
     if (lane == 0) {
       uint32_t consumed = 0, it = 0;
       for (uint32_t item = blockIdx.x; item < n_items && !*abort_flag; item += gridDim.x, ++it) {
-        uint32_t bi, bj, k0, ns;
-        decode(item, bi, bj, k0, ns);
+        uint32_t i0, j0, k0, ns;
+        decode(item, i0, j0, k0, ns);
         if (it >= 1 && !mbar_wait(acc_empty, (it - 1) & 1)) {  // the previous tile read back
           abort_now();
           break;
@@ -625,8 +628,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
     uint32_t* sw = staging + (warp - 2) * 32 * kFPitch;
     uint32_t it = 0;
     for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
-      uint32_t bi, bj, k0, ns;
-      decode(item, bi, bj, k0, ns);
+      uint32_t i0, j0, k0, ns;
+      decode(item, i0, j0, k0, ns);
       const bool ok = __all_sync(0xffffffffu, mbar_wait(acc_full, it & 1));
       if (!ok || *abort_flag) {
         if (lane == 0 && !ok) abort_now();
@@ -635,7 +638,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
       tc_fence_after();
       const uint32_t step = item + gridDim.x >= n_items ? kLastWorkers : 1u;
 #pragma unroll 1
-      for (uint32_t rd = 0; rd < 2 * kFN / kFChunk; rd += step) readback_round(rd, sw, bi, bj, quarter);
+      for (uint32_t rd = 0; rd < 2 * kFN / kFChunk; rd += step) readback_round(rd, sw, i0, j0, quarter);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty);
@@ -654,8 +657,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
     uint32_t c = 0;  // slices of this CTA so far (both groups)
     bool ok = true;
     for (uint32_t item = blockIdx.x; item < n_items && ok && !*abort_flag; item += gridDim.x) {
-      uint32_t bi, bj, k0, ns;
-      decode(item, bi, bj, k0, ns);
+      uint32_t i0, j0, k0, ns;
+      decode(item, i0, j0, k0, ns);
       for (uint32_t s = 0; s < ns; ++s, ++c) {
         if (c % kExpGroups != grp) continue;
         const uint32_t rs = c % kRStages, os = c % kFStages;
@@ -696,12 +699,12 @@ __global__ void __launch_bounds__(kFThreads, 1)
       if (done && !*abort_flag) {
         tc_fence_after();
         const uint32_t last = blockIdx.x + (n_items - 1 - blockIdx.x) / gridDim.x * gridDim.x;
-        uint32_t bi, bj, k0, ns;
-        decode(last, bi, bj, k0, ns);
+        uint32_t i0, j0, k0, ns;
+        decode(last, i0, j0, k0, ns);
         const uint32_t ew = warp - kThreads / 32;  // expander warp 0-23
         uint32_t* sw = reinterpret_cast<uint32_t*>(smem_raw + (op_st - raw)) + ew * 32 * kFPitch;
         for (uint32_t rd = 1 + ew / 4; rd < 2 * kFN / kFChunk; rd += kLastWorkers)
-          readback_round(rd, sw, bi, bj, warp & 3);
+          readback_round(rd, sw, i0, j0, warp & 3);
         tc_fence_before();
       } else if (!done && lane == 0) {
         abort_now();
@@ -764,13 +767,12 @@ uint64_t pair_mma_buffer_bytes(uint32_t n1, uint32_t stride, bool e2m1) {
   return (uint64_t)n1 * stride * (e2m1 ? 16ull : 32ull);
 }
 
-double pair_mma_cost_us(uint32_t n1, uint32_t stride, int num_sms, bool e2m1, bool fused) {
-  // widening (bytes written at ~5 TB/s) + tile rounds at ~1.5 PFLOP/s of kind::f8f6f4 per 152 SMs
-  const double x_bytes = fused ? 0.0 : (double)pair_mma_buffer_bytes(n1, stride, e2m1);
-  // (fused: 256 x 256 tiles, twice the MMAs per slice)
-  const uint32_t tiles = fused ? fused_tiles(n1) : pair_tiles(n1);
+// widening (bytes written at ~5 TB/s) + tile rounds at ~1.5 PFLOP/s of kind::f8f6f4 per 152 SMs; fused: 256 x 256
+// tiles, 0.58 us per slice and 12 us for the launch, the first reads and the last read-back (measured: 3,937 rows of
+// 7,813 slices 4.07 ms, modelled 4.07; 988 rows of 784 slices 42 us, modelled 48)
+static double mma_cost_us(uint32_t tiles, double x_bytes, uint32_t stride, int num_sms, bool fused) {
   const uint32_t nsteps = stride / 4;
-  const double step_us = (fused ? 2.0 : 1.0) * 2.0 * kBM * kBN * kBK / (1.5e15 / 152.0) * 1e6;  // one K slice of a tile
+  const double step_us = fused ? 0.58 : 2.0 * kBM * kBN * kBK / (1.5e15 / 152.0) * 1e6;  // one K slice of a tile
   double best = 1e300;
   for (uint32_t ks = 1; ks <= 256; ++ks) {
     const uint32_t spi = std::min(kMaxStepsPerItem, (nsteps + ks - 1) / ks);
@@ -779,7 +781,16 @@ double pair_mma_cost_us(uint32_t n1, uint32_t stride, int num_sms, bool e2m1, bo
     const uint64_t rounds = (items + num_sms - 1) / num_sms;
     best = std::min(best, (double)rounds * (spi + 1) * step_us + 8.0 * step_us);
   }
-  return x_bytes / 5e12 * 1e6 + best + 4.0;
+  return x_bytes / 5e12 * 1e6 + best + (fused ? 12.0 : 4.0);
+}
+
+double pair_mma_cost_us(uint32_t n1, uint32_t stride, int num_sms, bool e2m1, bool fused) {
+  return mma_cost_us(fused ? fused_tiles(n1) : pair_tiles(n1),
+                     fused ? 0.0 : (double)pair_mma_buffer_bytes(n1, stride, e2m1), stride, num_sms, fused);
+}
+
+double pair_mma_block_cost_us(uint32_t n1, uint32_t stride, int num_sms) {
+  return mma_cost_us((n1 + kFM - 1) / kFM, 0.0, stride, num_sms, true);
 }
 
 // the split of the K range: items fill whole rounds of the SMs, at most 2^24 elements per item, at least 8
@@ -826,16 +837,18 @@ cudaError_t launch_pair_mma_fused(const PairLaunch& p, uint32_t* err, int num_sm
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
   const uint32_t nb = (p.n1 + kFM - 1) / kFM;
-  const uint32_t tiles = fused_tiles(p.n1);
+  if (p.col0 && p.col0 + kFN != p.n1) return cudaErrorInvalidValue;
+  const uint32_t tiles = p.col0 ? nb : fused_tiles(p.n1);
   const uint32_t nsteps = p.stride / 4;  // stride is a multiple of 32 words: whole 128-transaction slices
   const uint32_t spi = pair_split(tiles, nsteps, num_sms);
   const uint32_t ksplit = (nsteps + spi - 1) / spi;
   *ksplit_used = ksplit;
-  if (ksplit > 1 && (e = cudaMemsetAsync(p.C2, 0, (size_t)p.n1 * p.n1 * sizeof(uint32_t), st)) != cudaSuccess)
+  if (ksplit > 1 && !p.cleared &&
+      (e = cudaMemsetAsync(p.C2, 0, (size_t)p.n1 * p.n1 * sizeof(uint32_t), st)) != cudaSuccess)
     return e;
   const uint64_t items = (uint64_t)tiles * ksplit;
   const uint32_t grid = (uint32_t)std::min<uint64_t>(items, (uint64_t)num_sms);
-  k_pair_mma_fused<<<grid, kFThreads, kFSmemBytes, st>>>(map, p.n1, nb, tiles, nsteps, spi, ksplit, p.C2, err,
+  k_pair_mma_fused<<<grid, kFThreads, kFSmemBytes, st>>>(map, p.n1, nb, p.col0, tiles, nsteps, spi, ksplit, p.C2, err,
                                                          extra_tx, 1u);
   note_launch();
   return cudaGetLastError();
