@@ -163,7 +163,8 @@ __global__ void k_level2_fill(const uint32_t* __restrict__ C2, uint32_t n1, uint
                               uint2* __restrict__ entries, uint64_t* __restrict__ out_off,
                               uint32_t* __restrict__ out_items, uint32_t* __restrict__ out_supp, uint64_t cap_sets,
                               uint64_t cap_items, unsigned long long* __restrict__ class_sets,
-                              const uint32_t* __restrict__ eoffx, uint2* __restrict__ entries_f) {
+                              const uint32_t* __restrict__ eoffx, uint2* __restrict__ entries_f,
+                              const uint32_t* __restrict__ goff, uint2* __restrict__ entries_g) {
   __shared__ uint32_t wtot[33];
   const uint32_t q = blockIdx.x;
   const uint32_t i = row_order[q];
@@ -178,7 +179,7 @@ __global__ void k_level2_fill(const uint32_t* __restrict__ C2, uint32_t n1, uint
   const uint32_t ne = scnt[i] > 0 ? scnt[i] - 1 : 0u;
   // the projected DFS splits the entries into its own queue and the fallback queue (bit 31 of eoffx)
   const uint32_t ex = eoffx ? eoffx[q] : eoff[q];
-  uint2* const dst = (eoffx && (ex & 0x80000000u)) ? entries_f : entries;
+  uint2* const dst = (eoffx && (ex & 0x80000000u)) ? entries_f : goff && goff[i] != kNoGram ? entries_g : entries;
   const uint32_t e0 = eoffx ? (ex & 0x7fffffffu) : ex;
   for (uint32_t m = threadIdx.x; m < ne; m += blockDim.x) dst[e0 + m] = make_uint2(i, m);
   uint32_t pos0 = 0;
@@ -2057,7 +2058,7 @@ cudaError_t launch_level2_fill(const LevelLaunch& p, cudaStream_t st) {
   k_level2_fill<<<p.n1, 256, 0, st>>>(p.C2, p.n1, p.minsup, p.frows, p.row_supp, p.rank_item, p.row_order, p.scnt,
                                       p.soff, p.eoff, p.sitems, p.entries, p.leaves ? nullptr : p.out_off,
                                       p.out_items, p.out_supp, p.cap_sets, p.cap_items, p.class_sets, p.eoffx,
-                                      p.entries_f);
+                                      p.entries_f, p.goff, p.entries_g);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || !p.leaves) return e;

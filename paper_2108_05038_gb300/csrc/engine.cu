@@ -230,11 +230,25 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     if (!share) pocc = std::min<int>(pocc, (int)cfg.ctas_per_sm);
     ep->proj_grid = (uint32_t)db->num_sms * (uint32_t)pocc;
     uint32_t* meta = nullptr;
-    FIM_TRY(ws_get(ws, WS_PROJ_META, 6ull * n1 + 2, &meta));
+    FIM_TRY(ws_get(ws, WS_PROJ_META, 8ull * n1 + 4, &meta));
     ep->d_yoff = reinterpret_cast<uint64_t*>(meta);
     ep->d_toff = ep->d_yoff + n1;
     ep->d_itemoff = meta + 4ull * n1;
     ep->d_eoffx = ep->d_itemoff + n1 + 1;
+    ep->d_goff = ep->d_eoffx + n1;
+    ep->d_tileoff = ep->d_goff + n1;
+    // Small subtrees in shared memory first, unless the caller tunes the general walk (its hand-out threshold, its
+    // stacks, diffset frames), or its shared queue, which takes what they leave, is off.
+    ep->sub = share && !cfg.split_words && !cfg.pstack_words && !cfg.diffsets;
+    if (ep->sub) {
+      FIM_TRY(ws_get(ws, WS_ENTRIES_G, ep->npairs_max + 1, &ep->d_entries_g));
+      FIM_TRY(ws_get(ws, WS_SUB_G, kSubGramCap, &ep->d_G));
+      FIM_TRY(ws_get(ws, WS_SUB_ITEMS, 2ull * kSubItemCap, &ep->d_sub_items));
+      FIM_TRY(ws_get(ws, WS_SUB_TILES, kSubTileCap, &ep->d_sub_tiles));
+      FIM_TRY(ws_get(ws, WS_SUB_UNITS, kSubTileCap, &ep->d_sub_units));
+      FIM_TRY(ws_get(ws, WS_SUB_LISTS, 2 * kSubListCap, &ep->d_sub_lists));
+      FIM_TRY(ws_get(ws, WS_SUB_STATE, 1, &ep->d_sub_state));
+    }
     FIM_TRY(ws_get(ws, WS_ENTRIES_F, ep->npairs_max + 1, &ep->d_entries_f));
     // the arena holds the class regions (within proj_y_cap), then the regions of split frames
     ep->proj_arena_words = ep->proj_y_cap + (share ? std::max<uint64_t>(ep->proj_y_cap, 16ull << 20) : 0ull);
@@ -318,13 +332,18 @@ cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
     // queue), then the queue fill
     pj = ProjLaunch{ep.bits, ep.stride, ep.d_frows, ep.d_rsupp, ep.d_order, ep.d_scnt, ep.d_soff, ep.d_sitems,
                     ep.d_rank_item, ep.n1, ep.proj_y_cap, ep.proj_t_cap, ep.proj_w_cap, ep.d_yoff, ep.d_toff,
-                    ep.d_itemoff, ep.d_eoffx, ep.d_Y, ep.d_T, ep.d_ctrl};
+                    ep.d_itemoff, ep.d_eoffx, ep.d_Y, ep.d_T, ep.d_ctrl,
+                    ep.sub ? ep.d_sub_state : nullptr, ep.d_G, kSubGramCap / 2, ep.d_goff, ep.d_tileoff};
     ce = launch_level2_counts(ll, st);
     if (ce != cudaSuccess) return ce;
     ce = launch_proj_plan(pj, st);
     if (ce != cudaSuccess) return ce;
     ll.eoffx = ep.d_eoffx;
     ll.entries_f = ep.d_entries_f;
+    if (ep.sub) {
+      ll.goff = ep.d_goff;
+      ll.entries_g = ep.d_entries_g;
+    }
     ce = launch_level2_fill(ll, st);
   } else {
     ce = launch_level2(ll, st);
@@ -371,6 +390,14 @@ cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
       if (ce != cudaSuccess) return ce;
       if (ep.dq_cap) {
         ce = cudaMemsetAsync(ep.d_dq, 0, (size_t)ep.dq_cap * sizeof(uint4), st);  // no slot published yet
+        if (ce != cudaSuccess) return ce;
+      }
+      if (ep.sub) {
+        const SubLaunch sl{ep.d_Y, ep.proj_arena_words, ep.d_G, kSubGramCap, ep.d_yoff, ep.d_order, ep.d_tileoff, ep.n1,
+                           ep.minsup, ep.d_entries_g, ep.d_sub_items, ep.d_sub_tiles, ep.d_sub_units, ep.d_sub_lists, ep.d_sub_state, ep.d_off,
+                           ep.d_items, ep.d_supp, dl.cap_sets, dl.cap_items, ep.d_ctrl, ep.d_class_sets,
+                           ep.d_class_work, ep.max_sets, dl.leaves, ep.d_dq, ep.dq_cap};
+        ce = launch_sub(sl, ep.num_sms, st);
         if (ce != cudaSuccess) return ce;
       }
       DfsLaunch dp = dl;
@@ -442,6 +469,11 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
   if (h.err & DEV_ERR_TIMEOUT) return fail(FIM_ERR_TIMEOUT, "persistent kernel: bounded wait ran out without progress");
   if ((h.err & DEV_ERR_ABORTED) || (ep->max_sets && h.sets_total > ep->max_sets))
     return fail(FIM_ERR_OUTPUT_OVERFLOW, "more frequent itemsets than the limit: mining stopped early (counts are lower bounds)");
+  if (h.err & DEV_ERR_SUB) {  // no room in the small-subtree walk's queues: repeat without it
+    ep->sub = false;
+    *retry = true;
+    return FIM_OK;
+  }
   if (h.err & DEV_ERR_PSTACK) {  // a warp's stack of the projected DFS was too small: double it and repeat
     // (at least twice the largest stack a class asked for before the warps stopped)
     // (a multiple of 32 words, so every warp's stack starts on a 128-byte line)
@@ -490,7 +522,7 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
     stats->n_pair_intersections = ep->npairs_max;
     stats->n_intersections = ep->npairs_max + h.n_intersections;
     stats->n_classes = h.n_nodes;
-    stats->n_queue_entries = h.n_entries + (ep->proj ? h.n_entries_f : 0u);
+    stats->n_queue_entries = h.n_entries + (ep->proj ? h.n_entries_f + h.n_entries_g : 0u);
     stats->n_donations = h.n_donations;
     // sibling operand per intersection + one prefix read per class node + materialised prefixes
     stats->bytes_pair_kernel = ep->npairs_max * rb + (uint64_t)(n1 > 0 ? n1 - 1 : 0) * rb;

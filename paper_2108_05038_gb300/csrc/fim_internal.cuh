@@ -54,6 +54,7 @@ enum : uint32_t {
   DEV_ERR_ABORTED = 1u << 6,      // more itemsets than the caller's limit: mining stopped early
   DEV_ERR_PSTACK = 1u << 7,       // projected DFS: a warp's stack was too small (grown and repeated)
   DEV_NOTE_REPEATS = 1u << 8,     // (not an error) a transaction holds an item twice
+  DEV_ERR_SUB = 1u << 9,          // a subtree found no room in the small-subtree walk's queues (run repeated without)
 };
 
 // the k-th draw of the estimate's sample (with replacement, Sec. 6.1): transaction ((x_k >> 32) * D) >> 32, x_k the
@@ -129,6 +130,13 @@ enum WsSlot {
   WS_PSTACK,     // per-warp DFS stacks
   WS_ENTRIES_F,  // queue of the two-item classes whose class was not projected
   WS_PROJ_DQ,    // queue of the children of split frames
+  WS_ENTRIES_G,  // queue of the two-item classes that the small-subtree walk takes
+  WS_SUB_G,      // pair supports of the regions' rows
+  WS_SUB_ITEMS,  // items of the walk's later rounds
+  WS_SUB_UNITS,  // units of its parts' own rows
+  WS_SUB_TILES,  // tiles of pairs of its later rounds
+  WS_SUB_LISTS,  // row lists of its later rounds
+  WS_SUB_STATE,
   WS_FILT_TABLE, // closed / maximal output: hash table and flags
   WS_FILT_OFF,   // the kept itemsets: offsets
   WS_FILT_ITEMS, // items
@@ -160,7 +168,8 @@ struct alignas(128) DevCtrl {
   uint32_t n_proj_classes;           // classes whose database part was built
   uint32_t n_proj_items;             // work items of the projection
   uint32_t pstack_need;              // largest warp stack (words) a projected class asked for
-  uint32_t pad1[25];
+  uint32_t n_entries_g;              // two-item classes that the small-subtree walk takes
+  uint32_t pad1[24];
   // line 2: termination and progress (polled)
   alignas(128) uint32_t pending;     // unfinished queue entries
   uint32_t progress;                 // nodes finished (any CTA), the no-progress timer's clock
@@ -346,6 +355,39 @@ struct EngineConfig {
 
 // Everything one mining call launches, with its geometry and buffers.  The
 // buffers live in a Workspace (the db's, or a plan's own for graph replays).
+constexpr uint32_t kNoGram = 0xffffffffu;
+
+// The walk of small subtrees (proj_sub.cu), run in rounds between the projection and k_dfs_proj.
+constexpr uint32_t kSubRounds = 48;
+constexpr uint32_t kSubItemCap = 1u << 17;  // items of a round after the first
+constexpr uint32_t kSubTileCap = 1u << 17;  // tiles of pairs of a round after the first
+constexpr uint64_t kSubListCap = 1ull << 21;  // words of a round's row lists
+constexpr uint64_t kSubGramCap = 1ull << 24;  // words of G: two halves, of this round's and the next one's pairs
+constexpr uint32_t kSubTask = 0xfffffffeu;  // SubItem.m: the rest of a subtree
+// A part: the transactions of region roff4 (units of 4 words of Y; kNoop: no work) that hold path_len of its rows, and
+// n candidate rows (list: the path rows, then the candidates)
+struct alignas(32) SubItem {
+  uint32_t roff4, list, path_len, n;
+  uint32_t goff, m;  // its pair supports, and the extension to walk: by candidate m; kSubTask: the part itself
+  uint32_t pad[2];
+};
+struct alignas(32) SubTile {
+  uint32_t roff4, list, path_len, n;
+  uint32_t goff, blocks, chunk, pad;  // blocks of rows (a | b << 16), words
+};
+struct alignas(32) SubUnit {  // rows j0 .. of a part's own region, over 256 words of the source region
+  uint32_t src4, list, path_len_cnt, j0;  // (path_len | rows << 16)
+  uint32_t dst_lo, dst_hi, stride, unit;  // words of Y; unit | words << 16
+};
+struct SubState {
+  unsigned long long g_top[2], l_top[2];  // words in use of each half of G and of the lists
+  uint32_t arrived, progress;             // grid barrier: CTAs arrived, items and tiles taken
+  uint32_t item_head[kSubRounds], item_n[kSubRounds + 1], tile_n[kSubRounds + 1],
+      unit_n[kSubRounds + 1];
+};
+constexpr uint32_t kGramRows = 8;             // rows per side of a tile
+constexpr uint32_t kGramWords = 512;          // words per tile
+
 struct EnginePlan {
   uint32_t n1 = 0, minsup = 1, stride = 0, bytes_per_row_alg = 0;
   const uint32_t* bits = nullptr;
@@ -392,6 +434,14 @@ struct EnginePlan {
   uint2* d_entries_f = nullptr;
   uint4* d_dq = nullptr;
   uint32_t dq_cap = 0;
+  bool sub = false;  // small subtrees walked by proj_sub.cu
+  uint32_t *d_G = nullptr, *d_goff = nullptr, *d_tileoff = nullptr;
+  uint2* d_entries_g = nullptr;
+  SubItem* d_sub_items = nullptr;
+  SubTile* d_sub_tiles = nullptr;
+  SubUnit* d_sub_units = nullptr;
+  uint32_t* d_sub_lists = nullptr;
+  SubState* d_sub_state = nullptr;
   uint64_t proj_arena_words = 0, split_words = 0;
   float ms_pair = 0.f, ms_total = 0.f;  // device time of the pair kernel / of all launches so far
   unsigned long long* d_cta_time = nullptr;  // per-CTA [start, end] of the DFS (with timing only)
@@ -530,6 +580,8 @@ struct LevelLaunch {
   const uint32_t* eoffx;           // optional (projected DFS): entry offset per queue position, bit 31 =
                                    // the class's entries go to the fallback queue entries_f
   uint2* entries_f;
+  const uint32_t* goff;            // optional: by row, != kNoGram = the class's entries go to entries_g
+  uint2* entries_g;
   uint32_t leaves;                 // 1: records only for the leaves of levels 1 and 2 (k_level2_leaves)
 };
 cudaError_t launch_level2(const LevelLaunch& p, cudaStream_t st);
@@ -608,7 +660,42 @@ struct ProjLaunch {
   uint32_t* Y;
   uint32_t* T;
   DevCtrl* ctrl;
+  // small subtrees (NULL state: not used): pair supports of the classes' rows within g_cap words of G
+  SubState* state;
+  uint32_t* G;
+  uint64_t g_cap;
+  uint32_t* goff;        // n1, by class: word offset in G, or kNoGram
+  uint32_t* tileoff;     // n1 + 1, by queue position: tiles of k_gram
 };
+struct SubLaunch {
+  uint32_t* Y;
+  uint64_t arena_words;
+  uint32_t* G;
+  uint64_t g_cap;
+  const uint64_t* yoff;
+  const uint32_t *row_order, *tileoff;
+  uint32_t n1, minsup;
+  const uint2* entries_g;
+  SubItem* items;   // two arrays of kSubItemCap
+  SubTile* tiles;   // kSubTileCap
+  SubUnit* units;   // kSubTileCap
+  uint32_t* lists;  // two arrays of kSubListCap words
+  SubState* state;
+  uint64_t* out_off;
+  uint32_t *out_items, *out_supp;
+  uint64_t cap_sets, cap_items;
+  DevCtrl* ctrl;
+  unsigned long long *class_sets, *class_work;
+  uint64_t max_sets;
+  uint32_t leaves;
+  uint4* dq;
+  uint32_t dq_cap;
+};
+cudaError_t launch_sub(const SubLaunch& p, int num_sms, cudaStream_t st);
+__host__ __device__ inline uint32_t sub_gram_tiles(uint32_t k, uint32_t W) {
+  const uint32_t nb = (k + kGramRows - 1) / kGramRows;
+  return nb * (nb + 1) / 2 * ((W + kGramWords - 1) / kGramWords);
+}
 cudaError_t launch_proj_plan(const ProjLaunch& q, cudaStream_t st);
 cudaError_t launch_proj_build(const ProjLaunch& q, int num_sms, cudaStream_t st);
 cudaError_t launch_dfs_proj(const DfsLaunch& p, uint32_t grid, uint32_t max_len, cudaStream_t st);

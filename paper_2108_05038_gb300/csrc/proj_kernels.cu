@@ -39,54 +39,13 @@
 #include <map>
 #include <mutex>
 
-#include "fim_internal.cuh"
+#include "proj_device.cuh"
 
 namespace fim {
 namespace {
 
-constexpr uint32_t kFull = 0xffffffffu;
-constexpr uint64_t kNotProjected = ~0ull;
 constexpr uint32_t kQueueF = 0x80000000u;  // eoffx: the class's entries go to the fallback queue
-constexpr uint32_t kGroupWords = 4;         // projection work item: 4 bitmap words (128 transactions) ...
 constexpr uint32_t kGroupRows = 32;         // ... of up to 32 survivors
-constexpr uint32_t kNoop = 0xffffffffu;     // queue item that carries no work (its region did not fit)
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Exclusive block-wide scan.  tmp: 33 shared elements; tmp[32] receives the
-// block total.  Two barriers inside; the caller barriers before reusing tmp.
-template <typename T>
-__device__ __forceinline__ T block_excl_scan(T v, T* tmp) {
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  T x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const T y = __shfl_up_sync(kFull, x, o);
-    if (lane >= (uint32_t)o) x += y;
-  }
-  if (lane == 31) tmp[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    const T w = lane < nw ? tmp[lane] : T(0);
-    T wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const T y = __shfl_up_sync(kFull, wi, o);
-      if (lane >= (uint32_t)o) wi += y;
-    }
-    if (lane < nw) tmp[lane] = wi - w;
-    if (lane == 31) tmp[32] = wi;
-  }
-  __syncthreads();
-  return tmp[warp] + x - v;
-}
-
-__host__ __device__ inline uint32_t words_of(uint32_t supp) { return (supp + 31) / 32; }
-__host__ __device__ inline uint32_t padded_words(uint32_t supp) { return (words_of(supp) + 3) & ~3u; }
 
 // ---------------------------------------------------------------------------
 // Phase 3, planning (one CTA): which classes get a database part, where it
@@ -94,15 +53,19 @@ __host__ __device__ inline uint32_t padded_words(uint32_t supp) { return (words_
 // fallback queue, all in queue order (LPT on the estimate, Sec. 8.2), so the
 // budgets go to the classes that start first.
 __global__ void __launch_bounds__(1024) k_proj_plan(const ProjLaunch P) {
-  __shared__ unsigned long long sy[33], st[33], sbytes[33];
-  __shared__ uint32_t sa[33], sb[33], sc[33], sd[33], se[33];
-  __shared__ unsigned long long carry_y, carry_t, carry_b;
-  __shared__ uint32_t carry_p, carry_f, carry_i, carry_c, carry_n;
+  __shared__ unsigned long long sy[33], st[33], sg[33];
+  __shared__ uint32_t sa[33], sb[33], sc[33], sh[33], sx[33];
+  __shared__ unsigned long long carry_y, carry_t, carry_b, carry_g;
+  __shared__ uint32_t carry_p, carry_f, carry_i, carry_c, carry_n, carry_h, carry_x;
   if (threadIdx.x == 0) {
-    carry_y = carry_t = carry_b = 0;
-    carry_p = carry_f = carry_i = carry_c = carry_n = 0;
+    carry_y = carry_t = carry_b = carry_g = 0;
+    carry_p = carry_f = carry_i = carry_c = carry_n = carry_h = carry_x = 0;
   }
+  if (P.state)
+    for (uint32_t t = threadIdx.x; t < sizeof(SubState) / 4; t += blockDim.x) reinterpret_cast<uint32_t*>(P.state)[t] = 0;
   __syncthreads();
+  unsigned long long my_b = 0;        // totals that no position depends on: operand bytes,
+  uint32_t my_c = 0, my_n = 0;        // rows of the projected classes, projected classes
   for (uint32_t base = 0; base < P.n1; base += blockDim.x) {
     const uint32_t q = base + threadIdx.x;
     const bool in = q < P.n1;
@@ -118,24 +81,34 @@ __global__ void __launch_bounds__(1024) k_proj_plan(const ProjLaunch P) {
     const unsigned long long tex = block_excl_scan<unsigned long long>(tsz, st);
     const unsigned long long ybase = carry_y + yex, tbase = carry_t + tex;
     const bool proj = elig && ybase + ysz <= P.y_cap_words && tbase + tsz <= P.t_cap;
-    const uint32_t neP = proj ? ne : 0u, neF = proj ? 0u : ne;
+    // pair supports of the class's rows (small subtrees): a triangle of k (k - 1) / 2 words in G, and the k rows' own
+    const unsigned long long gsz = proj && P.state ? (unsigned long long)k * (k + 1) / 2 : 0ull;
+    const unsigned long long gex = P.state ? block_excl_scan<unsigned long long>(gsz, sg) : 0ull;
+    const bool gram = gsz && carry_g + gex + gsz <= P.g_cap;
+    const uint32_t neP = proj && !gram ? ne : 0u, neF = proj ? 0u : ne, neG = gram ? ne : 0u;
     const uint32_t nit = proj ? (Wp / kGroupWords) * ((k + kGroupRows - 1) / kGroupRows) : 0u;
     const uint32_t pex = block_excl_scan<uint32_t>(neP, sa);
     const uint32_t fex = block_excl_scan<uint32_t>(neF, sb);
     const uint32_t iex = block_excl_scan<uint32_t>(nit, sc);
-    const uint32_t cex = block_excl_scan<uint32_t>(proj ? k : 0u, sd);  // rows of the projected classes
-    const uint32_t nex = block_excl_scan<uint32_t>(proj ? 1u : 0u, se);   // projected classes
-    (void)cex;
-    (void)nex;
+    uint32_t hex = 0, xex = 0;
+    if (P.state) {
+      hex = block_excl_scan<uint32_t>(neG, sh);
+      xex = block_excl_scan<uint32_t>(gram ? sub_gram_tiles(k, words_of(s)) : 0u, sx);
+    }
     // Phase 3's operand bytes: the row read once, its transactions written and read, one word gathered per
     // (survivor, transaction), the bitmaps written
-    const unsigned long long pb = proj ? 4ull * P.stride + 8ull * s + 4ull * k * s + 4ull * k * Wp : 0ull;
-    (void)block_excl_scan<unsigned long long>(pb, sbytes);
+    my_b += proj ? 4ull * P.stride + 8ull * s + 4ull * k * s + 4ull * k * Wp : 0ull;
+    my_c += proj ? k : 0u;
+    my_n += proj ? 1u : 0u;
     if (in) {
       P.yoff[i] = proj ? ybase : kNotProjected;
       P.toff[i] = proj ? tbase : kNotProjected;
-      P.eoffx[q] = proj ? carry_p + pex : (kQueueF | (carry_f + fex));
+      P.eoffx[q] = gram ? carry_h + hex : proj ? carry_p + pex : (kQueueF | (carry_f + fex));
       P.itemoff[q] = carry_i + iex;
+      if (P.state) {
+        P.goff[i] = gram ? (uint32_t)(carry_g + gex) : kNoGram;
+        P.tileoff[q] = carry_x + xex;
+      }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -144,14 +117,30 @@ __global__ void __launch_bounds__(1024) k_proj_plan(const ProjLaunch P) {
       carry_p += sa[32];
       carry_f += sb[32];
       carry_i += sc[32];
-      carry_c += sd[32];
-      carry_n += se[32];
-      carry_b += sbytes[32];
+      if (P.state) {
+        carry_g += sg[32];
+        carry_h += sh[32];
+        carry_x += sx[32];
+      }
     }
     __syncthreads();
   }
+  my_c = __reduce_add_sync(kFull, my_c);
+  my_n = __reduce_add_sync(kFull, my_n);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) my_b += __shfl_xor_sync(kFull, my_b, o);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&carry_c, my_c);
+    atomicAdd(&carry_n, my_n);
+    atomicAdd(&carry_b, my_b);
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     P.itemoff[P.n1] = carry_i;
+    P.ctrl->n_entries_g = carry_h;
+    if (P.state) {
+      P.tileoff[P.n1] = carry_x;
+    }
     P.ctrl->arena_top = (carry_y + 31) & ~31ull;  // split regions are carved after the class regions
     P.ctrl->proj_bytes = carry_b;
     P.ctrl->proj_pending = carry_p;
@@ -189,9 +178,12 @@ __global__ void __launch_bounds__(256) k_proj_tids(const ProjLaunch P) {
     R[2] = 1;
     R[3] = words_of(s);
     R[4] = i;
-    R[5] = R[6] = R[7] = 0;
+    R[5] = P.state ? P.goff[i] : kNoGram;
+    R[6] = R[7] = 0;
     R[8] = P.rank_item[P.frows[i]];
   }
+  if (P.state && P.goff[i] != kNoGram && words_of(s) > kGramWords)  // (its pair supports are added up)
+    for (uint32_t j = threadIdx.x; j < k * (k + 1) / 2; j += blockDim.x) P.G[P.goff[i] + j] = 0;
   for (uint32_t j = threadIdx.x; j < k; j += blockDim.x)
     R[12 + j] = P.rank_item[P.frows[P.sitems[P.soff[i] + j]]];
   uint32_t carry = 0;
@@ -310,30 +302,7 @@ __global__ void __launch_bounds__(256) k_proj_bits(const ProjLaunch P) {
 constexpr int kG = 8;   // candidates counted per round
 constexpr int kPR = 2;  // prefix words per lane per chunk (64 words)
 constexpr unsigned long long kIdleNs = 2000000000ull;  // no item finished anywhere for 2 s: give up
-constexpr uint32_t kIdentity = 0xffffffffu;  // frame list: every row of the region, in order
 constexpr unsigned long long kDiffFrame = 1ull;  // frame prefix marker: the survivors are held as diffsets
-
-__device__ __forceinline__ uint32_t ld_volatile(const uint32_t* a) { return *(volatile const uint32_t*)a; }
-
-struct RegionView {
-  const uint32_t* R;     // header
-  const uint32_t* rids;  // item id of each row
-  const uint32_t* Y;     // rows
-  uint32_t k, Wp, xlen, W, cls;
-};
-
-__device__ __forceinline__ RegionView region_view(const uint32_t* R) {
-  RegionView v;
-  v.R = R;
-  v.k = R[0];
-  v.Wp = R[1];
-  v.xlen = R[2];
-  v.W = R[3];
-  v.cls = R[4];
-  v.rids = R + 8 + ((v.xlen + 3) & ~3u);
-  v.Y = R + region_rows_off(v.xlen, v.k);
-  return v;
-}
 
 __global__ void __launch_bounds__(kProjThreads, kProjCtasPerSm) k_dfs_proj(const DfsLaunch p, const uint32_t max_len) {
   if (p.cta_time && threadIdx.x == 0) p.cta_time[2 * blockIdx.x] = global_ns();
