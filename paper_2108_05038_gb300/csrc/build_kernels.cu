@@ -25,8 +25,9 @@ constexpr uint32_t kSmemHistMax = 12288;  // items counted in shared memory (48 
 // items).  Only items[0, off[D]) is ever read, whatever the offsets: a
 // transaction whose range is reversed or leaves [0, off[D]] is reported and
 // skipped, and so is every transaction when off[0] != 0.
-// flags = [error bits (and DEV_NOTE_REPEATS), longest transaction, off[0], off[D], pairs (u64)], pairs = the sum
-// of len (len - 1) / 2 over the transactions of len distinct items (what counting pairs from the transactions costs).
+// flags (kBuildFlags words) = [error bits (and DEV_NOTE_REPEATS), longest transaction, off[0], off[D], pairs (u64),
+// distinct (u64), rows (by k_item_rank)]: over the transactions of len distinct items the sums of len (len - 1) / 2
+// (what counting pairs from the transactions costs) and of len.
 constexpr uint32_t kShortTx = 64;
 
 __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* __restrict__ items, uint32_t D,
@@ -44,7 +45,7 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
     flags[3] = nnz;
   }
   uint32_t local_max = 0, local_err = first != 0 ? DEV_ERR_OFFSETS : 0u;
-  uint64_t local_pairs = 0;
+  uint64_t local_pairs = 0, local_distinct = 0;
   auto bump = [&](uint32_t it) {
     if (use_smem) atomicAdd(&hist[it], 1u);
     else atomicAdd(&cnt[it], 1u);
@@ -91,6 +92,7 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
       }
       local_max = max(local_max, distinct);
       local_pairs += (uint64_t)distinct * (distinct - 1) / 2;
+      local_distinct += distinct;
     }
     for (uint32_t pend = __ballot_sync(0xffffffffu, wide); pend; pend &= pend - 1) {
       const uint32_t src = __ffs(pend) - 1;
@@ -116,20 +118,61 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
         if (count) bump(it);
       }
       local_max = max(local_max, distinct);
-      if (lane == 0) local_pairs += (uint64_t)distinct * (distinct - 1) / 2;
+      if (lane == 0) {
+        local_pairs += (uint64_t)distinct * (distinct - 1) / 2;
+        local_distinct += distinct;
+      }
     }
   }
   if (local_err) atomicOr(&flags[0], local_err);
   local_max = __reduce_max_sync(0xffffffffu, local_max);
   if (lane == 0 && local_max) atomicMax(&flags[1], local_max);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) local_pairs += __shfl_xor_sync(0xffffffffu, local_pairs, o);
-  if (lane == 0 && local_pairs)
+  for (int o = 16; o > 0; o >>= 1) {
+    local_pairs += __shfl_xor_sync(0xffffffffu, local_pairs, o);
+    local_distinct += __shfl_xor_sync(0xffffffffu, local_distinct, o);
+  }
+  if (lane == 0 && local_distinct) {
     atomicAdd(reinterpret_cast<unsigned long long*>(flags + 4), (unsigned long long)local_pairs);
+    atomicAdd(reinterpret_cast<unsigned long long*>(flags + 6), (unsigned long long)local_distinct);
+  }
   if (use_smem) {
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < N; i += blockDim.x)
       if (hist[i]) atomicAdd(&cnt[i], hist[i]);
+  }
+}
+
+// Rows of the items: ascending support, ties by id, items below the prefilter support left out.  One warp per item i
+// counts the items before it, #{j : cnt_j < cnt_i, or cnt_j = cnt_i and j < i}, and those below the prefilter: N^2 / 32
+// comparisons (10,000 items: 9 us), against a copy of the counts to the host, a sort there (0.3 ms) and a copy back, with
+// the device idle meanwhile.  Also writes 0, 1, .. to iota and the number of rows to flags[8].
+__global__ void __launch_bounds__(256) k_item_rank(const uint32_t* __restrict__ cnt, uint32_t N, uint32_t prefilter,
+                                                   int32_t* __restrict__ item_rank, uint32_t* __restrict__ rank_item,
+                                                   uint32_t* __restrict__ supp, uint32_t* __restrict__ iota,
+                                                   uint32_t* __restrict__ flags) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= N) return;  // (whole warps leave together)
+  const uint32_t c = __ldg(cnt + i);
+  uint32_t before = 0, below = 0;
+#pragma unroll 4
+  for (uint32_t j = lane; j < N; j += 32) {
+    const uint32_t cj = __ldg(cnt + j);
+    before += cj < c || (cj == c && j < i);
+    below += cj < prefilter;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  below = __reduce_add_sync(0xffffffffu, below);
+  if (lane == 0) {
+    const bool kept = c >= prefilter;
+    item_rank[i] = kept ? (int32_t)(before - below) : -1;
+    iota[i] = i;
+    if (kept) {
+      rank_item[before - below] = i;
+      supp[before - below] = c;
+    }
+    if (i == 0) flags[8] = N - below;
   }
 }
 
@@ -138,9 +181,12 @@ __global__ void k_item_count(const uint32_t* __restrict__ off, const uint32_t* _
 // bit); at each position j the lanes whose j-th item maps to the same row are
 // grouped by __match_any_sync, and one lane ORs the whole group's bits into the
 // word, so a popular item costs one atomic per word and position instead of one
-// per transaction.  The offsets and ids were validated by K1.
+// per transaction.  The offsets and ids were validated by K1, whose flags are read first: a database that it
+// found invalid is not touched.
 __global__ void k_bitmap_build(const uint32_t* __restrict__ off, const uint32_t* __restrict__ items, uint32_t D,
-                               const int32_t* __restrict__ item_rank, uint32_t* __restrict__ bits, uint32_t stride) {
+                               const int32_t* __restrict__ item_rank, uint32_t* __restrict__ bits, uint32_t stride,
+                               const uint32_t* __restrict__ flags) {
+  if ((flags[0] & (DEV_ERR_OFFSETS | DEV_ERR_ITEM_RANGE)) != 0u || flags[2] != 0u) return;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
   for (uint32_t w0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32u; w0 < D; w0 += warps * 32u) {
@@ -315,10 +361,17 @@ cudaError_t launch_item_count(const uint32_t* off, const uint32_t* items, uint32
   return cudaGetLastError();
 }
 
+cudaError_t launch_item_rank(const uint32_t* cnt, uint32_t N, uint32_t prefilter, int32_t* item_rank, uint32_t* rank_item,
+                             uint32_t* supp, uint32_t* iota, uint32_t* flags, cudaStream_t st) {
+  k_item_rank<<<(N + 7) / 8, 256, 0, st>>>(cnt, N, prefilter, item_rank, rank_item, supp, iota, flags);
+  note_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_bitmap_build(const uint32_t* off, const uint32_t* items, uint32_t D, const int32_t* item_rank,
-                                uint32_t* bits, uint32_t stride, cudaStream_t st) {
+                                uint32_t* bits, uint32_t stride, const uint32_t* flags, cudaStream_t st) {
   const uint32_t threads = 256;
-  k_bitmap_build<<<grid_for(D, threads), threads, 0, st>>>(off, items, D, item_rank, bits, stride);  // 32 tx per warp
+  k_bitmap_build<<<grid_for(D, threads), threads, 0, st>>>(off, items, D, item_rank, bits, stride, flags);  // 32 tx per warp
   note_launch();
   return cudaGetLastError();
 }

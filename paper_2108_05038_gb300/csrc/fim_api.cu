@@ -269,92 +269,107 @@ static fim_status db_init(fim_db* db, uint32_t D, uint32_t N, uint32_t word_bits
 }
 
 
-// Items counted (K1) on the input CSR (the caller's device arrays or the db's
-// copy of host arrays), the offsets validated on the device, rows relabelled on
-// the host, the CSR copied into the db (device input), bitmaps built (K2).
+// Items counted (K1) on the input CSR (the caller's device arrays or the db's copy of host arrays), the offsets validated
+// and the items ranked on the device, bitmaps built (K2), and one wait for the flags and the ranks: without a prefilter
+// every item gets a row, so the bitmap block is known beforehand and nothing waits for the host in between.  With a
+// prefilter the block follows the wait; past kRankItems items the host sorts.  The CSR is copied into the db last
+// (device input), once the offsets are known to be valid.
 static fim_status db_build_rows(fim_db* db, const uint32_t* src_off, const uint32_t* src_items, bool device_input) {
   cudaStream_t st = db->stream;
   const uint32_t N = db->N, D = db->D;
-  uint32_t *d_cnt = nullptr, *d_flags = nullptr;
-  const size_t fl = ((size_t)N + 1) & ~(size_t)1, cnt_words = fl + 6;  // (the 64-bit flag on 8 bytes)
-  FIM_TRY(ws_get(db->ws, WS_TALLY, cnt_words, &d_cnt));
-  d_flags = d_cnt + fl;  // [err, max_len, off[0], off[D], pairs (u64)]
-  FIM_CUDA(cudaMemsetAsync(d_cnt, 0, cnt_words * 4, st));
+  const size_t a4 = ((size_t)N + 3) & ~(size_t)3;
+  uint32_t *d_cnt = nullptr, *small = nullptr;
+  FIM_TRY(ws_get(db->ws, WS_TALLY, N, &d_cnt));
+  FIM_TRY(ws_get(db->ws, WS_DB_SMALL, kBuildFlags + 4 * a4, &small));
+  uint32_t* const d_flags = small;
+  db->d_item_rank = reinterpret_cast<int32_t*>(small + kBuildFlags);
+  db->d_rank_item = small + kBuildFlags + a4;
+  db->d_supp = small + kBuildFlags + 2 * a4;
+  db->d_iota = small + kBuildFlags + 3 * a4;
+  FIM_CUDA(cudaMemsetAsync(d_cnt, 0, (size_t)N * 4, st));
+  FIM_CUDA(cudaMemsetAsync(d_flags, 0, kBuildFlags * 4, st));
   FIM_CUDA(launch_item_count(src_off, src_items, D, N, d_cnt, d_flags, st));
-  void* hcnt = nullptr;
-  FIM_TRY(stage_get(db, cnt_words * 4, &hcnt));
-  FIM_CUDA(cudaMemcpyAsync(hcnt, d_cnt, cnt_words * 4, cudaMemcpyDeviceToHost, st));
-  // Without a prefilter every item gets a row (n_rows = N), so the bitmap block is known before the counts:
-  // it is cleared behind the counts' copy, while the host waits for that copy alone and relabels the rows.
-  const bool early_bits = db->prefilter == 0 && (size_t)N * db->stride > 0;
-  if (early_bits) {
+  const bool on_device = N <= kRankItems;
+  const bool early = on_device && db->prefilter == 0;
+  if (on_device)
+    FIM_CUDA(launch_item_rank(d_cnt, N, db->prefilter, db->d_item_rank, db->d_rank_item, db->d_supp, db->d_iota, d_flags, st));
+  // flags, item_rank, rank_item and supp in one copy; or (host sort) the counts in place of item_rank
+  uint32_t* h = nullptr;
+  {
+    void* p = nullptr;
+    FIM_TRY(stage_get(db, (kBuildFlags + 3 * a4) * 4, &p));
+    h = static_cast<uint32_t*>(p);
+  }
+  FIM_CUDA(cudaMemcpyAsync(h, d_flags, (kBuildFlags + (on_device ? 3 * a4 : 0)) * 4, cudaMemcpyDeviceToHost, st));
+  if (!on_device) FIM_CUDA(cudaMemcpyAsync(h + kBuildFlags, d_cnt, (size_t)N * 4, cudaMemcpyDeviceToHost, st));
+  if (early) {
+    // (the copy's wait is on an event of its own: the host fills its lists while the bitmaps are built)
     if (!db->cnt_done) FIM_CUDA(cudaEventCreateWithFlags(&db->cnt_done, cudaEventDisableTiming));
     FIM_CUDA(cudaEventRecord(db->cnt_done, st));
     FIM_TRY(ws_get(db->ws, WS_DB_BITS, (size_t)N * db->stride, &db->d_bits));
     FIM_CUDA(cudaMemsetAsync(db->d_bits, 0, (size_t)N * db->stride * 4, st));
+    FIM_CUDA(launch_bitmap_build(src_off, src_items, D, db->d_item_rank, db->d_bits, db->stride, d_flags, st));
     FIM_CUDA(cudaEventSynchronize(db->cnt_done));
     db->stage_used = 0;
   } else {
     FIM_TRY(stream_sync(db));
   }
-  std::vector<uint32_t> cnt(static_cast<uint32_t*>(hcnt), static_cast<uint32_t*>(hcnt) + cnt_words);
-  const uint32_t* const flags = cnt.data() + fl;
-  const uint32_t err = flags[0];
-  if (flags[2] != 0) return fail(FIM_ERR_INVALID, "tx_offsets[0] must be 0");
+  const uint32_t err = h[0];
+  if (h[2] != 0) return fail(FIM_ERR_INVALID, "tx_offsets[0] must be 0");
   if (err & DEV_ERR_OFFSETS) return fail(FIM_ERR_INVALID, "tx_offsets is not non-decreasing");
   if (err & DEV_ERR_ITEM_RANGE) return fail(FIM_ERR_INVALID, "an item id is >= N");
-  db->max_tx_len = flags[1];
+  db->max_tx_len = h[1];
   db->tx_repeats = (err & DEV_NOTE_REPEATS) != 0;
-  db->tx_pairs = flags[4] | (uint64_t)flags[5] << 32;
-  db->tx_distinct = std::accumulate(cnt.begin(), cnt.begin() + N, (uint64_t)0);
-  if (device_input) {  // the offsets are valid: keep a copy of the CSR (the sample draw reads it)
-    db->nnz = flags[3];
+  db->tx_pairs = h[4] | (uint64_t)h[5] << 32;
+  db->tx_distinct = h[6] | (uint64_t)h[7] << 32;
+  if (device_input) {  // keep a copy of the CSR (the sample draw reads it)
+    db->nnz = h[3];
     FIM_TRY(ws_get(db->ws, WS_DB_TXOFF, (size_t)D + 1, &db->d_tx_off));
     FIM_TRY(ws_get(db->ws, WS_DB_TXITEMS, std::max<uint64_t>(1, db->nnz), &db->d_tx_items));
     FIM_CUDA(cudaMemcpyAsync(db->d_tx_off, src_off, ((size_t)D + 1) * 4, cudaMemcpyDeviceToDevice, st));
     if (db->nnz)
       FIM_CUDA(cudaMemcpyAsync(db->d_tx_items, src_items, db->nnz * 4ull, cudaMemcpyDeviceToDevice, st));
   }
-  // kept items by ascending support, ties by id: one sort of (support, id) keys
-  std::vector<uint64_t> key;
-  key.reserve(N);
-  for (uint32_t i = 0; i < N; ++i)
-    if (cnt[i] >= db->prefilter) key.push_back(((uint64_t)cnt[i] << 32) | i);
-  std::sort(key.begin(), key.end());
-  std::vector<uint32_t> kept(key.size());
-  for (size_t k = 0; k < key.size(); ++k) kept[k] = (uint32_t)key[k];
-  db->n_rows = (uint32_t)kept.size();
-  db->rank_item = kept;
-  db->supp.resize(db->n_rows);
-  db->item_rank.assign(N, -1);
-  for (uint32_t r = 0; r < db->n_rows; ++r) {
-    db->supp[r] = cnt[kept[r]];
-    db->item_rank[kept[r]] = (int32_t)r;
-  }
-  // item_rank | rank_item | supp | iota in one block (each part 16-byte aligned), filled by one copy
-  const size_t a4 = ((size_t)N + 3) & ~(size_t)3, r4 = ((size_t)db->n_rows + 3) & ~(size_t)3;
-  uint32_t* small = nullptr;
-  FIM_TRY(ws_get(db->ws, WS_DB_SMALL, a4 + 3 * r4 + 4, &small));
-  db->d_item_rank = reinterpret_cast<int32_t*>(small);
-  db->d_rank_item = small + a4;
-  db->d_supp = small + a4 + r4;
-  db->d_iota = small + a4 + 2 * r4;
-  FIM_TRY(ws_get(db->ws, WS_DB_BITS, std::max<size_t>(1, (size_t)db->n_rows * db->stride), &db->d_bits));
-  {
-    void* h = nullptr;
-    FIM_TRY(stage_get(db, (a4 + 2 * r4) * 4, &h));
-    uint32_t* hu = static_cast<uint32_t*>(h);
+  if (on_device) {
+    const uint32_t* const q = h + kBuildFlags;
+    db->n_rows = h[8];
+    db->item_rank.assign(reinterpret_cast<const int32_t*>(q), reinterpret_cast<const int32_t*>(q) + N);
+    db->rank_item.assign(q + a4, q + a4 + db->n_rows);
+    db->supp.assign(q + 2 * a4, q + 2 * a4 + db->n_rows);
+  } else {
+    // kept items by ascending support, ties by id: one sort of (support, id) keys
+    const std::vector<uint32_t> cnt(h + kBuildFlags, h + kBuildFlags + N);
+    std::vector<uint64_t> key;
+    key.reserve(N);
+    for (uint32_t i = 0; i < N; ++i)
+      if (cnt[i] >= db->prefilter) key.push_back(((uint64_t)cnt[i] << 32) | i);
+    std::sort(key.begin(), key.end());
+    db->n_rows = (uint32_t)key.size();
+    db->rank_item.resize(db->n_rows);
+    db->supp.resize(db->n_rows);
+    db->item_rank.assign(N, -1);
+    for (uint32_t r = 0; r < db->n_rows; ++r) {
+      db->rank_item[r] = (uint32_t)key[r];
+      db->supp[r] = (uint32_t)(key[r] >> 32);
+      db->item_rank[(uint32_t)key[r]] = (int32_t)r;
+    }
+    void* p = nullptr;
+    FIM_TRY(stage_get(db, 3 * a4 * 4, &p));
+    uint32_t* hu = static_cast<uint32_t*>(p);
     std::memcpy(hu, db->item_rank.data(), (size_t)N * 4);
     if (db->n_rows) {
       std::memcpy(hu + a4, db->rank_item.data(), (size_t)db->n_rows * 4);
-      std::memcpy(hu + a4 + r4, db->supp.data(), (size_t)db->n_rows * 4);
+      std::memcpy(hu + 2 * a4, db->supp.data(), (size_t)db->n_rows * 4);
     }
-    FIM_CUDA(cudaMemcpyAsync(small, hu, (a4 + 2 * r4) * 4, cudaMemcpyHostToDevice, st));
+    FIM_CUDA(cudaMemcpyAsync(db->d_item_rank, hu, 3 * a4 * 4, cudaMemcpyHostToDevice, st));
+    FIM_CUDA(launch_iota(db->d_iota, db->n_rows, st));
   }
-  FIM_CUDA(launch_iota(db->d_iota, db->n_rows, st));
-  if (db->n_rows) {
-    if (!early_bits) FIM_CUDA(cudaMemsetAsync(db->d_bits, 0, (size_t)db->n_rows * db->stride * 4, st));
-    FIM_CUDA(launch_bitmap_build(db->d_tx_off, db->d_tx_items, D, db->d_item_rank, db->d_bits, db->stride, st));
+  if (!early) {
+    FIM_TRY(ws_get(db->ws, WS_DB_BITS, std::max<size_t>(1, (size_t)db->n_rows * db->stride), &db->d_bits));
+    if (db->n_rows) {
+      FIM_CUDA(cudaMemsetAsync(db->d_bits, 0, (size_t)db->n_rows * db->stride * 4, st));
+      FIM_CUDA(launch_bitmap_build(src_off, src_items, D, db->d_item_rank, db->d_bits, db->stride, d_flags, st));
+    }
   }
   return FIM_OK;
 }

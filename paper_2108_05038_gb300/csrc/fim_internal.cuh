@@ -122,7 +122,7 @@ enum WsSlot {
   WS_DB_TXOFF,
   WS_DB_TXITEMS,
   WS_DB_BITS,
-  WS_DB_SMALL,  // item_rank (N) | rank_item (rows) | supp (rows) | iota (rows), each 16-byte aligned
+  WS_DB_SMALL,  // flags | item_rank | rank_item | supp | iota (N words each, 16-byte aligned)
   // projected DFS: per-class database parts and the warps' stacks
   WS_PROJ_META,  // yoff (n1 u64) | toff (n1 u64) | itemoff (n1 + 1 u32) | eoffx (n1 u32)
   WS_PROJ_Y,     // bitmaps of every class's survivors over the class's transactions
@@ -243,7 +243,7 @@ struct fim_db {
   bool est_redo = false;  // the deferred sample needs the synchronous path (itemset limit or a retry)
   uint32_t est_redo_minsup = 0;  // the sample minsup that redo starts at (0: the estimate's own)
   cudaEvent_t est_done = nullptr;
-  cudaEvent_t cnt_done = nullptr;  // the build's item counts copied to the host (the bitmap clearing behind them)
+  cudaEvent_t cnt_done = nullptr;  // the build's flags and ranks copied to the host (the bitmaps built behind them)
   void* est_pin = nullptr;
   size_t est_pin_cap = 0;
   const uint32_t* d_est_order = nullptr;
@@ -507,7 +507,11 @@ fim_status stream_sync(fim_db* db);
 cudaError_t launch_item_count(const uint32_t* off, const uint32_t* items, uint32_t D, uint32_t N, uint32_t* cnt,
                               uint32_t* flags, cudaStream_t st);
 cudaError_t launch_bitmap_build(const uint32_t* off, const uint32_t* items, uint32_t D, const int32_t* item_rank,
-                                uint32_t* bits, uint32_t stride, cudaStream_t st);
+                                uint32_t* bits, uint32_t stride, const uint32_t* flags, cudaStream_t st);
+constexpr uint32_t kBuildFlags = 12;      // words of the item count's flags (three 16-byte units)
+constexpr uint32_t kRankItems = 16384;    // items ranked on the device (N^2 comparisons); more are sorted on the host
+cudaError_t launch_item_rank(const uint32_t* cnt, uint32_t N, uint32_t prefilter, int32_t* item_rank, uint32_t* rank_item,
+                             uint32_t* supp, uint32_t* iota, uint32_t* flags, cudaStream_t st);
 cudaError_t launch_sample_build(const uint32_t* off, const uint32_t* items, uint32_t D, const int32_t* item_rank,
                                 uint64_t seed, uint32_t m, uint32_t* sbits, uint32_t sstride, cudaStream_t st);
 cudaError_t launch_iota(uint32_t* out, uint32_t n, cudaStream_t st);
