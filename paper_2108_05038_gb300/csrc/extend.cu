@@ -15,57 +15,115 @@ namespace {
 
 __device__ __forceinline__ bool nz4(const uint4& v) { return (v.x | v.y | v.z | v.w) != 0u; }
 
-// dst[w] = AND of rows[0..n) at word w
-__global__ void k_and_rows(const uint4* __restrict__ bits4, uint32_t stride4, const uint32_t* __restrict__ rows,
-                           uint32_t n, uint4* __restrict__ dst) {
-  for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < stride4; w += gridDim.x * blockDim.x) {
-    uint4 a = __ldg(bits4 + (size_t)rows[0] * stride4 + w);
-    for (uint32_t k = 1; k < n && nz4(a); ++k) {
-      const uint4 b = __ldg(bits4 + (size_t)rows[k] * stride4 + w);
-      a = make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w);
+// Prefixes of at most kExtInline rows are ANDed word by word inside the counting kernel while the extra rows' reads (from
+// the L2) stay below kExtInlineBytes over all candidates, about 10 us; else t(P) is built once.
+constexpr uint32_t kExtInline = 8;
+constexpr uint64_t kExtInlineBytes = 64ull << 20;
+
+// dst[w] = AND of rows[0..n) at word w (the row list in the host's memory: each CTA reads it once, 256 rows at a time)
+__global__ void __launch_bounds__(256) k_and_rows(const uint4* __restrict__ bits4, uint32_t stride4, const uint32_t* rows,
+                                                  uint32_t n, uint4* dst) {
+  __shared__ uint32_t s_rows[256];
+  for (uint32_t k0 = 0; k0 < n; k0 += 256) {
+    const uint32_t m = min(256u, n - k0);
+    __syncthreads();
+    if (threadIdx.x < m) s_rows[threadIdx.x] = rows[k0 + threadIdx.x];
+    __syncthreads();
+    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < stride4; w += gridDim.x * blockDim.x) {
+      uint4 a = k0 ? dst[w] : make_uint4(~0u, ~0u, ~0u, ~0u);
+      for (uint32_t k = 0; k < m && nz4(a); ++k) {
+        const uint4 b = __ldg(bits4 + (size_t)s_rows[k] * stride4 + w);
+        a = make_uint4(a.x & b.x, a.y & b.y, a.z & b.z, a.w & b.w);
+      }
+      dst[w] = a;
     }
-    dst[w] = a;
   }
 }
 
-// out[c] = popc(pre & row(cand[c])); one CTA per candidate at a time, eight 16-byte loads per thread
-// in flight; a candidate whose row is absent (kNoRow) has no common transaction with anything
+// out[c] = popc(row(pre[0]) & .. & row(pre[n_pre - 1]) & row(cand[c])), or, with t(P) given (pre4), popc(t(P) & row(cand[c])).
+// kS warps of a CTA share a candidate, eight 16-byte loads per lane in flight; a candidate whose row is absent (kNoRow)
+// has no common transaction with anything.  The row lists are read from, and the counts written to, the host's pinned
+// memory: a call is one kernel, without the copies that moving them took and without a kernel for a short prefix (1,000
+// candidates of 12.5 KB, two prefix items: 35 us a call before, 22 now).  Bound by HBM once the rows exceed the L2: every
+// candidate's warps run at once, so that no last round of a few candidates leaves most of the chip idle (4,001 rows of
+// 125 KB: 102 us a call, 117 with a CTA per candidate and 4.4 rounds).
 constexpr uint32_t kNoRow = 0xffffffffu;
-__global__ void __launch_bounds__(256) k_extension_counts(const uint4* __restrict__ bits4, uint32_t stride4,
-                                                          const uint4* pre4, const uint32_t* __restrict__ cand,
-                                                          uint32_t n_cand, uint32_t* __restrict__ out) {
-  __shared__ uint32_t wsum[8];
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t c = blockIdx.x; c < n_cand; c += gridDim.x) {
-    const uint32_t row = cand[c];
+constexpr uint32_t kExtThreads = 256, kExtWarps = kExtThreads / 32;
+template <uint32_t kS>
+__global__ void __launch_bounds__(kExtThreads) k_extension_counts(const uint4* __restrict__ bits4, uint32_t stride4,
+                                                                  const uint4* __restrict__ pre4, const uint32_t* pre,
+                                                                  uint32_t n_pre, const uint32_t* cand, uint32_t n_cand,
+                                                                  uint32_t* out) {
+  __shared__ uint32_t wsum[kExtWarps];
+  __shared__ uint32_t s_pre[kExtInline];
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, part = warp % kS;
+  if (!pre4 && threadIdx.x < n_pre) s_pre[threadIdx.x] = pre[threadIdx.x];
+  __syncthreads();
+  for (uint32_t c0 = blockIdx.x * (kExtWarps / kS); c0 < n_cand; c0 += gridDim.x * (kExtWarps / kS)) {
+    const uint32_t c = c0 + warp / kS;
+    const uint32_t row = c < n_cand ? cand[c] : kNoRow;
     uint32_t s = 0;
     if (row != kNoRow) {
       const uint4* r4 = bits4 + (size_t)row * stride4;
+      const uint4* p4 = pre4 ? pre4 : bits4 + (size_t)s_pre[0] * stride4;
       constexpr uint32_t U = 8;
-      for (uint32_t w0 = threadIdx.x; w0 < stride4; w0 += U * blockDim.x) {
+      for (uint32_t w0 = part * 32 + lane; w0 < stride4; w0 += U * kS * 32) {
         uint4 a[U], b[U];
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u) {
-          const uint32_t w = w0 + u * blockDim.x;
-          a[u] = w < stride4 ? pre4[w] : make_uint4(0u, 0u, 0u, 0u);
+          const uint32_t w = w0 + u * kS * 32;
+          a[u] = w < stride4 ? __ldg(p4 + w) : make_uint4(0u, 0u, 0u, 0u);
         }
+        if (!pre4)
+          for (uint32_t t = 1; t < n_pre; ++t) {
+            const uint4* q4 = bits4 + (size_t)s_pre[t] * stride4;
 #pragma unroll
-        for (uint32_t u = 0; u < U; ++u) b[u] = nz4(a[u]) ? __ldcs(r4 + w0 + u * blockDim.x) : make_uint4(0u, 0u, 0u, 0u);
+            for (uint32_t u = 0; u < U; ++u) {
+              const uint4 x = nz4(a[u]) ? __ldg(q4 + w0 + u * kS * 32) : make_uint4(0u, 0u, 0u, 0u);
+              a[u] = make_uint4(a[u].x & x.x, a[u].y & x.y, a[u].z & x.z, a[u].w & x.w);
+            }
+          }
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) b[u] = nz4(a[u]) ? __ldcs(r4 + w0 + u * kS * 32) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (uint32_t u = 0; u < U; ++u)
           s += __popc(a[u].x & b[u].x) + __popc(a[u].y & b[u].y) + __popc(a[u].z & b[u].z) + __popc(a[u].w & b[u].w);
       }
     }
     s = __reduce_add_sync(0xffffffffu, s);
-    if (lane == 0) wsum[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t t = 0;
-      for (uint32_t k = 0; k < (blockDim.x >> 5); ++k) t += wsum[k];
-      out[c] = t;
+    if (kS == 1) {
+      if (lane == 0 && c < n_cand) out[c] = s;
+    } else {
+      if (lane == 0) wsum[warp] = s;
+      __syncthreads();
+      if (lane == 0 && part == 0 && c < n_cand) {
+        uint32_t t = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < kS; ++k) t += wsum[warp + k];
+        out[c] = t;
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
+}
+
+template <uint32_t kS>
+cudaError_t launch_counts(const uint4* bits4, uint32_t stride4, const uint4* pre4, const uint32_t* pre, uint32_t n_pre,
+                          const uint32_t* cand, uint32_t n_cand, uint32_t* out, uint32_t ctas, cudaStream_t st) {
+  const uint32_t per = kExtWarps / kS, need = (n_cand + per - 1) / per;
+  k_extension_counts<kS><<<std::min(need, ctas), kExtThreads, 0, st>>>(bits4, stride4, pre4, pre, n_pre, cand, n_cand, out);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// resident CTAs per SM of the counting kernel (its forms differ in the reduction alone), asked once
+uint32_t ext_ctas_per_sm() {
+  static const int occ = [] {
+    int o = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_extension_counts<8>, (int)kExtThreads, 0) != cudaSuccess) o = 1;
+    return std::max(1, o);
+  }();
+  return (uint32_t)occ;
 }
 
 }  // namespace
@@ -95,36 +153,40 @@ fim_status fim_extension_supports(fim_db* db, const uint32_t* prefix_items, uint
   cudaStream_t st = db->stream;
   const uint32_t stride4 = db->stride / 4;
   const uint4* bits4 = reinterpret_cast<const uint4*>(db->d_bits);
-  uint32_t* d_rows = nullptr;
-  uint32_t* d_out = nullptr;
-  FIM_TRY(ws_get(db->ws, WS_QUERY_ROWS, rows.size(), &d_rows));
-  FIM_TRY(ws_get(db->ws, WS_QUERY_OUT, n_cand, &d_out));
+  // rows, then the counts, in the pinned staging buffer, which the kernels read and write in place
   void* h = nullptr;
-  FIM_TRY(stage_get(db, rows.size() * 4, &h));
-  std::memcpy(h, rows.data(), rows.size() * 4);
-  FIM_CUDA(cudaMemcpyAsync(d_rows, h, rows.size() * 4, cudaMemcpyHostToDevice, st));
-  const uint4* pre4 = bits4 + (size_t)rows[0] * stride4;
-  if (n_prefix > 1) {
+  FIM_TRY(stage_get(db, (rows.size() + n_cand) * 4, &h));
+  uint32_t* const h_rows = static_cast<uint32_t*>(h);
+  uint32_t* const h_out = h_rows + rows.size();
+  std::memcpy(h_rows, rows.data(), rows.size() * 4);
+  const uint4* pre4 = nullptr;
+  if (n_prefix == 1) {
+    pre4 = bits4 + (size_t)rows[0] * stride4;
+  } else if (n_prefix > kExtInline || (uint64_t)n_cand * stride4 * 16 * (n_prefix - 1) > kExtInlineBytes) {
     uint4* d_pre = nullptr;
     FIM_TRY(ws_get(db->ws, WS_QUERY_PREFIX, stride4, &d_pre));
     const uint32_t threads = 256;
     const uint32_t grid = std::min<uint32_t>((stride4 + threads - 1) / threads, (uint32_t)db->num_sms * 8);
-    k_and_rows<<<std::max<uint32_t>(1, grid), threads, 0, st>>>(bits4, stride4, d_rows, n_prefix, d_pre);
+    k_and_rows<<<std::max<uint32_t>(1, grid), threads, 0, st>>>(bits4, stride4, h_rows, n_prefix, d_pre);
     note_launch();
     FIM_CUDA(cudaGetLastError());
     pre4 = d_pre;
   }
-  int occ = 0;
-  FIM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_extension_counts, 256, 0));
-  const uint32_t grid = std::min<uint32_t>(n_cand, (uint32_t)db->num_sms * (uint32_t)std::max(1, occ));
-  k_extension_counts<<<grid, 256, 0, st>>>(bits4, stride4, pre4, d_rows + n_prefix, n_cand, d_out);
-  note_launch();
-  FIM_CUDA(cudaGetLastError());
-  void* ho = nullptr;
-  FIM_TRY(stage_get(db, (size_t)n_cand * 4, &ho));
-  FIM_CUDA(cudaMemcpyAsync(ho, d_out, (size_t)n_cand * 4, cudaMemcpyDeviceToHost, st));
+  // warps per candidate: as many as still let every candidate's warps be resident at once; more candidates than
+  // that are taken eight warps at a time, so that the last round is short
+  const uint32_t ctas = (uint32_t)db->num_sms * ext_ctas_per_sm();
+  const uint64_t slots = (uint64_t)ctas * kExtWarps;
+  const uint32_t* const c = h_rows + n_prefix;
+  if (n_cand > slots || 8ull * n_cand <= slots)
+    FIM_CUDA(launch_counts<8>(bits4, stride4, pre4, h_rows, n_prefix, c, n_cand, h_out, ctas, st));
+  else if (4ull * n_cand <= slots)
+    FIM_CUDA(launch_counts<4>(bits4, stride4, pre4, h_rows, n_prefix, c, n_cand, h_out, ctas, st));
+  else if (2ull * n_cand <= slots)
+    FIM_CUDA(launch_counts<2>(bits4, stride4, pre4, h_rows, n_prefix, c, n_cand, h_out, ctas, st));
+  else
+    FIM_CUDA(launch_counts<1>(bits4, stride4, pre4, h_rows, n_prefix, c, n_cand, h_out, ctas, st));
   FIM_TRY(stream_sync(db));
-  std::memcpy(supports_out, ho, (size_t)n_cand * 4);
+  std::memcpy(supports_out, h_out, (size_t)n_cand * 4);
   return FIM_OK;
 }
 

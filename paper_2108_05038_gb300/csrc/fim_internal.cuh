@@ -115,8 +115,6 @@ enum WsSlot {
   WS_CTATIME,
   WS_PAIR_X,        // rows widened to bytes for the tensor-core pair kernel
   WS_TX_MAP,        // item -> index of its row among a sample's rows (pair counts from the transactions)
-  WS_QUERY_ROWS,    // fim_extension_supports: prefix rows | candidate rows
-  WS_QUERY_OUT,     // fim_extension_supports: one count per candidate
   WS_QUERY_PREFIX,  // fim_extension_supports: t(P) of a prefix of two or more items
   // the database's own arrays (kept in the workspace so that a freed database's memory serves the next)
   WS_DB_TXOFF,
