@@ -63,7 +63,9 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
   ep->cap_items = cfg.cap_items ? cfg.cap_items : ep->cap_sets * 6;
   ep->cap_sets = std::min(ep->cap_sets, kMaxCap);
   ep->cap_items = std::min(ep->cap_items, kMaxCap);
-  FIM_TRY(ws_get(ws, WS_CTRL, 1, &ep->d_ctrl));
+  uint8_t* ctrl = nullptr;  // the control block, then the state of the search by levels (cleared together)
+  FIM_TRY(ws_get(ws, WS_CTRL, sizeof(DevCtrl) + sizeof(LevState), &ctrl));
+  ep->d_ctrl = reinterpret_cast<DevCtrl*>(ctrl);
   if (n1 == 0) return FIM_OK;
 
   // row lists (pinned-staged uploads unless the caller already has them on the device)
@@ -258,6 +260,23 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     FIM_TRY(ws_get(ws, WS_PROJ_DQ, std::max<uint32_t>(1, ep->dq_cap), &ep->d_dq));
     FIM_TRY(ws_get(ws, WS_PROJ_T, std::max<uint64_t>(4, ep->proj_t_cap), &ep->d_T));
   }
+  // Automatic, few rows (where frame passes were chosen): by levels
+  ep->levels = cfg.mode == 2 && ep->mode == 1 && !cfg.donate && cfg.ctas_per_sm == 0 && !cfg.diffsets && !ep->leaves &&
+               n1 >= 3 && n1 < 1024 && ep->rows_base;
+  if (ep->levels) {
+    uint8_t* a = nullptr;
+    constexpr uint64_t kBytes = 2 * (kLevUnits * sizeof(LevUnit) + 4 * (kLevListWords + kLevSupWords + kLevNodes));
+    FIM_TRY(ws_get(ws, WS_LEVELS, kBytes, &a));
+    LevLaunch& l = ep->lev;
+    l.units = reinterpret_cast<LevUnit*>(a);
+    l.lists = reinterpret_cast<uint32_t*>(l.units + 2 * kLevUnits);
+    l.sups = l.lists + 2 * kLevListWords;
+    l.nodes = l.sups + 2 * kLevSupWords;
+    l.state = reinterpret_cast<LevState*>(ctrl + sizeof(DevCtrl));
+    l.rows4 = reinterpret_cast<const uint4*>(ep->rows_base);
+    l.ids = in.d_rank_item + in.frows.front();
+    FIM_CUDA(levels_ctas(db->num_sms, &ep->lev_grid));
+  }
   if (cfg.collect_times)
     for (auto& e : ep->ev) FIM_CUDA(cudaEventCreate(&e));
   return FIM_OK;
@@ -269,12 +288,12 @@ fim_status engine_alloc(Workspace& ws, EnginePlan* ep) {
     FIM_TRY(ws_get(ws, WS_OUT_ITEMS, std::max<uint64_t>(1, ep->cap_items), &ep->d_items));
     FIM_TRY(ws_get(ws, WS_OUT_SUPP, std::max<uint64_t>(1, ep->cap_sets), &ep->d_supp));
   }
-  if (ep->n1 >= 3)
+  if (ep->n1 >= 3 && !ep->levels)
     FIM_TRY(ws_get(ws, WS_ARENA, dfs_arena_cta_words(ep->stride, ep->n1, ep->maxd, ep->mode) * ep->grid, &ep->d_arena));
   if (ep->n1 >= 3 && ep->proj)
     FIM_TRY(ws_get(ws, WS_PSTACK, (uint64_t)ep->proj_grid * (kProjThreads / 32) * ep->pstack_words, &ep->d_pstack));
   if (ep->n1 >= 3 && ep->ev[0])
-    FIM_TRY(ws_get(ws, WS_CTATIME, 2ull * std::max(ep->grid, ep->proj_grid), &ep->d_cta_time));
+    FIM_TRY(ws_get(ws, WS_CTATIME, 2ull * std::max({ep->grid, ep->proj_grid, ep->lev_grid}), &ep->d_cta_time));
   return FIM_OK;
 }
 
@@ -284,7 +303,7 @@ cudaError_t engine_launch(const EnginePlan& ep, cudaStream_t st) {
 }
 
 cudaError_t engine_launch_front(const EnginePlan& ep, cudaStream_t st, bool pairs) {
-  cudaError_t ce = cudaMemsetAsync(ep.d_ctrl, 0, sizeof(DevCtrl), st);
+  cudaError_t ce = cudaMemsetAsync(ep.d_ctrl, 0, sizeof(DevCtrl) + (ep.levels ? sizeof(LevState) : 0), st);
   if (ce != cudaSuccess || ep.n1 == 0) return ce;
   if (ep.d_class_work) {
     ce = cudaMemsetAsync(ep.d_class_work, 0, (size_t)ep.n1 * sizeof(unsigned long long), st);
@@ -321,6 +340,30 @@ cudaError_t engine_launch_front(const EnginePlan& ep, cudaStream_t st, bool pair
 cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
   if (ep.n1 == 0) return cudaSuccess;
   cudaError_t ce = cudaSuccess;
+  if (ep.levels) {  // level 2's records and the search in one kernel
+    LevLaunch l = ep.lev;
+    l.stride = ep.stride;
+    l.n1 = ep.n1;
+    l.minsup = ep.minsup;
+    l.row_supp = ep.d_rsupp;
+    l.C2 = ep.d_C2;
+    l.out_off = ep.d_off;
+    l.out_items = ep.d_items;
+    l.out_supp = ep.d_supp;
+    l.cap_sets = ep.count_only ? 0ull : ep.cap_sets;
+    l.cap_items = ep.count_only ? 0ull : ep.cap_items;
+    l.ctrl = ep.d_ctrl;
+    l.class_sets = ep.d_class_sets;
+    l.class_work = ep.d_class_work;
+    l.max_sets = ep.max_sets;
+    l.cta_time = ep.d_cta_time;
+    if (ep.d_class_sets) ce = cudaMemsetAsync(ep.d_class_sets, 0, (size_t)ep.n1 * sizeof(unsigned long long), st);
+    if (ce != cudaSuccess) return ce;
+    if (ep.ev[2]) cudaEventRecord(ep.ev[2], st);
+    ce = launch_levels(l, ep.lev_grid, st);
+    if (ep.ev[3]) cudaEventRecord(ep.ev[3], st);
+    return ce;
+  }
   LevelLaunch ll{ep.d_C2, ep.n1, ep.minsup, ep.d_frows, ep.d_rsupp, ep.d_rank_item, ep.d_order, ep.d_scnt,
                  ep.d_soff, ep.d_eoff, ep.d_sitems, ep.d_entries, ep.d_off, ep.d_items, ep.d_supp,
                  ep.count_only ? 0ull : ep.cap_sets, ep.count_only ? 0ull : ep.cap_items, ep.d_ctrl,
@@ -470,7 +513,7 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
   if ((h.err & DEV_ERR_ABORTED) || (ep->max_sets && h.sets_total > ep->max_sets))
     return fail(FIM_ERR_OUTPUT_OVERFLOW, "more frequent itemsets than the limit: mining stopped early (counts are lower bounds)");
   if (h.err & DEV_ERR_SUB) {  // no room in the small-subtree walk's queues: repeat without it
-    ep->sub = false;
+    ep->sub = ep->levels = false;
     *retry = true;
     return FIM_OK;
   }
@@ -544,7 +587,7 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
       cudaEventElapsedTime(&stats->ms_dfs_kernel, ep->ev[2], ep->ev[3]);  // the last DFS run
       stats->ms_device_total = ep->ms_total;  // every launch, repeated runs included
     }
-    const uint32_t tgrid = ep->proj ? ep->proj_grid : ep->grid;  // CTAs whose times were recorded
+    const uint32_t tgrid = ep->levels ? ep->lev_grid : ep->proj ? ep->proj_grid : ep->grid;  // CTAs whose times were recorded
     if (ep->d_cta_time && tgrid) {  // load balance of the persistent DFS: busy time per CTA
       std::vector<unsigned long long> t(2ull * tgrid);
       FIM_CUDA(cudaMemcpyAsync(t.data(), ep->d_cta_time, t.size() * 8, cudaMemcpyDeviceToHost, st));

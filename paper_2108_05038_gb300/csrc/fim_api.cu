@@ -923,7 +923,7 @@ fim_status est_resolve(fim_db* db) {
   for (uint32_t r = 0; r < R; ++r) db->est_cost[r] = total ? (double)tally[r] / (double)total : 0.0;
   db->est_nfs = h.sets_total;
   const bool over = (h.err & DEV_ERR_ABORTED) || (db->est_limit && h.sets_total > db->est_limit);
-  db->est_redo = over || (h.err & (DEV_ERR_TIMEOUT | DEV_ERR_PSTACK | DEV_ERR_DEPTH)) != 0;
+  db->est_redo = over || (h.err & (DEV_ERR_TIMEOUT | DEV_ERR_PSTACK | DEV_ERR_DEPTH | DEV_ERR_SUB)) != 0;
   // past the itemset limit: the synchronous path continues the doubling from twice this minsup (and until
   // then the first output capacity is bounded by the limit, as after a doubling)
   db->est_redo_minsup = over ? (db->est_minsup > UINT32_MAX / 2 ? UINT32_MAX : 2 * db->est_minsup) : 0u;

@@ -135,6 +135,7 @@ enum WsSlot {
   WS_SUB_TILES,  // tiles of pairs of its later rounds
   WS_SUB_LISTS,  // row lists of its later rounds
   WS_SUB_STATE,
+  WS_LEVELS,     // arenas of the search by levels
   WS_FILT_TABLE, // closed / maximal output: hash table and flags
   WS_FILT_OFF,   // the kept itemsets: offsets
   WS_FILT_ITEMS, // items
@@ -386,6 +387,41 @@ struct SubState {
 constexpr uint32_t kGramRows = 8;             // rows per side of a tile
 constexpr uint32_t kGramWords = 512;          // words per tile
 
+// The search of a mine of few rows, a level at a time (levels.cu).  Sizes of its arenas, for each of two levels:
+constexpr uint32_t kLevMax = 64;                 // levels
+constexpr uint32_t kLevNodes = 1u << 18, kLevUnits = 1u << 18;
+constexpr uint64_t kLevListWords = 1ull << 20, kLevSupWords = 1ull << 21;
+struct LevCount {
+  uint32_t list, sup, nodes, units, pad[4];
+};
+struct LevState {
+  uint32_t arrived, pad[7];
+  LevCount level[kLevMax + 1];
+};
+// A unit: candidates block * 8 .. of node m of the frame whose plen prefix rows and n survivors are in list and whose
+// n (n - 1) / 2 supports are in sup, over words segment seg; node: the count of the node's units left
+struct alignas(32) LevUnit {
+  uint32_t list, plen, n, sup;
+  uint32_t m, block, seg, node;
+};
+struct LevLaunch {
+  const uint4* rows4;  // the frequent rows (consecutive)
+  uint32_t stride, n1, minsup;
+  const uint32_t *ids, *row_supp, *C2;
+  LevState* state;
+  LevUnit* units;
+  uint32_t *lists, *sups, *nodes;
+  uint64_t* out_off;
+  uint32_t *out_items, *out_supp;
+  uint64_t cap_sets, cap_items;
+  DevCtrl* ctrl;
+  unsigned long long *class_sets, *class_work;
+  uint64_t max_sets;
+  unsigned long long* cta_time;
+};
+cudaError_t levels_ctas(int num_sms, uint32_t* out);
+cudaError_t launch_levels(const LevLaunch& p, uint32_t ctas, cudaStream_t st);
+
 struct EnginePlan {
   uint32_t n1 = 0, minsup = 1, stride = 0, bytes_per_row_alg = 0;
   const uint32_t* bits = nullptr;
@@ -433,6 +469,9 @@ struct EnginePlan {
   uint4* d_dq = nullptr;
   uint32_t dq_cap = 0;
   bool sub = false;  // small subtrees walked by proj_sub.cu
+  bool levels = false;  // the search a level at a time (levels.cu)
+  uint32_t lev_grid = 0;
+  LevLaunch lev{};
   uint32_t *d_G = nullptr, *d_goff = nullptr, *d_tileoff = nullptr;
   uint2* d_entries_g = nullptr;
   SubItem* d_sub_items = nullptr;

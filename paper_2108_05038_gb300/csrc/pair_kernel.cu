@@ -198,7 +198,9 @@ cudaError_t launch_pair_counts(const PairLaunch& p, int num_sms, cudaStream_t st
     ksplit = 1;
     for (uint32_t ks = 1; ks <= std::min<uint32_t>(64, nchunks); ++ks) {
       const uint32_t c = (nchunks + ks - 1) / ks;
-      if (c < 4 && ks > 1) break;  // at least 4 chunks (128 words) per item to repay its prologue and epilogue
+      // at least 4 chunks (128 words) per item to repay its prologue and epilogue, except where all items run at
+      // once and only the longest counts (dense_deep, 49 chunks of one tile: 17 us with 13 items, 7 with 49)
+      if (c < 4 && ks > 1 && (uint64_t)tiles * ((nchunks + c - 1) / c) > slots) break;
       const uint32_t k2 = (nchunks + c - 1) / c;
       const uint64_t items = (uint64_t)tiles * k2;
       const uint64_t rounds = (items + slots - 1) / slots;

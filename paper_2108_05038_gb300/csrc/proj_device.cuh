@@ -71,5 +71,48 @@ __device__ __forceinline__ RegionView region_view(const uint32_t* R) {
   return v;
 }
 
+constexpr unsigned long long kBarrierIdleNs = 2000000000ull;
+
+// All CTAs of a cooperative grid meet (epoch: barriers passed so far); false when the wait ran out: no CTA arrived and
+// *progress did not change for 2 s, or another CTA gave up.
+__device__ inline bool grid_barrier(uint32_t* arrived, const uint32_t* progress, uint32_t* err, uint32_t& epoch) {
+  __shared__ uint32_t s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(arrived, 1u);
+    const uint32_t want = (epoch + 1) * gridDim.x;
+    uint32_t ok = 1, seen = kFull, taken = kFull;
+    unsigned long long t0 = 0;
+    for (uint32_t poll = 0;; ++poll) {
+      const uint32_t a = ld_volatile(arrived);
+      if (a >= want) break;
+      if (poll < 32) continue;  // (a microsecond or two: levels are short)
+      __nanosleep(40);
+      if (poll & 15u) continue;
+      if (ld_volatile(err) & DEV_ERR_TIMEOUT) {
+        ok = 0;
+        break;
+      }
+      const uint32_t h = ld_volatile(progress);
+      const unsigned long long now = global_ns();
+      if (a != seen || h != taken) {
+        seen = a;
+        taken = h;
+        t0 = now;
+      } else if (now - t0 > kBarrierIdleNs) {
+        atomicOr(err, DEV_ERR_TIMEOUT);
+        ok = 0;
+        break;
+      }
+    }
+    __threadfence();
+    s_ok = ok;
+  }
+  __syncthreads();
+  ++epoch;
+  return s_ok != 0;
+}
+
 }  // namespace
 }  // namespace fim

@@ -46,7 +46,6 @@ constexpr uint32_t kSubRows = 32;        // rows of a part held in shared memory
 constexpr long long kSubCycles = 400000;  // cycles (about 0.2 ms) after which a subtree's rest goes to the next round
 constexpr uint32_t kUnitWords = 512;      // words of a region that a unit of a part's rows covers
 constexpr uint32_t kSubAll = 5;          // at most so many survivors: every subset of them counted in one pass
-constexpr unsigned long long kBarrierIdleNs = 2000000000ull;
 
 // words of k_sub's shared memory per warp ahead of the pool
 struct SubSmem {
@@ -150,44 +149,6 @@ __device__ __forceinline__ void leave_to_dfs(const SubLaunch& p, uint64_t roff, 
   }
   atomicAdd(&p.ctrl->proj_pending, 1u);
   p.dq[slot] = make_uint4((uint32_t)roff, (uint32_t)(roff >> 32), m, 1u);
-}
-
-// All CTAs of the (cooperative) grid meet; false when the wait ran out.
-__device__ bool grid_barrier(const SubLaunch& p, uint32_t& epoch) {
-  __shared__ uint32_t s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&p.state->arrived, 1u);
-    const uint32_t want = (epoch + 1) * gridDim.x;
-    uint32_t ok = 1, seen = kFull, taken = kFull;
-    unsigned long long t0 = global_ns();
-    for (;;) {
-      const uint32_t a = ld_volatile(&p.state->arrived);
-      if (a >= want) break;
-      if (ld_volatile(&p.ctrl->err) & DEV_ERR_TIMEOUT) {
-        ok = 0;
-        break;
-      }
-      const uint32_t h = ld_volatile(&p.state->progress);
-      const unsigned long long now = global_ns();
-      if (a != seen || h != taken) {
-        seen = a;
-        taken = h;
-        t0 = now;
-      } else if (now - t0 > kBarrierIdleNs) {
-        atomicOr(&p.ctrl->err, DEV_ERR_TIMEOUT);
-        ok = 0;
-        break;
-      }
-      __nanosleep(100);
-    }
-    __threadfence();
-    s_ok = ok;
-  }
-  __syncthreads();
-  ++epoch;
-  return s_ok != 0;
 }
 
 constexpr uint32_t kSubStop = DEV_ERR_ABORTED | DEV_ERR_PSTACK | DEV_ERR_TIMEOUT | DEV_ERR_SUB;
@@ -393,7 +354,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
                   p.Y + ((uint64_t)d2.y << 32 | d2.x), d2.z, d2.w >> 16, cnt);
       if (lane == 0) atomicAdd(&p.state->progress, 1u);
     }
-    if (n_units && !grid_barrier(p, epoch)) break;
+    if (n_units && !grid_barrier(&p.state->arrived, &p.state->progress, &p.ctrl->err, epoch)) break;
     for (uint32_t t = gwarp; t < n_tiles; t += nwarps) {
       if (round == 0) {
         uint32_t lo = 0, hi = p.n1;  // the class: the last queue position q with tileoff[q] <= t
@@ -419,7 +380,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
       }
       if (lane == 0) atomicAdd(&p.state->progress, 1u);
     }
-    if (n_tiles && !grid_barrier(p, epoch)) break;
+    if (n_tiles && !grid_barrier(&p.state->arrived, &p.state->progress, &p.ctrl->err, epoch)) break;
     // (the other halves of G, the lists and the items are free: the round before is over.  This round's are the next
     // one's other halves: empty again)
     if (blockIdx.x == 0 && threadIdx.x == 0) p.state->g_top[par] = p.state->l_top[par] = 0;
@@ -1111,7 +1072,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
         if (p.class_work && cls_work) atomicAdd(&p.class_work[cls], cls_work);
       }
     }
-    if (!grid_barrier(p, epoch)) break;
+    if (!grid_barrier(&p.state->arrived, &p.state->progress, &p.ctrl->err, epoch)) break;
     if (round + 1 >= kSubRounds) break;
   }
   if (!p.out_off && pend_sets) flush_count();
