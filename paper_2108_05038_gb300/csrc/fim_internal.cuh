@@ -399,7 +399,7 @@ struct LevState {
   LevCount level[kLevMax + 1];
 };
 // A unit: candidates block * 8 .. of node m of the frame whose plen prefix rows and n survivors are in list and whose
-// n (n - 1) / 2 supports are in sup, over words segment seg; node: the count of the node's units left
+// n (n - 1) / 2 supports are in sup, over segment seg of the words; node: the count of the node's units left
 struct alignas(32) LevUnit {
   uint32_t list, plen, n, sup;
   uint32_t m, block, seg, node;
@@ -418,6 +418,7 @@ struct LevLaunch {
   unsigned long long *class_sets, *class_work;
   uint64_t max_sets;
   unsigned long long* cta_time;
+  uint32_t group;  // warps of a unit
 };
 cudaError_t levels_ctas(int num_sms, uint32_t* out);
 cudaError_t launch_levels(const LevLaunch& p, uint32_t ctas, cudaStream_t st);

@@ -8,9 +8,11 @@
 //
 //   frame   a prefix X with its survivors S (rows s_0 < s_1 < .. with X u {s} frequent), two or more.  Its nodes are
 //           X u {s_m}, m < |S| - 1, with the candidates s_{m+1} .. (Eclat-DFS-Computation, App. B.3.2).
-//   unit    up to 8 candidates of a node over 512 words: a warp ANDs the node's rows word by word (four words per lane
-//           and load) and counts the candidates under them.
-//   finish  the warp that counts a node's last unit reads the node's supports, writes its records behind one
+//   unit    up to 8 candidates of a node over 512 words a warp: one to eight warps of a CTA, by the length of the rows, AND
+//           the node's rows word by word (four words per lane and load), count the candidates under them and add their
+//           counts in shared memory.  (Added in global memory, a node of four warps paid four more L2 round trips a level:
+//           a replayed mine of dense_deep's database took 146 us against 131.)
+//   finish  the warp that has a node's last supports writes its records behind one
 //           reservation, and makes the child's frame and units for the next level; or, with two to five survivors and
 //           short rows, counts all their subsets in one pass, which ends the subtree there.
 //
@@ -18,8 +20,8 @@
 // units of two levels live in fixed arenas; a search that outgrows them is repeated by the frame passes (DEV_ERR_SUB).
 // The nodes, candidates and records are those of the other traversals.
 //
-// Measured (level-2 lists, queue and search, cold): dense_deep 107 -> 82 us, tiny 65 -> 48 us, its 738-row sample 70 -> 45 us.  What
-// bounds a level (about 9 us) is its chain of about six dependent L2 round trips: unit, rows, words, reservation, and the
+// Measured (level-2 lists, queue and search): dense_deep 107 -> 74 us, tiny 65 -> 48 us, its 738-row sample 70 -> 45 us.  What
+// bounds a level (about 8 us) is its chain of about six dependent L2 round trips: unit, rows, words, reservation, and the
 // next launch or barrier.
 #include <algorithm>
 #include <map>
@@ -35,11 +37,15 @@ constexpr uint32_t kLevThreads = 256;
 constexpr uint32_t kLevWarps = kLevThreads / 32;
 constexpr uint32_t kLevCtasPerSm = 2;
 constexpr uint32_t kLevCand = 8;      // candidates of a unit
-constexpr uint32_t kLevSeg4 = 128;    // 16-byte words of a unit (512 words)
+constexpr uint32_t kLevSeg4 = 128;    // 16-byte words of a unit for one warp (512 words; 64 or 256: 10% and 1% slower)
 constexpr uint32_t kLevPath = 62;     // longest prefix (rows)
 constexpr uint32_t kLevSingles = 3;   // levels launched by themselves
 constexpr uint32_t kLevFew = 5;       // at most so many survivors: all their subsets counted at once
-constexpr uint32_t kLevFewWork = 400; // words per lane x subsets up to which that is quicker than the levels it saves
+constexpr uint32_t kLevNone = ~0u;    // (of units: a level left untouched)
+// Longest rows for that with two survivors, with three to five.  One warp goes through the words, so that long rows take
+// longer than the levels they save: with no such limit dense_deep (1,568 words) takes 131 us a replay, with it 121; without
+// the pass for three to five survivors tiny (320 words) takes 270 us a step, with it 248.
+constexpr uint32_t kLevPairWords = 800, kLevFewWords = 400;
 
 __device__ __forceinline__ uint32_t tri_off(uint32_t m, uint32_t n) { return m * n - m * (m + 1) / 2; }  // of (m, m + 1)
 // units of the nodes before node m of a frame of n survivors, for one segment: sum over nodes of ceil(candidates / 8)
@@ -58,12 +64,16 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
                                                                        const bool single) {
   if (p.cta_time && threadIdx.x == 0) p.cta_time[2 * blockIdx.x] = global_ns();
   __shared__ uint32_t s_rows[kLevWarps][64], s_ids[kLevWarps][64], s_few[kLevWarps][4 * kLevFew];
+  __shared__ uint32_t s_part[2][kLevWarps][kLevCand], s_run;
   const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
   uint32_t* const prow = s_rows[threadIdx.x >> 5];  // the node's rows
   uint32_t* const xs = s_ids[threadIdx.x >> 5];     // their ids, ascending
   uint32_t* const few = s_few[threadIdx.x >> 5];    // the first survivors: rows, supports; ids ascending, whose they are
   const uint32_t gwarp = blockIdx.x * kLevWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kLevWarps;
-  const uint32_t stride4 = p.stride / 4, segs = (stride4 + kLevSeg4 - 1) / kLevSeg4;
+  // A unit is taken by a group of `group` warps of one CTA, a power of two: with rows of up to 512 words a warp, so that
+  // the supports of rows of up to 4,096 words are added in shared memory.
+  const uint32_t stride4 = p.stride / 4, group = p.group, sub = (threadIdx.x >> 5) & (group - 1);
+  const uint32_t segs = (stride4 + group * kLevSeg4 - 1) / (group * kLevSeg4);
   unsigned long long st_inter = 0, st_nodes = 0, st_frames = 0, st_sets = 0, st_items = 0, st_entries = 0;
   uint32_t st_maxlen = 0;
   constexpr uint32_t kStop = DEV_ERR_ABORTED | DEV_ERR_TIMEOUT | DEV_ERR_SUB;
@@ -83,16 +93,18 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
   // The whole subtree of a node with N survivors (few), counted in one pass over the words: lane M stands for the
   // subset M of the survivors, its record and its share of the nodes and intersections of the walk (frame M has the
   // survivors e > max(M) with M u {e} frequent).  One reservation for all records.
-  auto few_survivors = [&](auto tag, uint32_t plen, uint32_t own) {
-    constexpr uint32_t N = decltype(tag)::value;
+  auto few_survivors = [&](auto tag, uint32_t n, uint32_t plen, uint32_t own) {
+    constexpr uint32_t N = decltype(tag)::value;  // (n <= N: the rows past n hold nothing)
     uint32_t cnt[1u << N];
 #pragma unroll
     for (uint32_t m = 0; m < 1u << N; ++m) cnt[m] = 0;
+#pragma unroll 1
     for (uint32_t v = lane; v < stride4; v += 32) {
       uint4 a = __ldg(p.rows4 + (uint64_t)prow[0] * stride4 + v);
       uint4 y[N];
 #pragma unroll
-      for (uint32_t j = 0; j < N; ++j) y[j] = __ldg(p.rows4 + (uint64_t)few[j] * stride4 + v);
+      for (uint32_t j = 0; j < N; ++j)
+        y[j] = j < n ? __ldg(p.rows4 + (uint64_t)few[j] * stride4 + v) : make_uint4(0u, 0u, 0u, 0u);
       for (uint32_t q = 1; q < plen; ++q) {
         const uint4 x = __ldg(p.rows4 + (uint64_t)prow[q] * stride4 + v);
         a = make_uint4(a.x & x.x, a.y & x.y, a.z & x.z, a.w & x.w);
@@ -110,14 +122,14 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
       }
     }
     const uint32_t size = __popc(lane), top = lane ? 32 - __clz(lane) : 0;  // elements above max(M): bits top ..
-    uint32_t c = size == 1 && top <= N ? few[kLevFew + top - 1] : lane == 0 ? own : 0u;
+    uint32_t c = size == 1 && top <= n ? few[kLevFew + top - 1] : lane == 0 ? own : 0u;
 #pragma unroll
     for (uint32_t m = 3; m < 1u << N; ++m) {
       if (!(m & (m - 1))) continue;
       const uint32_t t = __reduce_add_sync(kFull, cnt[m]);
       if (lane == m) c = t;
     }
-    const uint32_t F = __ballot_sync(kFull, lane == 0 || (size == 1 && top <= N) || (size >= 2 && c >= p.minsup));
+    const uint32_t F = __ballot_sync(kFull, lane == 0 || (size == 1 && top <= n) || (size >= 2 && c >= p.minsup));
     const bool mine_f = (F >> lane) & 1u;
     uint32_t ns = 0;  // survivors of frame M
 #pragma unroll
@@ -149,14 +161,14 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
     st_sets += sets;
     st_items += items;
     st_maxlen = max(st_maxlen, __reduce_max_sync(kFull, len));
-    if (own) st_entries += N - 1;
+    if (own) st_entries += n - 1;
     if (!p.out_off) return;
     // the survivors by ascending id: their ids, and which survivor each is
-    const uint32_t id = lane < N ? __ldg(p.ids + few[lane]) : 0u;
+    const uint32_t id = lane < n ? __ldg(p.ids + few[lane]) : kFull;
     uint32_t r = 0;
 #pragma unroll
     for (uint32_t j = 0; j < N; ++j) r += __shfl_sync(kFull, id, j) < id;
-    if (lane < N) {
+    if (lane < n) {
       few[2 * kLevFew + r] = id;
       few[3 * kLevFew + r] = lane;
     }
@@ -169,7 +181,7 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
         uint32_t q = 0;
 #pragma unroll
         for (uint32_t j = 0; j < N; ++j)
-          if ((lane >> few[3 * kLevFew + j]) & 1u) {
+          if (j < n && (lane >> few[3 * kLevFew + j]) & 1u) {
             const uint32_t v = few[2 * kLevFew + j];
             for (; q < plen && xs[q] < v; ++q) *d++ = xs[q];
             *d++ = v;
@@ -183,11 +195,14 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
     }
   };
 
-  // A node whose rows are prow[0 .. plen) and whose survivors are the f-lanes of `sup(j)` over its nc candidates `row(j)`:
-  // its records (and, for a one-item class, its own: support own), and its frame for level `next`.
-  auto finish = [&](uint32_t plen, uint32_t nc, auto row, auto sup, uint32_t own, uint32_t next) {
+  // A node whose rows are prow[0 .. plen) and whose nc candidates have the supports sups[0 .. nc) (lane l has the l-th already,
+  // s0) and are the rows list[0 .. nc), or row0 .. when list is NULL: its records (and, for a one-item class, its own: support
+  // own), and its frame for level `next`.  (One call: the kernel's code has to stay within the instruction cache.)
+  auto finish = [&](uint32_t plen, uint32_t nc, uint32_t s0, const uint32_t* sups, const uint32_t* rows_of, uint32_t row0,
+                    uint32_t own, uint32_t next) {
+    auto sup = [&](uint32_t j) { return __ldcg(sups + j); };
+    auto row = [&](uint32_t j) { return rows_of ? __ldcg(rows_of + j) : row0 + j; };
     const uint32_t par = next & 1u, cls = prow[0];
-    const uint32_t s0 = lane < nc ? sup(lane) : 0u;  // (most nodes have no more)
     uint32_t n = 0;
     auto count = [&](uint32_t j, uint32_t c) {
       const uint32_t bal = __ballot_sync(kFull, c >= p.minsup), at = n + __popc(bal & lt);
@@ -206,11 +221,12 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
       for (uint32_t u = 0; u < 4; ++u) count(j0 + 32 * u + lane, c[u]);
     }
     __syncwarp();
-    if (n >= 2 && n <= kLevFew && p.stride / 32 << n <= kLevFewWork) {
-      if (n == 2) few_survivors(std::integral_constant<uint32_t, 2>{}, plen, own);
-      else if (n == 3) few_survivors(std::integral_constant<uint32_t, 3>{}, plen, own);
-      else if (n == 4) few_survivors(std::integral_constant<uint32_t, 4>{}, plen, own);
-      else few_survivors(std::integral_constant<uint32_t, 5>{}, plen, own);
+    if (n == 2 && p.stride <= kLevPairWords) {
+      few_survivors(std::integral_constant<uint32_t, 2>{}, n, plen, own);
+      return;
+    }
+    if (n >= 3 && n <= kLevFew && p.stride <= kLevFewWords) {
+      few_survivors(std::integral_constant<uint32_t, kLevFew>{}, n, plen, own);
       return;
     }
     const uint32_t singles = own ? 1u : 0u, sets = n + singles, items = n * (plen + 1) + singles;
@@ -298,88 +314,102 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
     }
   };
 
-  uint32_t epoch = 0;
+  uint32_t epoch = 0, round = 0;
   for (uint32_t level = first;; ++level) {
-    if (level == 0) {
-      // level 2: a warp per row (pair counts left incomplete by a timed-out pair kernel count as none)
-      if (ld_volatile(&p.ctrl->err) & DEV_ERR_TIMEOUT) return;
-      for (uint32_t i = gwarp; i < p.n1; i += nwarps) {
-        const uint32_t own = __ldg(p.row_supp + i);
-        if (own < p.minsup) continue;  // (a sample's row)
-        __syncwarp();
-        if (lane == 0) prow[0] = i;
-        __syncwarp();
-        const uint32_t* c2 = p.C2 + (uint64_t)i * p.n1 + i + 1;
-        finish(1u, p.n1 - i - 1, [&](uint32_t j) { return i + 1 + j; }, [&](uint32_t j) { return __ldg(c2 + j); }, own, 1u);
-      }
-      if (single || !grid_barrier(&p.state->arrived, &p.state->arrived, &p.ctrl->err, epoch)) break;
-      continue;
-    }
     const uint32_t par = level & 1u;
-    const uint32_t n_units = min(ld_volatile(&p.state->level[level].units), kLevUnits);
-    if (n_units == 0) break;
-    // After an error no unit is touched (a frame that found no room leaves its reserved units unwritten, and its error was
-    // set before the barrier); the CTAs go on meeting until a level has none, since the error may be seen at different levels.
-    const uint32_t n_run = (ld_volatile(&p.ctrl->err) & kStop) ? 0u : n_units;
+    if (threadIdx.x == 0) {
+      // After an error no unit is touched (a frame that found no room leaves its reserved units unwritten, and its error was
+      // set before the barrier); the CTAs go on meeting until a level has none, since the error may be seen at different levels.
+      const uint32_t err = ld_volatile(&p.ctrl->err);
+      const uint32_t n = level ? min(ld_volatile(&p.state->level[level].units), kLevUnits) : p.n1;
+      s_run = (level ? err & kStop : err & DEV_ERR_TIMEOUT) && n ? kLevNone : n;  // (a timeout: pair counts left incomplete)
+    }
+    __syncthreads();
+    uint32_t n_run = s_run;  // (one value for the CTA: a group's warps go through the units together)
+    __syncthreads();
+    if (n_run == 0) break;
+    if (n_run == kLevNone) n_run = 0;
     const LevUnit* const units = p.units + (uint64_t)par * kLevUnits;
-    for (uint32_t t = gwarp; t < n_run; t += nwarps) {
-      const uint4 f4 = __ldcg(reinterpret_cast<const uint4*>(units + t));
-      const uint4 u4 = __ldcg(reinterpret_cast<const uint4*>(units + t) + 1);
-      const uint32_t* const list = p.lists + (uint64_t)par * kLevListWords + f4.x;
-      const uint32_t plen = f4.y, n = f4.z, m = u4.x, c0 = u4.y * kLevCand, nc = n - 1 - m;
-      uint32_t* const sup = p.sups + (uint64_t)par * kLevSupWords + f4.w + tri_off(m, n);
+    const uint32_t step = level ? nwarps / group : nwarps;
+    for (uint32_t t = level ? gwarp / group : gwarp; t < n_run; t += step) {
+      uint32_t plen, nc, s0, own = 0, row0 = 0;
+      const uint32_t *sups, *rows_of = nullptr;
       __syncwarp();
-      for (uint32_t q = lane; q <= plen; q += 32) prow[q] = __ldcg(list + (q < plen ? q : plen + m));
-      const uint32_t cnt = min(kLevCand, nc - c0);
-      const uint32_t myrow = lane < cnt ? __ldcg(list + plen + m + 1 + c0 + lane) : 0u;
-      __syncwarp();
-      const uint4* rows4[kLevCand];
+      if (level == 0) {
+        own = __ldg(p.row_supp + t);
+        if (own < p.minsup) continue;  // (a sample's row)
+        if (lane == 0) prow[0] = t;
+        plen = 1;
+        nc = p.n1 - t - 1;
+        row0 = t + 1;
+        sups = p.C2 + (uint64_t)t * p.n1 + t + 1;
+        s0 = lane < nc ? __ldcg(sups + lane) : 0u;
+        __syncwarp();
+      } else {
+        const uint4 f4 = __ldcg(reinterpret_cast<const uint4*>(units + t));
+        const uint4 u4 = __ldcg(reinterpret_cast<const uint4*>(units + t) + 1);
+        const uint32_t* const list = p.lists + (uint64_t)par * kLevListWords + f4.x;
+        const uint32_t n = f4.z, m = u4.x, c0 = u4.y * kLevCand;
+        plen = f4.y + 1;
+        nc = n - 1 - m;
+        rows_of = list + plen + m;
+        uint32_t* const sup = p.sups + (uint64_t)par * kLevSupWords + f4.w + tri_off(m, n);
+        sups = sup;
+        for (uint32_t q = lane; q < plen; q += 32) prow[q] = __ldcg(list + (q + 1 < plen ? q : plen - 1 + m));
+        const uint32_t cnt = min(kLevCand, nc - c0);
+        const uint32_t myrow = lane < cnt ? __ldcg(rows_of + c0 + lane) : 0u;
+        __syncwarp();
+        const uint4* rows4[kLevCand];
 #pragma unroll
-      for (uint32_t g = 0; g < kLevCand; ++g)
-        rows4[g] = p.rows4 + (uint64_t)__shfl_sync(kFull, myrow, min(g, cnt - 1)) * stride4;
-      uint32_t acc[kLevCand];
+        for (uint32_t g = 0; g < kLevCand; ++g)
+          rows4[g] = p.rows4 + (uint64_t)__shfl_sync(kFull, myrow, min(g, cnt - 1)) * stride4;
+        uint32_t acc[kLevCand];
 #pragma unroll
-      for (uint32_t g = 0; g < kLevCand; ++g) acc[g] = 0;
-      const uint32_t v0 = u4.z * kLevSeg4, v1 = min(stride4, v0 + kLevSeg4);
-#pragma unroll 2
-      for (uint32_t v = v0 + lane; v < v1; v += 32) {
-        uint4 a = __ldg(p.rows4 + (uint64_t)prow[0] * stride4 + v);
-        for (uint32_t q = 1; q <= plen; ++q) {
-          const uint4 x = __ldg(p.rows4 + (uint64_t)prow[q] * stride4 + v);
-          a = make_uint4(a.x & x.x, a.y & x.y, a.z & x.z, a.w & x.w);
+        for (uint32_t g = 0; g < kLevCand; ++g) acc[g] = 0;
+        const uint32_t v0 = u4.z * group * kLevSeg4, v1 = min(stride4, v0 + group * kLevSeg4);
+#pragma unroll 1
+        for (uint32_t v = v0 + sub * 32 + lane; v < v1; v += 32 * group) {
+          uint4 a = __ldg(p.rows4 + (uint64_t)prow[0] * stride4 + v);
+          for (uint32_t q = 1; q < plen; ++q) {
+            const uint4 x = __ldg(p.rows4 + (uint64_t)prow[q] * stride4 + v);
+            a = make_uint4(a.x & x.x, a.y & x.y, a.z & x.z, a.w & x.w);
+          }
+#pragma unroll
+          for (uint32_t g = 0; g < kLevCand; ++g) {
+            const uint4 x = __ldg(rows4[g] + v);
+            acc[g] += __popc(a.x & x.x) + __popc(a.y & x.y) + __popc(a.z & x.z) + __popc(a.w & x.w);
+          }
         }
+        s0 = 0;
 #pragma unroll
         for (uint32_t g = 0; g < kLevCand; ++g) {
-          const uint4 x = __ldg(rows4[g] + v);
-          acc[g] += __popc(a.x & x.x) + __popc(a.y & x.y) + __popc(a.z & x.z) + __popc(a.w & x.w);
+          const uint32_t s = __reduce_add_sync(kFull, acc[g]);
+          if (lane == g && g < cnt) s0 = s;
         }
-      }
-      uint32_t mine = 0;
-#pragma unroll
-      for (uint32_t g = 0; g < kLevCand; ++g) {
-        const uint32_t s = __reduce_add_sync(kFull, acc[g]);
-        if (lane == g) mine = s;
-      }
-      if (nc <= kLevCand && segs == 1) {  // the node's only unit: its supports are in the lanes
+        if (group > 1) {  // (two buffers: a third round's supports are written after the second's barrier)
+          uint32_t(*const part)[kLevCand] = s_part[round++ & 1u] + ((threadIdx.x >> 5) & ~(group - 1));
+          if (sub && lane < kLevCand) part[sub][lane] = s0;
+          __syncwarp();
+          asm volatile("bar.sync %0, %1;" ::"r"(1 + (threadIdx.x >> 5) / group), "r"(group * 32) : "memory");
+          if (sub) continue;
+          if (lane < cnt)
+            for (uint32_t g = 1; g < group; ++g) s0 += part[g][lane];
+        }
+        if (nc > kLevCand || segs > 1) {  // (else: the node's only unit, its supports in the lanes)
+          if (s0) atomicAdd(sup + c0 + lane, s0);
+          __threadfence();
+          __syncwarp();
+          uint32_t left = 0;
+          if (lane == 0) left = atomicSub(p.nodes + (uint64_t)par * kLevNodes + u4.w, 1u);
+          if (__shfl_sync(kFull, left, 0) != 1u) continue;
+          __threadfence();  // the node's last unit
+          s0 = lane < nc ? __ldcg(sup + lane) : 0u;
+        }
         st_inter += nc;
         ++st_nodes;
         if (lane == 0 && p.class_work) atomicAdd(&p.class_work[prow[0]], (unsigned long long)nc);
-        finish(plen + 1, nc, [&](uint32_t) { return myrow; }, [&](uint32_t) { return mine; }, 0u, level + 1);
-        continue;
       }
-      if (lane < cnt && mine) atomicAdd(sup + c0 + lane, mine);
-      __threadfence();
-      __syncwarp();
-      uint32_t done = 0;
-      if (lane == 0) done = atomicSub(p.nodes + (uint64_t)par * kLevNodes + u4.w, 1u);
-      if (__shfl_sync(kFull, done, 0) != 1u) continue;
-      __threadfence();
-      // the node's last unit
-      st_inter += nc;
-      ++st_nodes;
-      if (lane == 0 && p.class_work) atomicAdd(&p.class_work[prow[0]], (unsigned long long)nc);
-      finish(plen + 1, nc, [&](uint32_t j) { return __ldcg(list + plen + m + 1 + j); },
-             [&](uint32_t j) { return __ldcg(sup + j); }, 0u, level + 1);
+      finish(plen, nc, s0, sups, rows_of, row0, own, level + 1);
     }
     if (single || !grid_barrier(&p.state->arrived, &p.state->arrived, &p.ctrl->err, epoch)) break;
   }
@@ -422,10 +452,11 @@ cudaError_t levels_ctas(int num_sms, uint32_t* out) {
 
 cudaError_t launch_levels(const LevLaunch& p, uint32_t ctas, cudaStream_t st) {
   // The first levels, which nearly every search has, as launches of their own, the others until one is empty.  A captured
-  // mine is the quicker for it (dense_deep: 132 us a replay, 134 with all levels in the cooperative launch), an eager one 3%
+  // mine is the quicker for it (dense_deep: 121 us a replay, 122 with all levels in the cooperative launch), an eager one 3%
   // slower (a step of dense_deep's database 325 us against 316); more such launches lose in both.
   LevLaunch q = p;
   q.cta_time = nullptr;
+  for (q.group = 1; q.group < kLevWarps && q.group * kLevSeg4 * 4 < p.stride; q.group *= 2) {}
   for (uint32_t level = 0; level < kLevSingles; ++level) {
     k_levels<<<ctas, kLevThreads, 0, st>>>(q, level, true);
     note_launch();

@@ -57,6 +57,21 @@ def test_same_search_as_frame_passes(name):
         db.free()
 
 
+@pytest.mark.parametrize("words", [384, 416, 512, 544, 800, 832, 1_024, 1_056, 2_048, 2_080, 4_096, 4_128])
+def test_row_lengths(words):
+    """Rows at the edges of one, two, four and eight warps a unit and one or two segments, and of the one-pass subtrees."""
+    off, items, N = groups(words, words * 32, [12, 4], 0.55, 0.2)
+    minsup = words * 32 // 25
+    db = fim.build_vertical_db(off, items, N)
+    try:
+        got = db.mine(minsup)
+        ref = db.mine(minsup, dfs_mode=fim.FIM_DFS_FRAMES)
+        assert got.as_dict() == ref.as_dict() == odict(oracle.eclat(off, items, N, minsup))
+        assert got.stats["n_intersections"] == ref.stats["n_intersections"] and got.stats["max_len"] >= 4
+    finally:
+        db.free()
+
+
 @pytest.mark.parametrize("cost", ["itemsets", "intersections"])
 @pytest.mark.parametrize("name", ["few_survivors", "many_survivors"])
 def test_class_costs_of_a_sample(name, cost):
