@@ -372,7 +372,8 @@ void fim_plan_free(fim_plan* plan);
  * ctas_per_sm caps each job's persistent CTAs per SM (0 = 1) so that
  * concurrent jobs share the SMs; max_itemsets (0 = none) stops a job whose
  * output grows past it (FIM_ERR_OUTPUT_OVERFLOW from fim_server_wait).  fim_server_submit copies the host CSR
- * database (as fim_build_vertical_db) and queues the job; jobs are admitted
+ * database (as fim_build_vertical_db) and queues the job: to the device while the budget has room for the job
+ * (its footprint is then in use from the submission on), else to host memory; jobs are admitted
  * in arrival order when a slot is free and their footprint fits the budget
  * left (a job larger than the budget runs alone), then run build (prefilter =
  * minsup), the sample estimate when sample_rate > 0, and the mine; the
@@ -396,7 +397,8 @@ fim_status fim_server_wait(fim_server* srv, uint64_t job_id, fim_result** out, d
                            double* service_s);
 /* As fim_server_wait, and the job's device interval: milliseconds from the
  * server's creation to CUDA events recorded on the job's stream just before its
- * first and just after its last device work (-1 when they could not be read).
+ * first and just after its last device work, without the copy of its database
+ * at the submission (-1 when they could not be read).
  * Jobs whose intervals intersect had device work in flight at the same time. */
 fim_status fim_server_wait_ex(fim_server* srv, uint64_t job_id, fim_result** out, double* latency_s,
                               double* service_s, double* device_start_ms, double* device_end_ms);

@@ -412,6 +412,25 @@ static fim_status build_common(const uint32_t* off, const uint32_t* items, uint3
   return FIM_OK;
 }
 
+fim_status build_uploaded_db(uint32_t* d_off, uint32_t* d_items, uint64_t nnz, uint32_t D, uint32_t N, uint32_t word_bits,
+                             uint32_t prefilter, cudaStream_t st, fim_db** out) {
+  fim_db* db = new (std::nothrow) fim_db();
+  if (!db) return fail(FIM_ERR_OOM, "host allocation");
+  fim_status s = db_init(db, D, N, word_bits, prefilter, st);
+  if (s == FIM_OK) {
+    db->nnz = nnz;
+    db->d_tx_off = d_off;
+    db->d_tx_items = d_items;
+    s = db_build_rows(db, d_off, d_items, false);
+  }
+  if (s != FIM_OK) {
+    fim_db_free(db);
+    return s;
+  }
+  *out = db;
+  return FIM_OK;
+}
+
 static void rows_for_minsup(const fim_db* db, uint32_t minsup, EngineInput* in) {
   // rows are sorted by ascending support: the frequent ones are a suffix
   uint32_t r0 = (uint32_t)(std::lower_bound(db->supp.begin(), db->supp.end(), minsup) - db->supp.begin());

@@ -515,6 +515,9 @@ fim_status mine_input(fim_db* db, uint32_t minsup, const fim_mine_opts* opts, En
 // the first output capacity that the database's estimate suggests for a minsup (0: none)
 uint64_t estimate_capacity(const fim_db* db, uint32_t minsup);
 // fim_estimate_class_costs_ex, allowed to leave its result on the device (see fim_api.cu)
+// A database from a valid host CSR that is on the device already (complete; kept until the database is freed).
+fim_status build_uploaded_db(uint32_t* d_off, uint32_t* d_items, uint64_t nnz, uint32_t D, uint32_t N, uint32_t word_bits,
+                             uint32_t prefilter, cudaStream_t st, fim_db** out);
 fim_status estimate_impl(fim_db* db, double sample_rate, double rel_minsup, uint64_t seed, uint32_t cost_kind,
                          uint64_t max_sample_itemsets, double* cost_out, uint32_t* order_out, bool allow_defer,
                          uint32_t first_minsup_s);
