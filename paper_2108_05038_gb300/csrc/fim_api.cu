@@ -946,7 +946,8 @@ fim_status est_resolve(fim_db* db) {
   // past the itemset limit: the synchronous path continues the doubling from twice this minsup (and until
   // then the first output capacity is bounded by the limit, as after a doubling)
   db->est_redo_minsup = over ? (db->est_minsup > UINT32_MAX / 2 ? UINT32_MAX : 2 * db->est_minsup) : 0u;
-  db->est_doubled = over;
+  // (so does a search that outgrew its arenas: its count is of the part that was searched)
+  db->est_doubled = over || (h.err & DEV_ERR_SUB);
   return FIM_OK;
 }
 

@@ -114,3 +114,20 @@ def test_search_past_the_arenas_and_limits():
             db.mine(D, max_itemsets=510)
     finally:
         db.free()
+
+
+def test_deferred_estimate_past_the_arenas():
+    """A deferred sample of 2^20 - 1 itemsets outgrows the arenas: the mine that uses it finds room for its result at once,
+    and the estimate is completed when it is read (k items alike: class i has 2^(k - 1 - i) itemsets)."""
+    k, D = 20, 64
+    db = fim.build_vertical_db((np.arange(D + 1) * k).astype(np.uint32), np.tile(np.arange(k, dtype=np.uint32), D), k)
+    try:
+        db.estimate_class_costs(1.0, 1.0, 3, outputs=False)
+        r = db.mine(D, result_on_device=True)
+        assert r.n_sets == 2 ** k - 1
+        r.free()
+        cost, order = db.estimate_result()[:2]
+        assert np.array_equal(order, np.arange(k))
+        assert np.allclose(cost, 2.0 ** np.arange(k - 1, -1, -1) / (2 ** k - 1), rtol=1e-12)
+    finally:
+        db.free()
