@@ -241,7 +241,7 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     ep->d_tileoff = ep->d_goff + n1;
     // Small subtrees in shared memory first, unless the caller tunes the general walk (its hand-out threshold, its
     // stacks, diffset frames), or its shared queue, which takes what they leave, is off.
-    ep->sub = share && !cfg.split_words && !cfg.pstack_words && !cfg.diffsets;
+    ep->sub = share && !db->served && !cfg.split_words && !cfg.pstack_words && !cfg.diffsets;
     if (ep->sub) {
       FIM_TRY(ws_get(ws, WS_ENTRIES_G, ep->npairs_max + 1, &ep->d_entries_g));
       FIM_TRY(ws_get(ws, WS_SUB_G, kSubGramCap, &ep->d_G));
@@ -261,7 +261,7 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     FIM_TRY(ws_get(ws, WS_PROJ_T, std::max<uint64_t>(4, ep->proj_t_cap), &ep->d_T));
   }
   // Automatic, few rows (where frame passes were chosen): by levels
-  ep->levels = cfg.mode == 2 && ep->mode == 1 && !cfg.donate && cfg.ctas_per_sm == 0 && !cfg.diffsets && !ep->leaves &&
+  ep->levels = !db->served && cfg.mode == 2 && ep->mode == 1 && !cfg.donate && cfg.ctas_per_sm == 0 && !cfg.diffsets && !ep->leaves &&
                n1 >= 3 && n1 < 1024 && ep->rows_base;
   if (ep->levels) {
     uint8_t* a = nullptr;

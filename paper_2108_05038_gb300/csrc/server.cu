@@ -108,6 +108,7 @@ void run_job(fim_server* srv, Job* j, cudaStream_t st) {
   } else {
     s = fim_build_vertical_db(j->off.data(), j->items.data(), j->D, j->N, 64, j->minsup, st, &db);
   }
+  if (s == FIM_OK) db->served = true;
   if (s == FIM_OK && j->sample_rate > 0.0) {
     s = fim_estimate_class_costs(db, j->sample_rate, (double)j->minsup / (double)j->D, 1000 + j->id, nullptr,
                                  nullptr);
