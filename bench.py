@@ -295,6 +295,10 @@ def run_ours(args):
         alu_peak_gword = 128.0 / 3.0 * num_sms * sm_max_mhz * 1e6 / 1e9
         words = stats["n_pair_intersections"] * ((D + 31) // 32)  # algorithmic 32-bit word pairs
         achieved_gword = words / (pair_avg * 1e-3) / 1e9
+        # (more word pairs or flops than the row kernels can do: counted from the transactions)
+        by_tx = (achieved_gword > alu_peak_gword if stats.get("pair_kernel", 1) == 1 else
+                 stats["pair_kernel"] == 4 and 2.0 * stats["n_pair_intersections"] * D / (pair_avg * 1e-3) / 1e12
+                 > 2.0 * float(peaks.get("bf16_tflops", 1900.0)))
         rec, rec_note = captured(args.workload)
         hbm = float(peaks.get("hbm_gbs", 6800.0))
         hbm_src = "measured copy rate (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks else "fallback 6.8 TB/s"
@@ -302,8 +306,8 @@ def run_ours(args):
             proj = stats.get("bytes_projected", 0) > 0
             alg = stats["bytes_projected"] if proj else stats["bytes_dfs_kernel"]
             dfs_gbs = alg / (dfs_avg * 1e-3) / 1e9
-            roofline = {"kernel": ("k_proj_tids + k_proj_bits + k_dfs_proj (+ k_dfs_sparse on the classes left out)"
-                                   if proj else "k_dfs"),
+            roofline = {"kernel": ("k_proj_tids + k_proj_bits + k_sub + k_dfs_proj (+ k_dfs_sparse on the classes left out)"
+                                   if proj else "k_levels (fewer than 1,024 rows) or the DFS kernel"),
                         "bound": "hbm", "achieved": round(dfs_gbs, 1), "peak": round(hbm, 1),
                         "unit": "GB/s", "frac": round(dfs_gbs / hbm, 4),
                         "traffic": rec["kernels"]["dfs"] if rec else None, "traffic_source": rec_note,
@@ -315,6 +319,14 @@ def run_ours(args):
                                  if proj else
                                  "algorithmic bytes count every candidate row in full (the dense definition); the "
                                  "kernel reads row words only under nonzero prefix words")}
+        elif by_tx:  # level 2 counted from the transactions: one addition in L2 per pair of a transaction's items
+            lens = np.diff(w["offsets"].astype(np.int64))
+            adds = float((lens * (lens - 1) // 2).sum()) / (pair_avg * 1e-3) / 1e9
+            roofline = {"kernel": "k_pair_tx" + (" + k_pair_mma_fused" if stats["pair_kernel"] == 4 else ""),
+                        "bound": "l2 atomics", "achieved": round(adds, 1), "peak": 180.0, "unit": "Gadd/s",
+                        "frac": round(adds / 180.0, 4), "traffic": None, "traffic_source": rec_note,
+                        "peak_source": "scattered 32-bit additions in L2, measured on a GB300",
+                        "note": "pairs of each transaction's items, an upper bound of the additions made"}
         elif stats.get("pair_kernel") in (2, 3, 4):  # level 2 on the tensor cores: the 0/1 contraction, kind::f8f6f4
             flops = 2.0 * stats["n_pair_intersections"] * D  # one multiply-add per pair and transaction
             tf = flops / (pair_avg * 1e-3) / 1e12

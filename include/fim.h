@@ -76,7 +76,8 @@ typedef struct {
   float dfs_cta_busy_max_ms;     /* longest time a persistent DFS CTA was resident (collect_times)  */
   float dfs_cta_busy_mean_ms;    /* mean over the CTAs; max / mean is the load imbalance           */
   uint32_t pair_kernel;          /* level-2 kernel that ran: FIM_PAIR_CORES / _TENSOR / _TENSOR_E4M3 /
-                                    _TENSOR_FUSED                                                      */
+                                    _TENSOR_FUSED; counted from the transactions alone: FIM_PAIR_CORES,
+                                    with the most frequent rows on the tensor cores: _TENSOR_FUSED     */
   uint32_t n_proj_classes;       /* FIM_DFS_PROJECTED: one-item classes given their database part   */
   uint64_t n_proj_splits;        /* frames handed to other warps with their own database part       */
   uint64_t n_fallback_entries;   /* two-item classes mined by the sparse node mode instead           */
@@ -104,9 +105,11 @@ enum { FIM_OUTPUT_ALL = 0, FIM_OUTPUT_CLOSED = 1, FIM_OUTPUT_MAXIMAL = 2 };
  * shared memory by TMA, spread to e4m3 there), no scratch and no widened copy in device memory;
  * needs the frequent rows to be consecutive rows of the bitmap, which they are in every fim_mine
  * (FIM_ERR_INVALID otherwise);
- * FIM_PAIR_AUTO: integer pipes or a tensor-core kernel, whichever has the smaller modelled time:
- * FIM_PAIR_TENSOR_FUSED for consecutive rows, else FIM_PAIR_TENSOR while its scratch is at most 1/16
- * of device memory. */
+ * FIM_PAIR_AUTO: whichever has the smallest modelled time of the integer pipes, a tensor-core kernel
+ * (FIM_PAIR_TENSOR_FUSED for consecutive rows, else FIM_PAIR_TENSOR while its scratch is at most 1/16
+ * of device memory), and one addition per pair of items of a transaction from the database's
+ * transactions, which are sparse (alone, or for all pairs but those of the 256 most frequent rows, which
+ * FIM_PAIR_TENSOR_FUSED counts); not with transactions that repeat an item. */
 enum { FIM_PAIR_AUTO = 0, FIM_PAIR_CORES = 1, FIM_PAIR_TENSOR = 2, FIM_PAIR_TENSOR_E4M3 = 3,
        FIM_PAIR_TENSOR_FUSED = 4 };
 
@@ -122,8 +125,10 @@ typedef struct {
                                   SM), dense in its stack slot otherwise; rows of at most 65,535
                                   16-byte words, no donation (else as NODES); FIM_DFS_AUTO (2, the
                                   default): projected with at least 1,024 frequent rows (and no
-                                  cap on the CTAs per SM), else frames for rows of at most 16,384
-                                  words (64 KB), else SPARSE;
+                                  cap on the CTAs per SM), else, for rows of at most 16,384 words
+                                  (64 KB), a level at a time over all extendable itemsets (no cap, no
+                                  donation, no diffsets; a search that outgrows its lists is repeated
+                                  as FRAMES) or frames, else SPARSE;
                                   FIM_DFS_WARP (4): one warp
                                   per two-item class, the
                                   prefix in its registers, no CTA-wide barrier; rows of at most 512
