@@ -63,7 +63,7 @@ typedef struct {
   uint64_t n_classes;            /* class nodes expanded by the persistent DFS kernel              */
   uint64_t n_queue_entries;      /* level-3 prefix classes put in the persistent queue             */
   uint64_t n_donations;          /* subclasses handed from a busy CTA to idle CTAs                 */
-  uint64_t bytes_algorithmic;    /* algorithmic bytes of all intersections (see DESIGN measurement) */
+  uint64_t bytes_algorithmic;    /* algorithmic bytes of all intersections                          */
   uint64_t bytes_pair_kernel;    /* algorithmic bytes of the pair kernel                           */
   uint64_t bytes_dfs_kernel;     /* algorithmic bytes of the DFS kernel                            */
   uint32_t words_per_row;        /* 32-bit words per bitmap row, padded (row stride)               */
