@@ -227,9 +227,9 @@ struct fim_db {
   std::vector<uint32_t> rank_item, supp;
   std::vector<int32_t> item_rank;
 
-  // A served job's: no cooperative launches, which start only when all their CTAs fit and so wait for the longest job in
-  // flight (2,000 served requests, four slots: p99 206 ms with them in the samples' mines; without them 137, and 133 for the
-  // first 1,000).
+  // A served job's: without the search by levels and the small-subtree walk, whose arenas (44 and 97 MB) its short-lived
+  // database would need as well (2,000 served requests, four slots: p50 2.7 ms with them in the samples' mines, 1.3 without;
+  // p99 136 and 141).
   bool served = false;
 
   // last estimate (fim_estimate_class_costs)
@@ -383,11 +383,16 @@ struct alignas(32) SubUnit {  // rows j0 .. of a part's own region, over 256 wor
   uint32_t src4, list, path_len_cnt, j0;  // (path_len | rows << 16)
   uint32_t dst_lo, dst_hi, stride, unit;  // words of Y; unit | words << 16
 };
+// One round: the words of G and of the lists that its parts take, its items, tiles and units, how many of each have been
+// claimed, and (on a line of their own: polled) how many are finished
+struct alignas(128) SubRound {
+  unsigned long long g_top, l_top;
+  uint32_t item_n, tile_n, unit_n, item_head, tile_head, unit_head;
+  alignas(64) uint32_t item_done, tile_done, unit_done;
+};
 struct SubState {
-  unsigned long long g_top[2], l_top[2];  // words in use of each half of G and of the lists
-  uint32_t arrived, progress;             // grid barrier: CTAs arrived, items and tiles taken
-  uint32_t item_head[kSubRounds], item_n[kSubRounds + 1], tile_n[kSubRounds + 1],
-      unit_n[kSubRounds + 1];
+  SubRound round[kSubRounds + 1];
+  alignas(128) uint32_t progress;  // raised by items that take long
 };
 constexpr uint32_t kGramRows = 8;             // rows per side of a tile
 constexpr uint32_t kGramWords = 512;          // words per tile
@@ -396,11 +401,10 @@ constexpr uint32_t kGramWords = 512;          // words per tile
 constexpr uint32_t kLevMax = 64;                 // levels
 constexpr uint32_t kLevNodes = 1u << 18, kLevUnits = 1u << 18;
 constexpr uint64_t kLevListWords = 1ull << 20, kLevSupWords = 1ull << 21;
-struct LevCount {
-  uint32_t list, sup, nodes, units, pad[4];
+struct LevCount {  // a level's words and units in use, and how many of its units have been claimed and finished
+  uint32_t list, sup, nodes, units, head, done, pad[2];
 };
 struct LevState {
-  uint32_t arrived, pad[7];
   LevCount level[kLevMax + 1];
 };
 // A unit: candidates block * 8 .. of node m of the frame whose plen prefix rows and n survivors are in list and whose

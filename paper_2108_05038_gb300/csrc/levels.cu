@@ -16,7 +16,8 @@
 //           reservation, and makes the child's frame and units for the next level; or, with two to five survivors and
 //           short rows, counts all their subsets in one pass, which ends the subtree there.
 //
-// The CTAs meet once per level.  Level 2 enters the same way: a warp per row reads its pair counts.  Lists, supports and
+// The groups of warps claim the units of a level one after the other, and a CTA goes on to the next level when all are
+// finished (phase_wait).  Level 2 enters the same way: a warp per row reads its pair counts.  Lists, supports and
 // units of two levels live in fixed arenas; a search that outgrows them is repeated by the frame passes (DEV_ERR_SUB).
 // The nodes, candidates and records are those of the other traversals.
 //
@@ -41,7 +42,6 @@ constexpr uint32_t kLevSeg4 = 128;    // 16-byte words of a unit for one warp (5
 constexpr uint32_t kLevPath = 62;     // longest prefix (rows)
 constexpr uint32_t kLevSingles = 3;   // levels launched by themselves
 constexpr uint32_t kLevFew = 5;       // at most so many survivors: all their subsets counted at once
-constexpr uint32_t kLevNone = ~0u;    // (of units: a level left untouched)
 // Longest rows for that with two survivors, with three to five.  One warp goes through the words, so that long rows take
 // longer than the levels they save: with no such limit dense_deep (1,568 words) takes 131 us a replay, with it 121; without
 // the pass for three to five survivors tiny (320 words) takes 270 us a step, with it 248.
@@ -58,18 +58,19 @@ __device__ __forceinline__ uint32_t units_before(uint32_t m, uint32_t n) {
   return upto(n - 1) - upto(n - 1 - m);
 }
 
-// first: the level to begin with (0: level 2 from the pair counts); single: that level alone, else until one is empty, the
-// CTAs meeting in between (cooperative launch)
+// first: the level to begin with (0: level 2 from the pair counts); single: that level alone, its units dealt out in order,
+// else until one is empty, the units claimed
 __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __grid_constant__ LevLaunch p, const uint32_t first,
                                                                        const bool single) {
   if (p.cta_time && threadIdx.x == 0) p.cta_time[2 * blockIdx.x] = global_ns();
   __shared__ uint32_t s_rows[kLevWarps][64], s_ids[kLevWarps][64], s_few[kLevWarps][4 * kLevFew];
-  __shared__ uint32_t s_part[2][kLevWarps][kLevCand], s_run;
+  __shared__ uint32_t s_part[2][kLevWarps][kLevCand], s_next[2][kLevWarps];
+  __shared__ uint32_t s_run, s_first, s_done;
   const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
   uint32_t* const prow = s_rows[threadIdx.x >> 5];  // the node's rows
   uint32_t* const xs = s_ids[threadIdx.x >> 5];     // their ids, ascending
   uint32_t* const few = s_few[threadIdx.x >> 5];    // the first survivors: rows, supports; ids ascending, whose they are
-  const uint32_t gwarp = blockIdx.x * kLevWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kLevWarps;
+  const uint32_t nwarps = gridDim.x * kLevWarps;
   // A unit is taken by a group of `group` warps of one CTA, a power of two: with rows of up to 512 words a warp, so that
   // the supports of rows of up to 4,096 words are added in shared memory.
   const uint32_t stride4 = p.stride / 4, group = p.group, sub = (threadIdx.x >> 5) & (group - 1);
@@ -314,24 +315,38 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
     }
   };
 
-  uint32_t epoch = 0, round = 0;
+  // A CTA claims the first units of a level, one for each of its groups, before the wait for the level above, and a group's
+  // first warp the next one while a unit is counted: no claim is waited for, and no group gets a second unit before each has
+  // had one.  (A claim per group for the first ones too: 2,432 additions to one word, a step of tiny 250 us against 245.)
+  const uint32_t wib = threadIdx.x >> 5;
+  uint32_t round = 0, claim = 0;  // (claim: thread 0)
+  auto claim_of = [&](uint32_t level) {
+    if (!single) claim = atomicAdd(&p.state->level[level].head, kLevWarps / group);
+  };
+  if (threadIdx.x == 0) {
+    s_done = 0;
+    claim_of(first);
+  }
   for (uint32_t level = first;; ++level) {
     const uint32_t par = level & 1u;
     if (threadIdx.x == 0) {
-      // After an error no unit is touched (a frame that found no room leaves its reserved units unwritten, and its error was
-      // set before the barrier); the CTAs go on meeting until a level has none, since the error may be seen at different levels.
+      // After an error no unit is touched: a frame that found no room leaves its reserved units unwritten, and its error was
+      // set before the level above was finished.
       const uint32_t err = ld_volatile(&p.ctrl->err);
       const uint32_t n = level ? min(ld_volatile(&p.state->level[level].units), kLevUnits) : p.n1;
-      s_run = (level ? err & kStop : err & DEV_ERR_TIMEOUT) && n ? kLevNone : n;  // (a timeout: pair counts left incomplete)
+      s_run = (level ? err & kStop : err & DEV_ERR_TIMEOUT) ? 0u : n;  // (a timeout: pair counts left incomplete)
+      s_first = single ? blockIdx.x * (level ? kLevWarps / group : kLevWarps) : claim;
     }
     __syncthreads();
-    uint32_t n_run = s_run;  // (one value for the CTA: a group's warps go through the units together)
-    __syncthreads();
+    const uint32_t n_run = s_run;  // (one value for the CTA: a group's warps go through the units together)
     if (n_run == 0) break;
-    if (n_run == kLevNone) n_run = 0;
     const LevUnit* const units = p.units + (uint64_t)par * kLevUnits;
     const uint32_t step = level ? nwarps / group : nwarps;
-    for (uint32_t t = level ? gwarp / group : gwarp; t < n_run; t += step) {
+    uint32_t finished = 0, next = 0;  // units of this group; its next one (group 1: in lane 0)
+    for (uint32_t t = s_first + (level ? wib / group : wib); t < n_run;
+         t = single ? t + step : __shfl_sync(kFull, next, 0)) {
+      if (sub == 0) ++finished;
+      if (!single && sub == 0 && lane == 0) next = atomicAdd(&p.state->level[level].head, 1u);
       uint32_t plen, nc, s0, own = 0, row0 = 0;
       const uint32_t *sups, *rows_of = nullptr;
       __syncwarp();
@@ -387,10 +402,14 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
           if (lane == g && g < cnt) s0 = s;
         }
         if (group > 1) {  // (two buffers: a third round's supports are written after the second's barrier)
-          uint32_t(*const part)[kLevCand] = s_part[round++ & 1u] + ((threadIdx.x >> 5) & ~(group - 1));
+          const uint32_t buf = round++ & 1u;
+          uint32_t(*const part)[kLevCand] = s_part[buf] + (wib - sub);
+          uint32_t* const nx = s_next[buf] + (wib - sub);
           if (sub && lane < kLevCand) part[sub][lane] = s0;
+          if (sub == 0 && lane == 0) *nx = next;
           __syncwarp();
-          asm volatile("bar.sync %0, %1;" ::"r"(1 + (threadIdx.x >> 5) / group), "r"(group * 32) : "memory");
+          asm volatile("bar.sync %0, %1;" ::"r"(1 + wib / group), "r"(group * 32) : "memory");
+          if (sub) next = *nx;
           if (sub) continue;
           if (lane < cnt)
             for (uint32_t g = 1; g < group; ++g) s0 += part[g][lane];
@@ -411,7 +430,10 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
       }
       finish(plen, nc, s0, sups, rows_of, row0, own, level + 1);
     }
-    if (single || !grid_barrier(&p.state->arrived, &p.state->arrived, &p.ctrl->err, epoch)) break;
+    if (single) break;
+    LevCount* const c = p.state->level + level;
+    if (!phase_wait(finished, &c->done, n_run, &c->head, &c->head, &p.ctrl->err, kStop, &s_done, [&] { claim_of(level + 1); }))
+      break;
   }
   if (lane == 0 && st_sets) {
     atomicAdd(&p.ctrl->sets_total, st_sets);
@@ -432,7 +454,7 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
 
 }  // namespace
 
-// co-resident CTAs of the launch, asked once per device
+// CTAs of the launch (as many as run at once), asked once per device
 cudaError_t levels_ctas(int num_sms, uint32_t* out) {
   static std::mutex mu;
   static std::map<int, uint32_t> known;
@@ -451,9 +473,7 @@ cudaError_t levels_ctas(int num_sms, uint32_t* out) {
 }
 
 cudaError_t launch_levels(const LevLaunch& p, uint32_t ctas, cudaStream_t st) {
-  // The first levels, which nearly every search has, as launches of their own, the others until one is empty.  A captured
-  // mine is the quicker for it (dense_deep: 121 us a replay, 122 with all levels in the cooperative launch), an eager one 3%
-  // slower (a step of dense_deep's database 325 us against 316); more such launches lose in both.
+  // The first levels, which nearly every search has, as launches of their own, the others until one is empty.
   LevLaunch q = p;
   q.cta_time = nullptr;
   for (q.group = 1; q.group < kLevWarps && q.group * kLevSeg4 * 4 < p.stride; q.group *= 2) {}
@@ -464,11 +484,7 @@ cudaError_t launch_levels(const LevLaunch& p, uint32_t ctas, cudaStream_t st) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   q.cta_time = p.cta_time;
-  uint32_t first = kLevSingles;
-  bool single = false;
-  void* args[] = {&q, &first, &single};
-  e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_levels), dim3(ctas), dim3(kLevThreads), args, 0, st);
-  if (e != cudaSuccess) return e;
+  k_levels<<<ctas, kLevThreads, 0, st>>>(q, kLevSingles, false);
   note_launch();
   return cudaGetLastError();
 }

@@ -71,36 +71,50 @@ __device__ __forceinline__ RegionView region_view(const uint32_t* R) {
   return v;
 }
 
-constexpr unsigned long long kBarrierIdleNs = 2000000000ull;
+constexpr unsigned long long kPhaseIdleNs = 2000000000ull;
 
-// All CTAs of a cooperative grid meet (epoch: barriers passed so far); false when the wait ran out: no CTA arrived and
-// *progress did not change for 2 s, or another CTA gave up.
-__device__ inline bool grid_barrier(uint32_t* arrived, const uint32_t* progress, uint32_t* err, uint32_t& epoch) {
+// The end of a phase whose `total` units the warps of the grid claim one after the other: the CTA adds the units that it has
+// finished (mine: this warp's, given by lane 0) to *done and waits until all are.  False when the kernel is to end: an error
+// in `stop` was set, or the wait ran out (no unit finished, claimed (*head) or reported alive (*progress) for 2 s:
+// DEV_ERR_TIMEOUT).
+// A CTA waits only for units that running CTAs have claimed, and these finish them without waiting, so the CTAs that are
+// resident get through the phases however few they are, and one that starts late goes past what is over.  That is why
+// these kernels need no cooperative launch, which starts only when all its CTAs fit and so waits for the longest kernel on
+// any other stream (three threads of steps on 100 items beside another thread's mines of 60 ms: 57 ms a step with
+// cooperative launches).
+// s_done is 0 on entry and on return.  meanwhile(): called by thread 0 once the units are added (claims ahead of that fence
+// would hold them back).
+template <typename F>
+__device__ inline bool phase_wait(uint32_t mine, uint32_t* done, uint32_t total, const uint32_t* head, const uint32_t* progress,
+                                  uint32_t* err, uint32_t stop, uint32_t* s_done, F&& meanwhile) {
   __shared__ uint32_t s_ok;
+  if ((threadIdx.x & 31) == 0 && mine) atomicAdd(s_done, mine);
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    atomicAdd(arrived, 1u);
-    const uint32_t want = (epoch + 1) * gridDim.x;
-    uint32_t ok = 1, seen = kFull, taken = kFull;
+    if (*s_done) atomicAdd(done, *s_done);
+    *s_done = 0;
+    meanwhile();
+    uint32_t ok = 1, seen = kFull, taken = kFull, alive = kFull;
     unsigned long long t0 = 0;
     for (uint32_t poll = 0;; ++poll) {
-      const uint32_t a = ld_volatile(arrived);
-      if (a >= want) break;
+      const uint32_t a = ld_volatile(done);
+      if (a >= total) break;
       if (poll < 32) continue;  // (a microsecond or two: levels are short)
       __nanosleep(40);
       if (poll & 15u) continue;
-      if (ld_volatile(err) & DEV_ERR_TIMEOUT) {
+      if (ld_volatile(err) & (stop | DEV_ERR_TIMEOUT)) {
         ok = 0;
         break;
       }
-      const uint32_t h = ld_volatile(progress);
+      const uint32_t h = ld_volatile(head), g = ld_volatile(progress);
       const unsigned long long now = global_ns();
-      if (a != seen || h != taken) {
+      if (a != seen || h != taken || g != alive) {
         seen = a;
         taken = h;
+        alive = g;
         t0 = now;
-      } else if (now - t0 > kBarrierIdleNs) {
+      } else if (now - t0 > kPhaseIdleNs) {
         atomicOr(err, DEV_ERR_TIMEOUT);
         ok = 0;
         break;
@@ -110,7 +124,6 @@ __device__ inline bool grid_barrier(uint32_t* arrived, const uint32_t* progress,
     s_ok = ok;
   }
   __syncthreads();
-  ++epoch;
   return s_ok != 0;
 }
 

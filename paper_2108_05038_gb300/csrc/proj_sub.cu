@@ -24,8 +24,9 @@
 //           rows, masked by the prefix), and so does what is left of a subtree that has taken
 //           kSubCycles: no warp keeps a round waiting for long.
 //
-// One cooperative launch runs all rounds; between the phases of a round its CTAs meet at a barrier
-// (bounded: no CTA arrived and no item taken anywhere for 2 s ends the kernel with DEV_ERR_TIMEOUT).
+// One launch runs all rounds.  The warps claim the units, tiles and items of a phase one after the other, and a CTA goes on
+// to the next phase when all are finished (phase_wait; bounded: no progress anywhere for 2 s ends the kernel with
+// DEV_ERR_TIMEOUT).
 // Whatever finds no room in the queues is left to k_dfs_proj, which takes any frame.  The classes,
 // nodes, candidates and records are those of k_dfs_proj.
 #include <algorithm>
@@ -306,7 +307,8 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
   const uint32_t lane = threadIdx.x & 31;
   SubSmem& S = reinterpret_cast<SubSmem*>(smem)[threadIdx.x >> 5];
   const uint32_t lt = (1u << lane) - 1u;
-  const uint32_t gwarp = blockIdx.x * kSubWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kSubWarps;
+  const uint32_t nwarps = gridDim.x * kSubWarps;
+  __shared__ uint32_t s_done, s_first[2][3];  // of phase_wait; the claims of this round and the next
   unsigned long long st_inter = 0, st_nodes = 0, st_frames = 0, st_bytes = 0, st_sets = 0, st_items = 0;
   uint32_t st_maxlen = 0, st_parts = 0;
   uint32_t nrec = 0;                  // buffered records
@@ -331,19 +333,52 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
     pend_sets = 0;
   };
 
-  uint32_t epoch = 0;
+  // A CTA claims the first units, tiles and items of a round, one of each for every warp, before the wait for the round
+  // above: no claim is waited for, and no warp gets a second one before each has had one.  The others of a long list are
+  // claimed a few at a time.
+  const uint32_t wib = threadIdx.x >> 5;
+  auto claim_round = [&](uint32_t round) {  // (thread 0)
+    SubRound& r = p.state->round[round];
+    s_first[round & 1u][0] = round ? atomicAdd(&r.unit_head, kSubWarps) : 0u;
+    s_first[round & 1u][1] = atomicAdd(&r.tile_head, kSubWarps);
+    s_first[round & 1u][2] = atomicAdd(&r.item_head, kSubWarps);
+  };
+  // f(t) for the warp's share of 0 .. n - 1; returns how many it took
+  auto share = [&](uint32_t first, uint32_t* head, uint32_t n, auto&& f) {
+    const uint32_t chunk = max(1u, min(8u, n / (8 * nwarps)));
+    uint32_t t0 = first, t1 = t0 + 1, taken = 0, next = 0;
+    while (t0 < n) {
+      if (lane == 0) next = atomicAdd(head, chunk);
+      for (uint32_t t = t0; t < min(t1, n); ++t, ++taken) f(t);
+      t0 = __shfl_sync(kFull, next, 0);
+      t1 = t0 + chunk;
+    }
+    return taken;
+  };
+  auto wait = [&](uint32_t mine, uint32_t* done, uint32_t total, const uint32_t* head, bool claim, uint32_t round) {
+    return phase_wait(mine, done, total, head, &p.state->progress, &p.ctrl->err, kSubStop, &s_done, [&] {
+      if (claim) claim_round(round + 1);
+    });
+  };
+  if (threadIdx.x == 0) {
+    s_done = 0;
+    claim_round(0);
+  }
+  __syncthreads();
   for (uint32_t round = 0;; ++round) {
     // ---------------- pairs ----------------
     const uint32_t par = round & 1u;
-    const uint32_t n_tiles = round ? min(ld_volatile(&p.state->tile_n[round]), kSubTileCap) : p.tileoff[p.n1];
-    const uint32_t n_items = round ? min(ld_volatile(&p.state->item_n[round]), kSubItemCap) : p.ctrl->n_entries_g;
+    SubRound& now = p.state->round[round];
+    SubRound& next_round = p.state->round[round + 1];
+    const uint32_t n_tiles = round ? min(ld_volatile(&now.tile_n), kSubTileCap) : p.tileoff[p.n1];
+    const uint32_t n_items = round ? min(ld_volatile(&now.item_n), kSubItemCap) : p.ctrl->n_entries_g;
     if (n_items == 0) break;
     // ---------------- rows of the parts that get their own ----------------
-    const uint32_t n_units = round ? min(ld_volatile(&p.state->unit_n[round]), kSubTileCap) : 0u;
-    for (uint32_t t = gwarp; t < n_units; t += nwarps) {
+    const uint32_t n_units = round ? min(ld_volatile(&now.unit_n), kSubTileCap) : 0u;
+    const uint32_t my_units = share(s_first[par][0] + wib, &now.unit_head, n_units, [&](uint32_t t) {
       const uint4 d = __ldcg(reinterpret_cast<const uint4*>(p.units + t));
       const uint4 d2 = __ldcg(reinterpret_cast<const uint4*>(p.units + t) + 1);
-      if (d.x == kNoop) continue;
+      if (d.x == kNoop) return;
       const RegionView V = region_view(p.Y + (uint64_t)d.x * 4);
       const uint32_t path_len = d.z & 0xffffu, cnt = d.z >> 16, u = d2.w & 0xffffu;
       __syncwarp();
@@ -352,10 +387,9 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
       __syncwarp();
       gather_rows(&S, V.Y, V.Wp, path_len, u * kUnitWords, min(V.W, (u + 1) * kUnitWords),
                   p.Y + ((uint64_t)d2.y << 32 | d2.x), d2.z, d2.w >> 16, cnt);
-      if (lane == 0) atomicAdd(&p.state->progress, 1u);
-    }
-    if (n_units && !grid_barrier(&p.state->arrived, &p.state->progress, &p.ctrl->err, epoch)) break;
-    for (uint32_t t = gwarp; t < n_tiles; t += nwarps) {
+    });
+    if (n_units && !wait(my_units, &now.unit_done, n_units, &now.unit_head, false, round)) break;
+    const uint32_t my_tiles = share(s_first[par][1] + wib, &now.tile_head, n_tiles, [&](uint32_t t) {
       if (round == 0) {
         uint32_t lo = 0, hi = p.n1;  // the class: the last queue position q with tileoff[q] <= t
         while (hi - lo > 1) {
@@ -373,31 +407,28 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
       } else {
         const uint4 d = __ldcg(reinterpret_cast<const uint4*>(p.tiles + t));
         const uint4 d2 = __ldcg(reinterpret_cast<const uint4*>(p.tiles + t) + 1);
-        if (d.x == kNoop) continue;
+        if (d.x == kNoop) return;
         const RegionView V = region_view(p.Y + (uint64_t)d.x * 4);
         gram_tile(V, d.y == kIdentity ? nullptr : p.lists + d.y, d.z, d.w, p.G + d2.x, d2.y & 0xffffu, d2.y >> 16, d2.z * kGramWords,
                   min(V.W, (d2.z + 1) * kGramWords), V.W > kGramWords);
       }
-      if (lane == 0) atomicAdd(&p.state->progress, 1u);
-    }
-    if (n_tiles && !grid_barrier(&p.state->arrived, &p.state->progress, &p.ctrl->err, epoch)) break;
-    // (the other halves of G, the lists and the items are free: the round before is over.  This round's are the next
-    // one's other halves: empty again)
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.state->g_top[par] = p.state->l_top[par] = 0;
+    });
+    if (n_tiles && !wait(my_tiles, &now.tile_done, n_tiles, &now.tile_head, false, round)) break;
+    // (the other halves of G, the lists and the items are free: the round before is over)
     const bool last = round + 2 >= kSubRounds;
     SubItem* const items = p.items + (uint64_t)par * kSubItemCap;
     SubItem* const next_items = p.items + (uint64_t)(par ^ 1u) * kSubItemCap;
     const uint64_t g_lo = (uint64_t)(par ^ 1u) * (p.g_cap / 2), l_lo = (uint64_t)(par ^ 1u) * kSubListCap;
 
     // ---------------- walk ----------------
-    for (;;) {
+    uint32_t my_items = 0;
+    auto next_item = [&]() {
       uint32_t e = 0;
-      if (lane == 0) {
-        e = (ld_volatile(&p.ctrl->err) & kSubStop) ? kFull : atomicAdd(&p.state->item_head[round], 1u);
-        atomicAdd(&p.state->progress, 1u);
-      }
-      e = __shfl_sync(kFull, e, 0);
-      if (e >= n_items || stop) break;
+      if (lane == 0) e = (ld_volatile(&p.ctrl->err) & kSubStop) ? kFull : atomicAdd(&now.item_head, 1u);
+      ++my_items;
+      return __shfl_sync(kFull, e, 0);
+    };
+    for (uint32_t e = s_first[par][2] + wib; e < n_items && !stop; e = next_item()) {
       SubItem it;
       if (round) {
         const uint4 d = __ldcg(reinterpret_cast<const uint4*>(items + e));
@@ -523,12 +554,12 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
           if (lane == 0) {
             const unsigned long long gw = (unsigned long long)n * (n + 1) / 2;
             const unsigned long long size = own ? (rows_off + (unsigned long long)n * Wpn + 31) & ~31ull : 0ull;
-            const unsigned long long l = atomicAdd(&p.state->l_top[par ^ 1u], (unsigned long long)(np_rows + n));
-            const unsigned long long gq = atomicAdd(&p.state->g_top[par ^ 1u], gw);
-            ti = atomicAdd(&p.state->tile_n[round + 1], nt * chunks);
-            ii = atomicAdd(&p.state->item_n[round + 1], n - 1);
+            const unsigned long long l = atomicAdd(&next_round.l_top, (unsigned long long)(np_rows + n));
+            const unsigned long long gq = atomicAdd(&next_round.g_top, gw);
+            ti = atomicAdd(&next_round.tile_n, nt * chunks);
+            ii = atomicAdd(&next_round.item_n, n - 1);
             if (own) {
-              ui = atomicAdd(&p.state->unit_n[round + 1], n_units * nj);
+              ui = atomicAdd(&next_round.unit_n, n_units * nj);
               dst = atomicAdd(&p.ctrl->arena_top, size);
             }
             ok = l + np_rows + n <= kSubListCap && gq + gw <= p.g_cap / 2 && ti + nt * chunks <= kSubTileCap &&
@@ -1003,8 +1034,8 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
             }
             uint32_t slot = 0, at = 0, ok = 0;
             if (cnt && lane == 0) {
-              const unsigned long long l = atomicAdd(&p.state->l_top[par ^ 1u], (unsigned long long)words);
-              slot = atomicAdd(&p.state->item_n[round + 1], cnt);
+              const unsigned long long l = atomicAdd(&next_round.l_top, (unsigned long long)words);
+              slot = atomicAdd(&next_round.item_n, cnt);
               ok = l + words <= kSubListCap && slot + cnt <= kSubItemCap;
               at = (uint32_t)(l_lo + l);
             }
@@ -1072,7 +1103,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
         if (p.class_work && cls_work) atomicAdd(&p.class_work[cls], cls_work);
       }
     }
-    if (!grid_barrier(&p.state->arrived, &p.state->progress, &p.ctrl->err, epoch)) break;
+    if (!wait(my_items, &now.item_done, n_items, &now.item_head, round + 1 < kSubRounds, round)) break;
     if (round + 1 >= kSubRounds) break;
   }
   if (!p.out_off && pend_sets) flush_count();
@@ -1090,7 +1121,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
   }
 }
 
-// dynamic shared memory and co-resident CTAs of k_sub, asked once per device
+// dynamic shared memory and CTAs of k_sub (as many as run at once), asked once per device
 cudaError_t sub_ctas(int num_sms, uint32_t* out) {
   static std::mutex mu;
   static std::map<int, uint32_t> known;
@@ -1117,11 +1148,7 @@ cudaError_t launch_sub(const SubLaunch& p, int num_sms, cudaStream_t st) {
   cudaError_t e = sub_ctas(num_sms, &ctas);
   if (e != cudaSuccess) return e;
   if (ctas == 0) return cudaErrorInvalidConfiguration;
-  SubLaunch q = p;
-  void* args[] = {&q};
-  e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_sub), dim3(ctas), dim3(kSubThreads), args,
-                                  kSubWarps * sizeof(SubSmem), st);
-  if (e != cudaSuccess) return e;
+  k_sub<<<ctas, kSubThreads, kSubWarps * sizeof(SubSmem), st>>>(p);
   note_launch();
   return cudaGetLastError();
 }

@@ -82,7 +82,7 @@ def test_itemset_limit_stops_the_walk(limit):
 
 
 def test_plan_replays_the_walk():
-    """The cooperative launch inside a captured graph."""
+    """The walk's launch inside a captured graph."""
     off, items, N = CASES["some_rows"][0]()
     db = fim.build_vertical_db(off, items, N)
     try:
