@@ -198,6 +198,13 @@ typedef struct {
                                   the AND+popcount intersections of the class [r | rows after r],
                                   level 2 and below (the actual cost that the sample estimate
                                   predicts); 0 for rows that are not frequent                      */
+  /* room and time of the search by levels and of the small-subtree walk (0 = automatic; below it: tests of what they do
+   * without room).  A caller built without these four fields passes the struct_size that it has without them. */
+  uint32_t walk_queue;         /* entries of each of their queues                                  */
+  uint32_t walk_words;         /* 32-bit words of row lists, of pair supports and (walk) of database
+                                  parts beside the classes' own                                    */
+  uint32_t walk_rounds;        /* rounds of the walk                                               */
+  uint32_t walk_cycles;        /* clock cycles after which a subtree's rest is handed on           */
 } fim_mine_opts;
 
 /* Fill *opts with the defaults (struct_size set, all options default). */

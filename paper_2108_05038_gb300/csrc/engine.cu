@@ -57,6 +57,7 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
   ep->leaves = cfg.output == FIM_OUTPUT_MAXIMAL;  // (mine_input made such a mine projected)
   ep->diffsets = cfg.diffsets;
   ep->donate = ep->mode == 0 ? cfg.donate : 0u;  // only dense node expansion donates
+  ep->walk = cfg.walk;
   ep->spin_limit = cfg.spin_limit ? cfg.spin_limit : 2000000ull;
   ep->fixed_capacity = cfg.fixed_capacity;
   ep->cap_sets = cfg.cap_sets ? cfg.cap_sets : std::max<uint64_t>((uint64_t)1 << 18, 8ull * n1 + 64);
@@ -253,7 +254,9 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     }
     FIM_TRY(ws_get(ws, WS_ENTRIES_F, ep->npairs_max + 1, &ep->d_entries_f));
     // the arena holds the class regions (within proj_y_cap), then the regions of split frames
-    ep->proj_arena_words = ep->proj_y_cap + (share ? std::max<uint64_t>(ep->proj_y_cap, 16ull << 20) : 0ull);
+    ep->proj_arena_words = ep->proj_y_cap + (!share           ? 0ull
+                                             : cfg.walk.words ? cfg.walk.words
+                                                              : std::max<uint64_t>(ep->proj_y_cap, 16ull << 20));
     ep->split_words = cfg.split_words;  // 0: chosen on the device from the class regions' mean width
     ep->dq_cap = share ? kProjDqCap : 0u;
     FIM_TRY(ws_get(ws, WS_PROJ_Y, ep->proj_arena_words, &ep->d_Y));
@@ -337,6 +340,9 @@ cudaError_t engine_launch_front(const EnginePlan& ep, cudaStream_t st, bool pair
   return cudaSuccess;
 }
 
+// room of an arena of `own`, or the caller's limit of it
+static uint64_t capped(uint64_t own, uint64_t limit) { return limit ? std::min(own, limit) : own; }
+
 cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
   if (ep.n1 == 0) return cudaSuccess;
   cudaError_t ce = cudaSuccess;
@@ -356,6 +362,10 @@ cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
     l.class_sets = ep.d_class_sets;
     l.class_work = ep.d_class_work;
     l.max_sets = ep.max_sets;
+    l.node_cap = (uint32_t)capped(kLevNodes, ep.walk.queue);
+    l.unit_cap = (uint32_t)capped(kLevUnits, ep.walk.queue);
+    l.list_cap = capped(kLevListWords, ep.walk.words);
+    l.sup_cap = capped(kLevSupWords, ep.walk.words);
     l.cta_time = ep.d_cta_time;
     if (ep.d_class_sets) ce = cudaMemsetAsync(ep.d_class_sets, 0, (size_t)ep.n1 * sizeof(unsigned long long), st);
     if (ce != cudaSuccess) return ce;
@@ -436,7 +446,10 @@ cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
         if (ce != cudaSuccess) return ce;
       }
       if (ep.sub) {
-        const SubLaunch sl{ep.d_Y, ep.proj_arena_words, ep.d_G, kSubGramCap, ep.d_yoff, ep.d_order, ep.d_tileoff, ep.n1,
+        const SubLaunch sl{ep.d_Y, ep.proj_arena_words, ep.d_G, capped(kSubGramCap / 2, ep.walk.words),
+                           (uint32_t)capped(kSubItemCap, ep.walk.queue), (uint32_t)capped(kSubTileCap, ep.walk.queue),
+                           capped(kSubListCap, ep.walk.words), (uint32_t)capped(kSubRounds, ep.walk.rounds),
+                           ep.walk.cycles ? ep.walk.cycles : kSubCycles, ep.d_yoff, ep.d_order, ep.d_tileoff, ep.n1,
                            ep.minsup, ep.d_entries_g, ep.d_sub_items, ep.d_sub_tiles, ep.d_sub_units, ep.d_sub_lists, ep.d_sub_state, ep.d_off,
                            ep.d_items, ep.d_supp, dl.cap_sets, dl.cap_items, ep.d_ctrl, ep.d_class_sets,
                            ep.d_class_work, ep.max_sets, dl.leaves, ep.d_dq, ep.dq_cap};

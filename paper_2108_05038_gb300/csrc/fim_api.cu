@@ -486,6 +486,11 @@ static void engine_config_from_opts(const fim_mine_opts* o, EngineConfig* c) {
     if (!c->cap_items) c->cap_items = 1;
   }
   c->collect_times = o->collect_times != 0;
+  if (o->struct_size == sizeof(fim_mine_opts)) c->walk = {o->walk_queue, o->walk_words, o->walk_rounds, o->walk_cycles};
+}
+
+bool opts_size_ok(const fim_mine_opts* o) {
+  return o->struct_size == sizeof(fim_mine_opts) || o->struct_size == offsetof(fim_mine_opts, walk_queue);
 }
 
 
@@ -505,7 +510,7 @@ fim_status mine_input(fim_db* db, uint32_t minsup_abs, const fim_mine_opts* opts
   if (!db) return fail(FIM_ERR_INVALID, "db is NULL");
   if (minsup_abs == 0) return fail(FIM_ERR_INVALID, "minsup 0 makes every subset frequent");
   if (minsup_abs < db->prefilter) return fail(FIM_ERR_INVALID, "minsup below the prefilter support of the database");
-  if (opts && opts->struct_size != 0 && opts->struct_size != sizeof(fim_mine_opts))
+  if (opts && opts->struct_size != 0 && !opts_size_ok(opts))
     return fail(FIM_ERR_INVALID, "fim_mine_opts.struct_size mismatch");
   rows_for_minsup(db, minsup_abs, in);
   in->bits = db->d_bits;

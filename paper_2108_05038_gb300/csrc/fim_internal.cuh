@@ -329,6 +329,11 @@ struct EngineOutput {
   DevCtrl ctrl{};
 };
 
+// the caller's limits of the two searches' room (0: their arenas' own)
+struct WalkRoom {
+  uint32_t queue = 0, words = 0, rounds = 0, cycles = 0;
+};
+
 struct EngineConfig {
   uint32_t depth_first = 0;  // 0 = automatic
   uint32_t threads = 0;      // 0 = automatic
@@ -355,6 +360,7 @@ struct EngineConfig {
   uint64_t split_words = 0;  // 0 = automatic; else a frame whose next level reads more words is split
   uint32_t output = 0;       // FIM_OUTPUT_*: maximal makes the DFS write its leaves only
   uint32_t diffsets = 0;     // projected DFS: 0 never, 1 where smaller than bitmaps, 2 always
+  WalkRoom walk;
 };
 
 // Everything one mining call launches, with its geometry and buffers.  The
@@ -366,6 +372,7 @@ constexpr uint32_t kSubRounds = 48;
 constexpr uint32_t kSubItemCap = 1u << 17;  // items of a round after the first
 constexpr uint32_t kSubTileCap = 1u << 17;  // tiles of pairs of a round after the first
 constexpr uint64_t kSubListCap = 1ull << 21;  // words of a round's row lists
+constexpr uint32_t kSubCycles = 400000;      // cycles (about 0.2 ms) after which a subtree's rest is handed on
 constexpr uint64_t kSubGramCap = 1ull << 24;  // words of G: two halves, of this round's and the next one's pairs
 constexpr uint32_t kSubTask = 0xfffffffeu;  // SubItem.m: the rest of a subtree
 // A part: the transactions of region roff4 (units of 4 words of Y; kNoop: no work) that hold path_len of its rows, and
@@ -428,6 +435,8 @@ struct LevLaunch {
   uint64_t max_sets;
   unsigned long long* cta_time;
   uint32_t group;  // warps of a unit
+  uint32_t node_cap, unit_cap;  // room of a level
+  uint64_t list_cap, sup_cap;
 };
 cudaError_t levels_ctas(int num_sms, uint32_t* out);
 cudaError_t launch_levels(const LevLaunch& p, uint32_t ctas, cudaStream_t st);
@@ -479,6 +488,7 @@ struct EnginePlan {
   uint4* d_dq = nullptr;
   uint32_t dq_cap = 0;
   bool sub = false;  // small subtrees walked by proj_sub.cu
+  WalkRoom walk;
   bool levels = false;  // the search a level at a time (levels.cu)
   uint32_t lev_grid = 0;
   LevLaunch lev{};
@@ -519,6 +529,8 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
                          bool* retry);
 // the EngineInput / EngineConfig of a fim_mine call (validation included); with defer_ok a pending estimate
 // stays pending (the queue order is derived on the device, the output capacity left to the caller)
+// fim_mine_opts.struct_size is that of the struct, or of the struct as it was without the walk_* fields
+bool opts_size_ok(const fim_mine_opts* o);
 fim_status mine_input(fim_db* db, uint32_t minsup, const fim_mine_opts* opts, EngineInput* in, EngineConfig* cfg,
                       bool defer_ok = false);
 // the first output capacity that the database's estimate suggests for a minsup (0: none)
@@ -725,7 +737,12 @@ struct SubLaunch {
   uint32_t* Y;
   uint64_t arena_words;
   uint32_t* G;
-  uint64_t g_cap;
+  // room: of a half of G, items, tiles (and units), list words; rounds; cycles for a subtree
+  uint64_t g_half;
+  uint32_t item_cap, tile_cap;
+  uint64_t list_cap;
+  uint32_t rounds;
+  long long cycles;
   const uint64_t* yoff;
   const uint32_t *row_order, *tileoff;
   uint32_t n1, minsup;

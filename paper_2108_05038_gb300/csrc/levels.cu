@@ -256,9 +256,9 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
     const uint32_t ni = __shfl_sync(kFull, g32, 4), ui = __shfl_sync(kFull, g32, 5);
     const unsigned long long after = (base >> 32) + sets;
     if (lane == 0 && ((p.max_sets && after > p.max_sets) || after > 0xfffffff0ull)) atomicOr(&p.ctrl->err, DEV_ERR_ABORTED);
-    const bool fits = frame && (uint64_t)li + plen + n <= kLevListWords &&
-                      (uint64_t)si + n * (n - 1) / 2 <= kLevSupWords && (uint64_t)ni + n - 1 <= kLevNodes &&
-                      (uint64_t)ui + n_units <= kLevUnits && plen + 1 < kLevPath && next + 1 < kLevMax;
+    const bool fits = frame && (uint64_t)li + plen + n <= p.list_cap &&
+                      (uint64_t)si + n * (n - 1) / 2 <= p.sup_cap && (uint64_t)ni + n - 1 <= p.node_cap &&
+                      (uint64_t)ui + n_units <= p.unit_cap && plen + 1 < kLevPath && next + 1 < kLevMax;
     if (frame && !fits && lane == 0) atomicOr(&p.ctrl->err, DEV_ERR_SUB);
     uint32_t* const list = p.lists + (uint64_t)par * kLevListWords + li;
     uint32_t* const nsup = p.sups + (uint64_t)par * kLevSupWords + si;
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kLevThreads, kLevCtasPerSm) k_levels(const __g
       // After an error no unit is touched: a frame that found no room leaves its reserved units unwritten, and its error was
       // set before the level above was finished.
       const uint32_t err = ld_volatile(&p.ctrl->err);
-      const uint32_t n = level ? min(ld_volatile(&p.state->level[level].units), kLevUnits) : p.n1;
+      const uint32_t n = level ? min(ld_volatile(&p.state->level[level].units), p.unit_cap) : p.n1;
       s_run = (level ? err & kStop : err & DEV_ERR_TIMEOUT) ? 0u : n;  // (a timeout: pair counts left incomplete)
       s_first = single ? blockIdx.x * (level ? kLevWarps / group : kLevWarps) : claim;
     }

@@ -61,7 +61,7 @@ using namespace fim;
 extern "C" {
 
 fim_status fim_autotune(fim_db* db, uint32_t minsup_abs, fim_mine_opts* opts, float* best_ms) {
-  if (!opts || opts->struct_size != sizeof(fim_mine_opts)) return fail(FIM_ERR_INVALID, "opts must be initialised");
+  if (!opts || !opts_size_ok(opts)) return fail(FIM_ERR_INVALID, "opts must be initialised");
   EngineInput in;
   EngineConfig cfg;
   FIM_TRY(mine_input(db, minsup_abs, opts, &in, &cfg));

@@ -44,7 +44,6 @@ constexpr uint32_t kSubWarps = kSubThreads / 32;
 constexpr uint32_t kSubCtasPerSm = 2;
 constexpr uint32_t kSubPool = 2576;      // words per warp: rows, prefix, child masks
 constexpr uint32_t kSubRows = 32;        // rows of a part held in shared memory (with the prefix ids at most 64)
-constexpr long long kSubCycles = 400000;  // cycles (about 0.2 ms) after which a subtree's rest goes to the next round
 constexpr uint32_t kUnitWords = 512;      // words of a region that a unit of a part's rows covers
 constexpr uint32_t kSubAll = 5;          // at most so many survivors: every subset of them counted in one pass
 
@@ -370,11 +369,11 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
     const uint32_t par = round & 1u;
     SubRound& now = p.state->round[round];
     SubRound& next_round = p.state->round[round + 1];
-    const uint32_t n_tiles = round ? min(ld_volatile(&now.tile_n), kSubTileCap) : p.tileoff[p.n1];
-    const uint32_t n_items = round ? min(ld_volatile(&now.item_n), kSubItemCap) : p.ctrl->n_entries_g;
+    const uint32_t n_tiles = round ? min(ld_volatile(&now.tile_n), p.tile_cap) : p.tileoff[p.n1];
+    const uint32_t n_items = round ? min(ld_volatile(&now.item_n), p.item_cap) : p.ctrl->n_entries_g;
     if (n_items == 0) break;
     // ---------------- rows of the parts that get their own ----------------
-    const uint32_t n_units = round ? min(ld_volatile(&now.unit_n), kSubTileCap) : 0u;
+    const uint32_t n_units = round ? min(ld_volatile(&now.unit_n), p.tile_cap) : 0u;
     const uint32_t my_units = share(s_first[par][0] + wib, &now.unit_head, n_units, [&](uint32_t t) {
       const uint4 d = __ldcg(reinterpret_cast<const uint4*>(p.units + t));
       const uint4 d2 = __ldcg(reinterpret_cast<const uint4*>(p.units + t) + 1);
@@ -415,10 +414,10 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
     });
     if (n_tiles && !wait(my_tiles, &now.tile_done, n_tiles, &now.tile_head, false, round)) break;
     // (the other halves of G, the lists and the items are free: the round before is over)
-    const bool last = round + 2 >= kSubRounds;
+    const bool last = round + 1 >= p.rounds;
     SubItem* const items = p.items + (uint64_t)par * kSubItemCap;
     SubItem* const next_items = p.items + (uint64_t)(par ^ 1u) * kSubItemCap;
-    const uint64_t g_lo = (uint64_t)(par ^ 1u) * (p.g_cap / 2), l_lo = (uint64_t)(par ^ 1u) * kSubListCap;
+    const uint64_t g_lo = (uint64_t)(par ^ 1u) * (kSubGramCap / 2), l_lo = (uint64_t)(par ^ 1u) * kSubListCap;
 
     // ---------------- walk ----------------
     uint32_t my_items = 0;
@@ -562,8 +561,8 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
               ui = atomicAdd(&next_round.unit_n, n_units * nj);
               dst = atomicAdd(&p.ctrl->arena_top, size);
             }
-            ok = l + np_rows + n <= kSubListCap && gq + gw <= p.g_cap / 2 && ti + nt * chunks <= kSubTileCap &&
-                 ii + n - 1 <= kSubItemCap && (!own || (ui + n_units * nj <= kSubTileCap && dst + size <= p.arena_words));
+            ok = l + np_rows + n <= p.list_cap && gq + gw <= p.g_half && ti + nt * chunks <= p.tile_cap &&
+                 ii + n - 1 <= p.item_cap && (!own || (ui + n_units * nj <= p.tile_cap && dst + size <= p.arena_words));
             lo = (uint32_t)(l_lo + l);
             go = (uint32_t)(g_lo + gq);
           }
@@ -577,12 +576,12 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
           // (reserved slots below the capacities are filled in any case)
           const uint32_t r4 = !ok ? kNoop : own ? (uint32_t)(dst / 4) : it.roff4, plen = own ? 0u : np_rows;
           const uint32_t lrows = lo + np_rows - plen;  // (own rows: the list, which names rows of the region, is not used)
-          for (uint32_t t = lane; t < nt * chunks && ti + t < kSubTileCap; t += 32) {
+          for (uint32_t t = lane; t < nt * chunks && ti + t < p.tile_cap; t += 32) {
             uint32_t ba, bb;
             tile_of(t % nt, ba, bb);
             p.tiles[ti + t] = SubTile{r4, own ? kIdentity : lrows, plen, n, go, ba | bb << 16, t / nt, 0};
           }
-          for (uint32_t t = lane; t < n - 1 && ii + t < kSubItemCap; t += 32)
+          for (uint32_t t = lane; t < n - 1 && ii + t < p.item_cap; t += 32)
             next_items[ii + t] = SubItem{r4, own ? kIdentity : lrows, plen, n, go, t, {0, 0}};
           if (own)
             for (uint32_t u = 0; u < n_units; ++u) {
@@ -590,7 +589,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
               for (uint32_t j = lane; j < nj; j += 32) {
                 const uint32_t slot = ui + u * nj + j;
                 const unsigned long long d = dst + rows_off + (unsigned long long)(32 * j) * Wpn + off;
-                if (slot < kSubTileCap)
+                if (slot < p.tile_cap)
                   p.units[slot] = SubUnit{ok && words ? it.roff4 : kNoop, lo, np_rows | min(32u, n - 32 * j) << 16, 32 * j,
                                           (uint32_t)d, (uint32_t)(d >> 32), Wpn, u | words << 16};
               }
@@ -1022,7 +1021,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
           }
           cm_top += nf;
           __syncwarp();
-          if (!tried && clock64() - t_start > kSubCycles) {
+          if (!tried && clock64() - t_start > p.cycles) {
             // what is left goes to the next round: every open child of every open frame, with its rows
             tried = true;
             uint32_t cnt = 0, words = 0, base = cm_top;
@@ -1036,7 +1035,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
             if (cnt && lane == 0) {
               const unsigned long long l = atomicAdd(&next_round.l_top, (unsigned long long)words);
               slot = atomicAdd(&next_round.item_n, cnt);
-              ok = l + words <= kSubListCap && slot + cnt <= kSubItemCap;
+              ok = l + words <= p.list_cap && slot + cnt <= p.item_cap;
               at = (uint32_t)(l_lo + l);
             }
             ok = __shfl_sync(kFull, ok, 0);
@@ -1056,7 +1055,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
                     if ((rows_p >> lane) & 1u) p.lists[at + np_rows + popm(rows_p & lt)] = S.lrow[lane];
                     if ((rows_s >> lane) & 1u) p.lists[at + pl + popm(rows_s & lt)] = S.lrow[lane];
                   }
-                  if (lane == 0 && slot < kSubItemCap)
+                  if (lane == 0 && slot < p.item_cap)
                     next_items[slot] = SubItem{ok ? it.roff4 : kNoop, at, pl, ns, 0, kSubTask, {0, 0}};
                   at += pl + ns;
                 }
@@ -1103,8 +1102,8 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
         if (p.class_work && cls_work) atomicAdd(&p.class_work[cls], cls_work);
       }
     }
-    if (!wait(my_items, &now.item_done, n_items, &now.item_head, round + 1 < kSubRounds, round)) break;
-    if (round + 1 >= kSubRounds) break;
+    if (!wait(my_items, &now.item_done, n_items, &now.item_head, round + 1 < p.rounds, round)) break;
+    if (round + 1 >= p.rounds) break;
   }
   if (!p.out_off && pend_sets) flush_count();
   if (lane == 0 && st_nodes) {

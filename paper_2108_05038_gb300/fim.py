@@ -75,6 +75,8 @@ class MineOpts(ctypes.Structure):
         ("out_needed_sets", ctypes.c_uint64),
         ("out_needed_items", ctypes.c_uint64), ("stats", ctypes.POINTER(MineStats)),
         ("class_work_out", ctypes.c_void_p),
+        ("walk_queue", ctypes.c_uint32), ("walk_words", ctypes.c_uint32), ("walk_rounds", ctypes.c_uint32),
+        ("walk_cycles", ctypes.c_uint32),
     ]
 
 
@@ -336,7 +338,7 @@ class Database:
 
     def _opts(self, class_order="estimate", threads_per_cta=0, vec_per_lane=0, ctas_per_sm=0, donate=False,
               result_on_device=False, collect_times=False, out_capacity_sets=0, out_capacity_items=0, spin_limit=0,
-              stats=True, shape=None, dfs_mode=None, max_itemsets=0, pair_kernel=FIM_PAIR_AUTO):
+              stats=True, shape=None, dfs_mode=None, max_itemsets=0, pair_kernel=FIM_PAIR_AUTO, walk=None):
         opts = MineOpts()
         self._lib.fim_mine_opts_init(ctypes.byref(opts))
         opts.pair_kernel = pair_kernel
@@ -357,6 +359,9 @@ class Database:
         opts.out_capacity_items = out_capacity_items
         opts.spin_limit = spin_limit
         opts.max_itemsets = max_itemsets
+        for key, value in (walk or {}).items():  # queue, words, rounds, cycles
+            setattr(opts, {"queue": "walk_queue", "words": "walk_words", "rounds": "walk_rounds",
+                           "cycles": "walk_cycles"}[key], value)
         st = MineStats() if stats else None
         if st is not None:
             opts.stats = ctypes.pointer(st)
@@ -384,12 +389,12 @@ class Database:
              shape=None, dfs_mode: int | None = None, max_itemsets: int = 0, class_work: bool = False,
              dfs_depth_first: int = 0, pair_kernel: int = FIM_PAIR_AUTO, fault_pair_wait: bool = False,
              proj_bitmap_words: int = 0, proj_stack_words: int = 0, proj_max_row_words: int = 0,
-             proj_split_words: int = 0, output: str = "all", diffsets: int = 0):
-        """fim_mine; with ``class_work`` the result carries ``class_work`` (u64[n_rows]): the intersections
+             proj_split_words: int = 0, output: str = "all", diffsets: int = 0, walk: dict | None = None):
+        """fim_mine; ``walk``: the opts' walk_* fields by their last word; with ``class_work`` the result carries ``class_work`` (u64[n_rows]): the intersections
         of every one-row class, level 2 and below."""
         opts, st = self._opts(class_order, threads_per_cta, vec_per_lane, ctas_per_sm, donate, result_on_device,
                               collect_times, out_capacity_sets, out_capacity_items, spin_limit, stats, shape, dfs_mode,
-                              max_itemsets, pair_kernel)
+                              max_itemsets, pair_kernel, walk)
         opts.dfs_depth_first = dfs_depth_first
         opts.fault_pair_wait = 1 if fault_pair_wait else 0
         opts.proj_bitmap_words = proj_bitmap_words

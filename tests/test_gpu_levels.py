@@ -57,6 +57,29 @@ def test_same_search_as_frame_passes(name):
         db.free()
 
 
+@pytest.mark.parametrize("room", [dict(queue=1), dict(queue=20), dict(words=1), dict(words=100)], ids=str)
+@pytest.mark.parametrize("name", ["many_survivors", "wide_rows", "deep"])
+def test_without_room(name, room):
+    """A search that finds no room in its arenas is repeated by the frame passes."""
+    make, minsup = CASES[name]
+    off, items, N = make()
+    want = odict(oracle.eclat(off, items, N, minsup))
+    db = fim.build_vertical_db(off, items, N)
+    try:
+        n = [fim.kernel_launches()]
+        got = db.mine(minsup, class_work=True)
+        n.append(fim.kernel_launches())
+        got2 = db.mine(minsup, class_work=True, walk=room)
+        n.append(fim.kernel_launches())
+        assert n[2] - n[1] > n[1] - n[0]  # (repeated)
+        assert got.as_dict() == want and got2.as_dict() == want
+        for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len"):
+            assert got.stats[key] == got2.stats[key], key
+        assert np.array_equal(got.class_work, got2.class_work)
+    finally:
+        db.free()
+
+
 @pytest.mark.parametrize("words", [384, 416, 512, 544, 800, 832, 1_024, 1_056, 2_048, 2_080, 4_096, 4_128])
 def test_row_lengths(words):
     """Rows at the edges of one, two, four and eight warps a unit and one or two segments, and of the one-pass subtrees."""

@@ -67,6 +67,55 @@ def test_same_walk_as_sparse_nodes(name):
         db.free()
 
 
+# what the walk does without room: parts, subtrees' rests and their rows go to the projected DFS, or the run is repeated
+# without the walk; a cycle per subtree hands on everything that can be
+ROOMS = {
+    "one_entry": dict(queue=1, cycles=1),
+    "forty_entries": dict(queue=40, cycles=2_000),
+    "some_entries": dict(queue=700, cycles=1),
+    "no_words": dict(words=1, cycles=1),
+    "some_words": dict(words=6_000, cycles=1),
+    "one_round": dict(rounds=1, cycles=1),
+    "three_rounds": dict(rounds=3, cycles=1),
+    "all_rounds": dict(cycles=1),
+}
+
+
+@pytest.fixture(scope="module")
+def searched():
+    """The cases' databases, their itemsets and the sparse node mode's counters, made once."""
+    made = {}
+
+    def get(name):
+        if name not in made:
+            make, minsup = CASES[name]
+            off, items, N = make()
+            db = fim.build_vertical_db(off, items, N)
+            ref = db.mine(minsup, dfs_mode=fim.FIM_DFS_SPARSE, class_work=True, class_order="uniform")
+            want = odict(oracle.eclat(off, items, N, minsup))
+            assert ref.as_dict() == want
+            made[name] = db, minsup, want, ref
+        return made[name]
+
+    yield get
+    for db, *_ in made.values():
+        db.free()
+
+
+@pytest.mark.parametrize("room", ROOMS)
+@pytest.mark.parametrize("name", ["many_rows", "deep", "wide", "wide_dense"])
+def test_without_room(searched, name, room):
+    db, minsup, want, ref = searched(name)
+    got = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, class_work=True, class_order="uniform", walk=ROOMS[room])
+    assert got.as_dict() == want
+    for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len"):
+        assert got.stats[key] == ref.stats[key], key
+    assert np.array_equal(got.class_work, ref.class_work)
+    top = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, output="maximal", walk=ROOMS[room]).as_dict()
+    covered = {k[:i] + k[i + 1:] for k in want for i in range(len(k))}
+    assert top == {k: v for k, v in want.items() if k not in covered}
+
+
 @pytest.mark.parametrize("limit", [50, 2_000])
 def test_itemset_limit_stops_the_walk(limit):
     off, items, N = CASES["deep"][0]()
