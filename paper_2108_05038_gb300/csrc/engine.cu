@@ -452,7 +452,7 @@ cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
                            ep.walk.cycles ? ep.walk.cycles : kSubCycles, ep.d_yoff, ep.d_order, ep.d_tileoff, ep.n1,
                            ep.minsup, ep.d_entries_g, ep.d_sub_items, ep.d_sub_tiles, ep.d_sub_units, ep.d_sub_lists, ep.d_sub_state, ep.d_off,
                            ep.d_items, ep.d_supp, dl.cap_sets, dl.cap_items, ep.d_ctrl, ep.d_class_sets,
-                           ep.d_class_work, ep.max_sets, dl.leaves, ep.d_dq, ep.dq_cap};
+                           ep.d_class_work, ep.max_sets, dl.leaves, ep.d_dq, ep.dq_cap / 2};  // (the rest for k_dfs_proj's own)
         ce = launch_sub(sl, ep.num_sms, st);
         if (ce != cudaSuccess) return ce;
       }

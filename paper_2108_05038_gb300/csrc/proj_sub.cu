@@ -22,7 +22,7 @@
 //           kept in a small buffer and written up to 64 at a time behind one reservation.  A part
 //           that does not fit goes to the next round with its candidates (and the class region's
 //           rows, masked by the prefix), and so does what is left of a subtree that has taken
-//           kSubCycles: no warp keeps a round waiting for long.
+//           kSubCycles (without room there it goes to k_dfs_proj): no warp keeps a round waiting for long.
 //
 // One launch runs all rounds.  The warps claim the units, tiles and items of a phase one after the other, and a CTA goes on
 // to the next phase when all are finished (phase_wait; bounded: no progress anywhere for 2 s ends the kernel with
@@ -149,6 +149,48 @@ __device__ __forceinline__ void leave_to_dfs(const SubLaunch& p, uint64_t roff, 
   }
   atomicAdd(&p.ctrl->proj_pending, 1u);
   p.dq[slot] = make_uint4((uint32_t)roff, (uint32_t)(roff >> 32), m, 1u);
+}
+
+// Leaves a frame of the part in S.pool (W words a row) to k_dfs_proj: prefix rows rows_p, prefix ids pid (positions in
+// S.ids), two or more survivors rows_s.  Its database part, the survivors' words under the prefix, becomes a region of the
+// arena, its extensions items of the shared queue.  False without room in the arena (the run is repeated without k_sub).
+__device__ __noinline__ bool leave_subtree(const SubLaunch* pp, SubSmem* Sp, uint32_t rows_p, uint32_t rows_s,
+                                           unsigned long long pid, uint32_t W, uint32_t cls) {
+  const SubLaunch& p = *pp;
+  SubSmem& S = *Sp;
+  const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+  const uint32_t ns = __popc(rows_s), plen = __popcll(pid), Ws = W | 1u, Wp = (W + 3) & ~3u;
+  const uint64_t rows_off = region_rows_off(plen, ns);
+  const unsigned long long size = (rows_off + (unsigned long long)ns * Wp + 31) & ~31ull;
+  unsigned long long off = 0;
+  if (lane == 0) off = atomicAdd(&p.ctrl->arena_top, size);
+  off = __shfl_sync(kFull, off, 0);
+  if (off + size > p.arena_words) {
+    if (lane == 0) atomicOr(&p.ctrl->err, DEV_ERR_SUB);
+    return false;
+  }
+  uint32_t* const R = p.Y + off;
+  if (lane == 0) {
+    R[0] = ns;
+    R[1] = Wp;
+    R[2] = plen;
+    R[3] = W;
+    R[4] = cls;
+    R[5] = kNoGram;
+    R[6] = R[7] = 0;
+  }
+  for (uint32_t q = lane; q < 64; q += 32)
+    if ((pid >> q) & 1ull) R[8 + __popcll(pid & ((1ull << q) - 1ull))] = S.ids[q];
+  if ((rows_s >> lane) & 1u) R[8 + ((plen + 3) & ~3u) + __popc(rows_s & lt)] = S.ids[S.at[lane]];
+  uint32_t* const Y2 = R + rows_off;
+  for (uint32_t w = lane; w < Wp; w += 32) {
+    uint32_t v = w < W ? kFull : 0u;
+    for (uint32_t t = rows_p; t && v; t &= t - 1) v &= S.pool[(__ffs(t) - 1) * Ws + w];
+    uint32_t j = 0;
+    for (uint32_t t = rows_s; t; t &= t - 1, ++j) Y2[(uint64_t)j * Wp + w] = v ? S.pool[(__ffs(t) - 1) * Ws + w] & v : 0u;
+  }
+  for (uint32_t t = lane; t + 1 < ns; t += 32) leave_to_dfs(p, off, t);
+  return true;
 }
 
 constexpr uint32_t kSubStop = DEV_ERR_ABORTED | DEV_ERR_PSTACK | DEV_ERR_TIMEOUT | DEV_ERR_SUB;
@@ -669,6 +711,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
           for (uint32_t j0 = 0; j0 < n; j0 += 32) {
             __syncwarp();
             if (j0 + lane < n) S.lrow[lane] = rows[j0 + lane];
+            if (lane == 0) atomicAdd(&p.state->progress, 1u);
             gather_rows(&S, V.Y, V.Wp, np_rows, 0, V.W, Y2 + (uint64_t)j0 * Wp, Wp, Wp, min(32u, n - j0));
           }
           st_bytes += 4ull * n * supp + 4ull * n * Wp;
@@ -864,7 +907,6 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
         uint32_t plen = xlen, cm_top = 0;
         const long long t_start = clock64();
         int32_t depth = -1;
-        bool tried = last;
         // one record per lane with f: rec and its support
         auto put = [&](bool f, unsigned long long rec, uint32_t supp_rec) {
           const uint32_t bal = __ballot_sync(kFull, f), cnt = __popc(bal);
@@ -1021,9 +1063,11 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
           }
           cm_top += nf;
           __syncwarp();
-          if (!tried && clock64() - t_start > p.cycles) {
-            // what is left goes to the next round: every open child of every open frame, with its rows
-            tried = true;
+          if (clock64() - t_start > p.cycles) {
+            // what is left goes to the next round: every open child of every open frame, with its rows; without room there,
+            // and in the last round, to k_dfs_proj, whose warps share large frames.  (A warp that walked on alone kept the
+            // others waiting, past the end of their patience: 27 items in every transaction, queues of one entry: a timeout
+            // after 4.4 s, now 0.8 s; 24 items 2.5 s, now 1.35.)
             uint32_t cnt = 0, words = 0, base = cm_top;
             for (int32_t d = depth; d >= 0; --d) {
               const M sd = surv[d];
@@ -1031,8 +1075,8 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
               const uint32_t pl = np_rows + popm((M)S.path[d]) + 1;
               for (M t = todo[d]; t; t &= t - 1, ++cnt) words += pl + popm(cm0[base + popm(sd & ((one << low(t)) - 1))]);
             }
-            uint32_t slot = 0, at = 0, ok = 0;
-            if (cnt && lane == 0) {
+            uint32_t slot = p.item_cap, at = 0, ok = 0;
+            if (cnt && !last && lane == 0) {
               const unsigned long long l = atomicAdd(&next_round.l_top, (unsigned long long)words);
               slot = atomicAdd(&next_round.item_n, cnt);
               ok = l + words <= p.list_cap && slot + cnt <= p.item_cap;
@@ -1041,27 +1085,29 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
             ok = __shfl_sync(kFull, ok, 0);
             at = __shfl_sync(kFull, at, 0);
             slot = __shfl_sync(kFull, slot, 0);
-            if (cnt) {
-              base = cm_top;
-              for (int32_t d = depth; d >= 0; --d) {
-                const M sd = surv[d], pd = (M)S.path[d];
-                base -= popm(sd);
-                for (M t = todo[d]; t; t &= t - 1, ++slot) {
-                  const uint32_t r = low(t);
-                  const M rows_p = pd | one << r, rows_s = cm0[base + popm(sd & ((one << r) - 1))];
-                  const uint32_t pl = np_rows + popm(rows_p), ns = popm(rows_s);
-                  if (ok) {
-                    for (uint32_t q = lane; q < np_rows; q += 32) p.lists[at + q] = S.prow[q];
-                    if ((rows_p >> lane) & 1u) p.lists[at + np_rows + popm(rows_p & lt)] = S.lrow[lane];
-                    if ((rows_s >> lane) & 1u) p.lists[at + pl + popm(rows_s & lt)] = S.lrow[lane];
-                  }
-                  if (lane == 0 && slot < p.item_cap)
-                    next_items[slot] = SubItem{ok ? it.roff4 : kNoop, at, pl, ns, 0, kSubTask, {0, 0}};
-                  at += pl + ns;
+            base = cm_top;
+            for (int32_t d = depth; d >= 0; --d) {
+              const M sd = surv[d], pd = (M)S.path[d];
+              base -= popm(sd);
+              for (M t = todo[d]; t; t &= t - 1, ++slot) {
+                const uint32_t r = low(t);
+                const M rows_p = pd | one << r, rows_s = cm0[base + popm(sd & ((one << r) - 1))];
+                const uint32_t pl = np_rows + popm(rows_p), ns = popm(rows_s);
+                if (ok) {
+                  for (uint32_t q = lane; q < np_rows; q += 32) p.lists[at + q] = S.prow[q];
+                  if ((rows_p >> lane) & 1u) p.lists[at + np_rows + popm(rows_p & lt)] = S.lrow[lane];
+                  if ((rows_s >> lane) & 1u) p.lists[at + pl + popm(rows_s & lt)] = S.lrow[lane];
+                } else {
+                  ++st_frames;
+                  st_bytes += 4ull * W * (popm(rows_p) + 2 * ns);
+                  stop |= !leave_subtree(&p, &S, rows_p, rows_s, S.pids[d] | 1ull << S.at[r], W, cls);
                 }
+                if (lane == 0 && slot < p.item_cap)
+                  next_items[slot] = SubItem{ok ? it.roff4 : kNoop, at, pl, ns, 0, kSubTask, {0, 0}};
+                at += pl + ns;
               }
             }
-            if (ok || cnt == 0) break;  // (without room for all of them the walk goes on here)
+            break;
           }
           // ---- the next child: of the deepest frame that has one ----
           M t = todo[depth];

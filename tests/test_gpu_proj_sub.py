@@ -116,6 +116,20 @@ def test_without_room(searched, name, room):
     assert top == {k: v for k, v in want.items() if k not in covered}
 
 
+def test_large_subtree_without_room():
+    """27 items in every one of 64 transactions, queues of one entry: a part with 2^25 itemsets below it finds no room for
+    its rest in the next round, and is shared by the warps of the projected DFS all the same."""
+    k, D = 27, 64
+    db = fim.build_vertical_db((np.arange(D + 1) * k).astype(np.uint32), np.tile(np.arange(k, dtype=np.uint32), D), k)
+    try:
+        for walk in (dict(), dict(queue=1)):
+            r = db.mine(D, dfs_mode=fim.FIM_DFS_PROJECTED, result_on_device=True, walk=walk)
+            assert r.n_sets == 2 ** k - 1 and r.stats["max_len"] == k and r.stats["n_items_out"] == k * 2 ** (k - 1)
+            r.free()
+    finally:
+        db.free()
+
+
 @pytest.mark.parametrize("limit", [50, 2_000])
 def test_itemset_limit_stops_the_walk(limit):
     off, items, N = CASES["deep"][0]()
