@@ -393,8 +393,8 @@ struct alignas(32) SubUnit {  // rows j0 .. of a part's own region, over 256 wor
 // One round: the words of G and of the lists that its parts take, its items, tiles and units, how many of each have been
 // claimed, and (on a line of their own: polled) how many are finished
 struct alignas(128) SubRound {
-  unsigned long long g_top, l_top;
-  uint32_t item_n, tile_n, unit_n, item_head, tile_head, unit_head;
+  unsigned long long g_top, l_top, item_n, tile_n, unit_n;  // (64 bits: parts that found no room are counted too)
+  uint32_t item_head, tile_head, unit_head;
   alignas(64) uint32_t item_done, tile_done, unit_done;
 };
 struct SubState {

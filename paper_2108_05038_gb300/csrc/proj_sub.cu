@@ -411,11 +411,14 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
     const uint32_t par = round & 1u;
     SubRound& now = p.state->round[round];
     SubRound& next_round = p.state->round[round + 1];
-    const uint32_t n_tiles = round ? min(ld_volatile(&now.tile_n), p.tile_cap) : p.tileoff[p.n1];
-    const uint32_t n_items = round ? min(ld_volatile(&now.item_n), p.item_cap) : p.ctrl->n_entries_g;
+    auto within = [](const unsigned long long* n, uint32_t cap) {
+      return (uint32_t)min(*(volatile const unsigned long long*)n, (unsigned long long)cap);
+    };
+    const uint32_t n_tiles = round ? within(&now.tile_n, p.tile_cap) : p.tileoff[p.n1];
+    const uint32_t n_items = round ? within(&now.item_n, p.item_cap) : p.ctrl->n_entries_g;
     if (n_items == 0) break;
     // ---------------- rows of the parts that get their own ----------------
-    const uint32_t n_units = round ? min(ld_volatile(&now.unit_n), p.tile_cap) : 0u;
+    const uint32_t n_units = round ? within(&now.unit_n, p.tile_cap) : 0u;
     const uint32_t my_units = share(s_first[par][0] + wib, &now.unit_head, n_units, [&](uint32_t t) {
       const uint4 d = __ldcg(reinterpret_cast<const uint4*>(p.units + t));
       const uint4 d2 = __ldcg(reinterpret_cast<const uint4*>(p.units + t) + 1);
@@ -564,7 +567,8 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
       const bool all = small && n <= kSubAll && !(task && p.leaves);  // (a task's rows come without their supports)
       if (walk && !task && !all && !sub_fits(n, xlen, W)) {
         // not a part for one warp: the next round's (its candidates, their pairs to count, and its extensions)
-        uint32_t ok = 0, lo = 0, go = 0, ti = 0, ii = 0, ui = 0;
+        uint32_t ok = 0, lo = 0, go = 0;
+        unsigned long long ti = 0, ii = 0, ui = 0;
         const uint32_t nb = (n + kGramRows - 1) / kGramRows, nt = nb * (nb + 1) / 2;
         // When X's transactions are few among the region's, the part gets rows of its own over them, built by units of
         // kUnitWords words x 32 rows (every unit's transactions start at a whole word); else it is the region's rows, masked.
@@ -589,6 +593,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
         }
         const uint32_t Wn = own ? unit_words : V.W, Wpn = (Wn + 3) & ~3u;
         const uint32_t chunks = (Wn + kGramWords - 1) / kGramWords;
+        const unsigned long long n_part_tiles = (unsigned long long)nt * chunks;
         const uint64_t rows_off = region_rows_off(xlen, n);
         unsigned long long dst = 0;
         if (!last && n <= 0xffffu && np_rows < 60) {
@@ -597,13 +602,13 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
             const unsigned long long size = own ? (rows_off + (unsigned long long)n * Wpn + 31) & ~31ull : 0ull;
             const unsigned long long l = atomicAdd(&next_round.l_top, (unsigned long long)(np_rows + n));
             const unsigned long long gq = atomicAdd(&next_round.g_top, gw);
-            ti = atomicAdd(&next_round.tile_n, nt * chunks);
-            ii = atomicAdd(&next_round.item_n, n - 1);
+            ti = atomicAdd(&next_round.tile_n, n_part_tiles);
+            ii = atomicAdd(&next_round.item_n, (unsigned long long)(n - 1));
             if (own) {
-              ui = atomicAdd(&next_round.unit_n, n_units * nj);
+              ui = atomicAdd(&next_round.unit_n, (unsigned long long)n_units * nj);
               dst = atomicAdd(&p.ctrl->arena_top, size);
             }
-            ok = l + np_rows + n <= p.list_cap && gq + gw <= p.g_half && ti + nt * chunks <= p.tile_cap &&
+            ok = l + np_rows + n <= p.list_cap && gq + gw <= p.g_half && ti + n_part_tiles <= p.tile_cap &&
                  ii + n - 1 <= p.item_cap && (!own || (ui + n_units * nj <= p.tile_cap && dst + size <= p.arena_words));
             lo = (uint32_t)(l_lo + l);
             go = (uint32_t)(g_lo + gq);
@@ -618,7 +623,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
           // (reserved slots below the capacities are filled in any case)
           const uint32_t r4 = !ok ? kNoop : own ? (uint32_t)(dst / 4) : it.roff4, plen = own ? 0u : np_rows;
           const uint32_t lrows = lo + np_rows - plen;  // (own rows: the list, which names rows of the region, is not used)
-          for (uint32_t t = lane; t < nt * chunks && ti + t < p.tile_cap; t += 32) {
+          for (uint32_t t = lane; t < n_part_tiles && ti + t < p.tile_cap; t += 32) {
             uint32_t ba, bb;
             tile_of(t % nt, ba, bb);
             p.tiles[ti + t] = SubTile{r4, own ? kIdentity : lrows, plen, n, go, ba | bb << 16, t / nt, 0};
@@ -629,7 +634,7 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
             for (uint32_t u = 0; u < n_units; ++u) {
               const uint32_t words = __shfl_sync(kFull, my_words, u), off = __shfl_sync(kFull, my_off, u);
               for (uint32_t j = lane; j < nj; j += 32) {
-                const uint32_t slot = ui + u * nj + j;
+                const unsigned long long slot = ui + u * nj + j;
                 const unsigned long long d = dst + rows_off + (unsigned long long)(32 * j) * Wpn + off;
                 if (slot < p.tile_cap)
                   p.units[slot] = SubUnit{ok && words ? it.roff4 : kNoop, lo, np_rows | min(32u, n - 32 * j) << 16, 32 * j,
@@ -1075,10 +1080,11 @@ __global__ void __launch_bounds__(kSubThreads, kSubCtasPerSm) k_sub(const __grid
               const uint32_t pl = np_rows + popm((M)S.path[d]) + 1;
               for (M t = todo[d]; t; t &= t - 1, ++cnt) words += pl + popm(cm0[base + popm(sd & ((one << low(t)) - 1))]);
             }
-            uint32_t slot = p.item_cap, at = 0, ok = 0;
+            unsigned long long slot = p.item_cap;
+            uint32_t at = 0, ok = 0;
             if (cnt && !last && lane == 0) {
               const unsigned long long l = atomicAdd(&next_round.l_top, (unsigned long long)words);
-              slot = atomicAdd(&next_round.item_n, cnt);
+              slot = atomicAdd(&next_round.item_n, (unsigned long long)cnt);
               ok = l + words <= p.list_cap && slot + cnt <= p.item_cap;
               at = (uint32_t)(l_lo + l);
             }
