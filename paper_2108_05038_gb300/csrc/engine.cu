@@ -241,8 +241,10 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
     ep->d_goff = ep->d_eoffx + n1;
     ep->d_tileoff = ep->d_goff + n1;
     // Small subtrees in shared memory first, unless the caller tunes the general walk (its hand-out threshold, its
-    // stacks, diffset frames), or its shared queue, which takes what they leave, is off.
-    ep->sub = share && !db->served && !cfg.split_words && !cfg.pstack_words && !cfg.diffsets;
+    // stacks, diffset frames), or its shared queue, which takes what they leave, is off.  (Its row offsets within a region
+    // are 32-bit words: not with a budget of class bitmaps, which only the caller sets so large, of 2^32 words.)
+    ep->sub = share && !db->served && !cfg.split_words && !cfg.pstack_words && !cfg.diffsets &&
+              ep->proj_y_cap < (1ull << 32);
     if (ep->sub) {
       FIM_TRY(ws_get(ws, WS_ENTRIES_G, ep->npairs_max + 1, &ep->d_entries_g));
       FIM_TRY(ws_get(ws, WS_SUB_G, kSubGramCap, &ep->d_G));

@@ -130,6 +130,18 @@ def test_large_subtree_without_room():
         db.free()
 
 
+def test_class_bitmaps_past_32_bit_offsets(searched):
+    """With a budget that lets a class region hold 2^32 words the walk, whose row offsets have 32 bits, is left out."""
+    db, minsup, want, ref = searched("many_rows")
+    count = []
+    for words in (1 << 24, (1 << 32) - 1, 1 << 32):
+        c = fim.kernel_launches()
+        got = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, proj_bitmap_words=words, walk=dict(words=100_000))
+        count.append(fim.kernel_launches() - c)
+        assert got.as_dict() == want and got.stats["n_intersections"] == ref.stats["n_intersections"]
+    assert count[1] == count[0] and count[2] == count[0] - 1
+
+
 @pytest.mark.parametrize("limit", [50, 2_000])
 def test_itemset_limit_stops_the_walk(limit):
     off, items, N = CASES["deep"][0]()
