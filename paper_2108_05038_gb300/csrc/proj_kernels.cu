@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kProjThreads, kProjCtasPerSm) k_dfs_proj(const
   unsigned long long pend_sets = 0;
   uint32_t st_maxlen = 0;
   bool static_done = false;
-  constexpr uint32_t kStop = DEV_ERR_ABORTED | DEV_ERR_PSTACK | DEV_ERR_TIMEOUT;
+  constexpr uint32_t kStop = DEV_ERR_ABORTED | DEV_ERR_PSTACK | DEV_ERR_TIMEOUT | DEV_ERR_SUB;  // (SUB: k_sub asks for a repeat)
 
   auto sort_path = [&](uint32_t len) {
     __syncwarp();
