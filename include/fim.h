@@ -199,12 +199,15 @@ typedef struct {
                                   level 2 and below (the actual cost that the sample estimate
                                   predicts); 0 for rows that are not frequent                      */
   /* room and time of the search by levels and of the small-subtree walk (0 = automatic; below it: tests of what they do
-   * without room).  A caller built without these four fields passes the struct_size that it has without them. */
+   * without room).  A caller built without these fields passes the struct_size that it has without them. */
   uint32_t walk_queue;         /* entries of each of their queues                                  */
   uint32_t walk_words;         /* 32-bit words of row lists, of pair supports and (walk) of database
                                   parts beside the classes' own                                    */
   uint32_t walk_rounds;        /* rounds of the walk                                               */
   uint32_t walk_cycles;        /* clock cycles after which a subtree's rest is handed on           */
+  uint32_t fault_plan_room;    /* 0 (default); 1 = failure-detection test: the replays of a plan have
+                                  room for one entry and one word (and hand work on at once), its
+                                  sizing run the room asked for                                    */
 } fim_mine_opts;
 
 /* Fill *opts with the defaults (struct_size set, all options default). */
@@ -367,6 +370,9 @@ fim_status fim_autotune(fim_db* db, uint32_t minsup_abs, fim_mine_opts* opts, fl
  * fim_plan_launch enqueues one replay (asynchronous); fim_plan_result waits
  * for the last replay and returns its itemsets (host or device per
  * opts->result_on_device; opts may be NULL; opts->stats receives counters).
+ * The room that a search takes can differ between replays (it hands work on by
+ * the clock): one that found too little is repeated by fim_plan_result itself,
+ * and the plan captured anew with what was missing.
  * db must outlive the plan and stay unchanged.
  * Errors: as fim_mine; FIM_ERR_INVALID for a result before any launch.
  */

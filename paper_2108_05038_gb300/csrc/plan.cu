@@ -5,7 +5,9 @@
 // DFS launch over all classes in queue order - and captures it once in a CUDA
 // graph, so that repeated mining of the same database replays one graph.
 // Sizes (output capacity, DFS stack depth) come from one eager run at
-// creation, so a replay never needs to grow a buffer.
+// creation, so a replay rarely needs to grow a buffer: the searches hand work
+// on by the clock, and one that finds no room where the eager run did is
+// repeated eagerly, and the graph captured anew (fim_plan_result).
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -50,6 +52,25 @@ struct TuneKey {
     return std::tie(stride, n1, minsup, rows) < std::tie(o.stride, o.n1, o.minsup, o.rows);
   }
 };
+// The launch sequence captured with the plan's sizes, in place of an earlier capture.
+fim_status plan_capture(fim_plan* plan) {
+  if (plan->exec) cudaGraphExecDestroy(plan->exec);
+  if (plan->graph) cudaGraphDestroy(plan->graph);
+  plan->exec = nullptr;
+  plan->graph = nullptr;
+  FIM_CUDA(cudaStreamBeginCapture(plan->stream, cudaStreamCaptureModeRelaxed));
+  const uint64_t before = launches_so_far();
+  const cudaError_t le = engine_launch(plan->ep, plan->stream);
+  // launches recorded into the graph run only when it is launched
+  plan->kernels = launches_so_far() - before;
+  note_launch(0 - plan->kernels);
+  const cudaError_t e = cudaStreamEndCapture(plan->stream, &plan->graph);
+  if (le != cudaSuccess) return cuda_fail(le, "capturing the mining kernels");
+  if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
+  FIM_CUDA(cudaGraphInstantiate(&plan->exec, plan->graph, 0));
+  return FIM_OK;
+}
+
 std::mutex g_tune_mu;
 std::map<TuneKey, std::pair<Shape, float>> g_tuned;
 
@@ -145,18 +166,12 @@ fim_status fim_plan_create(fim_db* db, uint32_t minsup_abs, fim_mine_opts* opts,
   fim_status s = engine_mine(db, plan->ws, in, cfg, &eo, nullptr, &plan->ep);
   if (s != FIM_OK) return bail(s);
   plan->ep.fixed_capacity = true;
-  cudaError_t e = cudaStreamBeginCapture(plan->stream, cudaStreamCaptureModeRelaxed);
-  if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamBeginCapture"));
-  const uint64_t before = launches_so_far();
-  cudaError_t le = engine_launch(plan->ep, plan->stream);
-  // launches recorded into the graph run only when it is launched
-  plan->kernels = launches_so_far() - before;
-  note_launch(0 - plan->kernels);
-  e = cudaStreamEndCapture(plan->stream, &plan->graph);
-  if (le != cudaSuccess) return bail(cuda_fail(le, "capturing the mining kernels"));
-  if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamEndCapture"));
-  e = cudaGraphInstantiate(&plan->exec, plan->graph, 0);
-  if (e != cudaSuccess) return bail(cuda_fail(e, "cudaGraphInstantiate"));
+  if (opts && opts->struct_size == sizeof(fim_mine_opts) && opts->fault_plan_room) {
+    plan->ep.walk = {1, 1, 0, 1};
+    plan->ep.proj_arena_words = 1;
+  }
+  s = plan_capture(plan);
+  if (s != FIM_OK) return bail(s);
   *out = plan;
   return FIM_OK;
 }
@@ -179,7 +194,14 @@ fim_status fim_plan_result(fim_plan* plan, fim_mine_opts* opts, fim_result** out
   EngineOutput eo;
   bool retry = false;
   FIM_TRY(engine_finish(plan->db, plan->stream, &plan->ep, &eo, stats, &retry));
-  if (retry) return fail(FIM_ERR_OUTPUT_OVERFLOW, "plan buffers no longer fit the database");
+  const bool again = retry;
+  for (int attempt = 0; retry; ++attempt) {  // (engine_finish has grown, or left out, what ran out of room)
+    if (attempt == 8) return fail(FIM_ERR_OUTPUT_OVERFLOW, "plan buffers no longer fit the database");
+    FIM_TRY(engine_alloc(plan->ws, &plan->ep));
+    FIM_CUDA(engine_launch(plan->ep, plan->stream));
+    FIM_TRY(engine_finish(plan->db, plan->stream, &plan->ep, &eo, stats, &retry));
+  }
+  if (again) FIM_TRY(plan_capture(plan));
   return make_result(plan->stream, eo, opts && opts->struct_size && opts->result_on_device, out);
 }
 

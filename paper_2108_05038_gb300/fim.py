@@ -76,7 +76,7 @@ class MineOpts(ctypes.Structure):
         ("out_needed_items", ctypes.c_uint64), ("stats", ctypes.POINTER(MineStats)),
         ("class_work_out", ctypes.c_void_p),
         ("walk_queue", ctypes.c_uint32), ("walk_words", ctypes.c_uint32), ("walk_rounds", ctypes.c_uint32),
-        ("walk_cycles", ctypes.c_uint32),
+        ("walk_cycles", ctypes.c_uint32), ("fault_plan_room", ctypes.c_uint32),
     ]
 
 
@@ -338,7 +338,7 @@ class Database:
 
     def _opts(self, class_order="estimate", threads_per_cta=0, vec_per_lane=0, ctas_per_sm=0, donate=False,
               result_on_device=False, collect_times=False, out_capacity_sets=0, out_capacity_items=0, spin_limit=0,
-              stats=True, shape=None, dfs_mode=None, max_itemsets=0, pair_kernel=FIM_PAIR_AUTO, walk=None):
+              stats=True, shape=None, dfs_mode=None, max_itemsets=0, pair_kernel=FIM_PAIR_AUTO, walk=None, fault_plan_room=False):
         opts = MineOpts()
         self._lib.fim_mine_opts_init(ctypes.byref(opts))
         opts.pair_kernel = pair_kernel
@@ -362,6 +362,7 @@ class Database:
         for key, value in (walk or {}).items():  # queue, words, rounds, cycles
             setattr(opts, {"queue": "walk_queue", "words": "walk_words", "rounds": "walk_rounds",
                            "cycles": "walk_cycles"}[key], value)
+        opts.fault_plan_room = 1 if fault_plan_room else 0
         st = MineStats() if stats else None
         if st is not None:
             opts.stats = ctypes.pointer(st)

@@ -78,16 +78,16 @@ def test_struct_offsets_match_header(cname, pycls, tmp_path):
 
 
 def test_opts_of_a_caller_without_the_walk_fields():
-    """struct_size of the struct before its last four fields is accepted (and those are not read); others are refused."""
+    """struct_size of the struct before the walk_* fields is accepted (and those are not read); others are refused."""
     lib = fim.load()
     o = fim.MineOpts()
     lib.fim_mine_opts_init(ctypes.byref(o))
-    for size in (fim.MineOpts.walk_queue.offset, ctypes.sizeof(fim.MineOpts), ctypes.sizeof(fim.MineOpts) - 4):
+    for size in (fim.MineOpts.walk_queue.offset, ctypes.sizeof(fim.MineOpts), ctypes.sizeof(fim.MineOpts) - 8):
         o.struct_size = size
         status = lib.fim_autotune(None, 1, ctypes.byref(o), None)
         text = lib.fim_last_error().decode()
         assert status == fim.FIM_ERR_INVALID
-        assert ("initialised" in text) == (size == ctypes.sizeof(fim.MineOpts) - 4), text
+        assert ("initialised" in text) == (size == ctypes.sizeof(fim.MineOpts) - 8), text
 
 
 def test_invalid_arguments_rejected_without_gpu():

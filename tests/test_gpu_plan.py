@@ -72,6 +72,34 @@ def test_autotune_shape_is_valid_and_output_unchanged():
     db.free()
 
 
+@pytest.mark.parametrize("mode", [None, fim.FIM_DFS_PROJECTED])
+def test_replay_without_room_is_repeated(mode):
+    """Replays whose search by levels, or small-subtree walk, has no room (the sizing run has it): the first result comes
+    from a repeated run, and the plan is captured anew for the launches after it."""
+    rng = np.random.default_rng(8)
+    D, k = 3_000, 45
+    tx = [np.nonzero(rng.random(k) < 0.35)[0] for _ in range(D)]
+    off = np.concatenate([[0], np.cumsum([len(v) for v in tx])]).astype(np.uint32)
+    items = np.concatenate(tx).astype(np.uint32)
+    want = odict(oracle.eclat(off, items, k, 60))
+    db = fim.build_vertical_db(off, items, k)
+    kw = {} if mode is None else {"dfs_mode": mode}
+    try:
+        plan = db.plan(60, fault_plan_room=True, **kw)
+        counts = []
+        for _ in range(3):
+            c = fim.kernel_launches()
+            plan.launch()
+            plan.launch()
+            assert plan.result().as_dict() == want
+            counts.append(fim.kernel_launches() - c)
+        assert counts[0] > counts[1] == counts[2]
+        plan.free()
+        assert db.mine(60, **kw).as_dict() == want
+    finally:
+        db.free()
+
+
 def test_launch_counter_counts_graph_kernels_per_replay():
     """fim_kernel_launches: a mine adds its kernels; each plan replay adds the kernels of its graph."""
     w = synth.make_workload("dense_deep", D=20_000)
