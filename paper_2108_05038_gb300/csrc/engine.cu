@@ -268,6 +268,12 @@ fim_status engine_prepare(fim_db* db, Workspace& ws, const EngineInput& in, cons
   // Automatic, few rows (where frame passes were chosen): by levels
   ep->levels = !db->served && cfg.mode == 2 && ep->mode == 1 && !cfg.donate && cfg.ctas_per_sm == 0 && !cfg.diffsets && !ep->leaves &&
                n1 >= 3 && n1 < 1024 && ep->rows_base;
+  if (ep->levels) {  // not one that has outgrown its arenas before
+    const Outgrown& o = db->outgrown[in.of_sample];
+    ep->rel = in.n_tx ? (double)in.minsup / (double)in.n_tx : 0.0;
+    ep->of_sample = in.of_sample;
+    ep->levels = !(ep->rel <= o.rel && o.queue == cfg.walk.queue && o.words == cfg.walk.words);
+  }
   if (ep->levels) {
     uint8_t* a = nullptr;
     constexpr uint64_t kBytes = 2 * (kLevUnits * sizeof(LevUnit) + 4 * (kLevListWords + kLevSupWords + kLevNodes));
@@ -481,6 +487,12 @@ cudaError_t engine_launch_back(const EnginePlan& ep, cudaStream_t st) {
   return cudaSuccess;
 }
 
+void note_outgrown(fim_db* db, bool of_sample, double rel, const WalkRoom& walk) {
+  Outgrown& o = db->outgrown[of_sample];
+  if (o.queue != walk.queue || o.words != walk.words) o = Outgrown{0.0, walk.queue, walk.words};
+  o.rel = std::max(o.rel, rel);
+}
+
 uint64_t proj_footprint_bytes(uint32_t rows, uint32_t stride, uint64_t nnz, uint32_t grid) {
   const uint64_t y = std::max<uint64_t>((uint64_t)rows * stride / 4, 16ull << 20);  // class bitmaps (words)
   return 4ull * y + 4ull * nnz + 4ull * (uint64_t)grid * (kProjThreads / 32) * kProjStackWords +
@@ -528,6 +540,7 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
   if ((h.err & DEV_ERR_ABORTED) || (ep->max_sets && h.sets_total > ep->max_sets))
     return fail(FIM_ERR_OUTPUT_OVERFLOW, "more frequent itemsets than the limit: mining stopped early (counts are lower bounds)");
   if (h.err & DEV_ERR_SUB) {  // no room in the small-subtree walk's queues: repeat without it
+    if (ep->levels) note_outgrown(db, ep->of_sample, ep->rel, ep->walk);
     ep->sub = ep->levels = false;
     *retry = true;
     return FIM_OK;

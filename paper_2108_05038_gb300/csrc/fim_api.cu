@@ -519,6 +519,7 @@ fim_status mine_input(fim_db* db, uint32_t minsup_abs, const fim_mine_opts* opts
   in->d_rank_item = db->d_rank_item;
   in->minsup = minsup_abs;
   in->max_len_bound = db->max_tx_len;
+  in->n_tx = db->D;
   in->tx = tx_pairs(db, false, 0, 0, (int32_t)(db->n_rows - in->n1));
   if (in->n1) {
     in->d_frows = db->d_iota + (db->n_rows - in->n1);  // frequent rows are the suffix
@@ -766,6 +767,8 @@ fim_status estimate_impl(fim_db* db, double sample_rate, double rel_minsup, uint
       in.d_rank_item = db->d_rank_item;
       in.minsup = minsup_s;
       in.max_len_bound = db->max_tx_len;
+      in.n_tx = m;
+      in.of_sample = true;
       in.tx = tx_pairs(db, true, m, seed, 0);
       EngineConfig cfg;
       cfg.donate = 0;
@@ -801,6 +804,7 @@ fim_status estimate_impl(fim_db* db, double sample_rate, double rel_minsup, uint
       db->d_est_order = d_order;
       db->est_pending = true;
       db->est_redo = false;
+      db->est_lev_rel = ep.levels ? ep.rel : 0.0;
       db->has_estimate = true;
       db->est_nfs = 0;  // known once resolved
       db->est_m = m;
@@ -865,6 +869,8 @@ fim_status estimate_impl(fim_db* db, double sample_rate, double rel_minsup, uint
     in.d_rank_item = db->d_rank_item;
     in.minsup = minsup_s;
     in.max_len_bound = db->max_tx_len;
+    in.n_tx = m;
+    in.of_sample = true;
     in.tx = tx_pairs(db, true, m, seed, 0);
     if (!all_rows) in.tx.map = nullptr;  // (rows of a choice: their map is built)
     EngineConfig cfg;
@@ -951,6 +957,7 @@ fim_status est_resolve(fim_db* db) {
   // past the itemset limit: the synchronous path continues the doubling from twice this minsup (and until
   // then the first output capacity is bounded by the limit, as after a doubling)
   db->est_redo_minsup = over ? (db->est_minsup > UINT32_MAX / 2 ? UINT32_MAX : 2 * db->est_minsup) : 0u;
+  if ((h.err & DEV_ERR_SUB) && db->est_lev_rel > 0.0) note_outgrown(db, true, db->est_lev_rel, WalkRoom{});
   // (so does a search that outgrew its arenas: its count is of the part that was searched)
   db->est_doubled = over || (h.err & DEV_ERR_SUB);
   return FIM_OK;

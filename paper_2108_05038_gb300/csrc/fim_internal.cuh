@@ -199,6 +199,12 @@ struct alignas(128) DevCtrl {
 
 }  // namespace fim
 
+// What a search by levels that outgrew its arenas was (one per kind: mines of the whole database, of samples)
+struct Outgrown {
+  double rel = 0.0;              // minsup over transactions: searches at or below it outgrow them too
+  uint32_t queue = 0, words = 0;  // the caller's limits it ran under
+};
+
 struct fim_db {
   uint32_t D = 0, N = 0, n_rows = 0;
   uint32_t W32 = 0;      // ceil(D / 32): 32-bit words holding D bits
@@ -232,6 +238,10 @@ struct fim_db {
   // p99 136 and 141).
   bool served = false;
 
+  // searches by levels that outgrew their arenas (of the whole database; of samples): such a search is not tried
+  // again, since the frame passes repeat all of it (20,000 transactions of 100 items, 1.9 M itemsets: 37.6 ms a mine, 36.4
+  // without the try)
+  Outgrown outgrown[2];
   // last estimate (fim_estimate_class_costs)
   bool has_estimate = false;
   std::vector<double> est_cost;
@@ -244,6 +254,7 @@ struct fim_db {
   // a deferred estimate (no host outputs asked for): costs and order on the device (d_est_order, R rows),
   // the sample's control block, costs and order copied to est_pin behind est_done; est_pending until read
   bool est_pending = false;
+  double est_lev_rel = 0.0;  // the deferred sample was searched by levels: its minsup over its transactions
   bool est_redo = false;  // the deferred sample needs the synchronous path (itemset limit or a retry)
   uint32_t est_redo_minsup = 0;  // the sample minsup that redo starts at (0: the estimate's own)
   cudaEvent_t est_done = nullptr;
@@ -317,6 +328,8 @@ struct EngineInput {
   const uint32_t* d_rank_item = nullptr;  // row -> original item id
   uint32_t minsup = 1;
   uint32_t max_len_bound = 2;      // upper bound on the length of a frequent itemset
+  uint32_t n_tx = 0;               // transactions that the rows stand for
+  bool of_sample = false;
   // the transactions the rows stand for (n = 0: not to be used; map NULL: the rows are not consecutive, a map is built)
   TxPairs tx;
 };
@@ -490,6 +503,8 @@ struct EnginePlan {
   bool sub = false;  // small subtrees walked by proj_sub.cu
   WalkRoom walk;
   bool levels = false;  // the search a level at a time (levels.cu)
+  double rel = 0.0;     // minsup over the rows' transactions
+  bool of_sample = false;
   uint32_t lev_grid = 0;
   LevLaunch lev{};
   uint32_t *d_G = nullptr, *d_goff = nullptr, *d_tileoff = nullptr;
@@ -557,6 +572,8 @@ fim_status make_result(cudaStream_t st, const EngineOutput& eo, bool on_device, 
 fim_status engine_mine(fim_db* db, Workspace& ws, const EngineInput& in, const EngineConfig& cfg,
                        EngineOutput* out, fim_mine_stats* stats, EnginePlan* plan_out = nullptr,
                        const std::function<fim_status(EnginePlan*)>& after_pairs = {});
+// the search by levels of a mine at minsup / transactions = rel outgrew its arenas under these limits
+void note_outgrown(fim_db* db, bool of_sample, double rel, const WalkRoom& walk);
 void engine_release_events(EnginePlan* ep);
 // pinned staging of a database (see fim_api.cu)
 fim_status stage_get(fim_db* db, size_t bytes, void** out);

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_2108_05038_gb300 import fim
+from paper_2108_05038_gb300 import fim, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -135,6 +135,48 @@ def test_search_past_the_arenas_and_limits():
         assert db.mine(D, max_itemsets=511).n_sets == 511
         with pytest.raises(fim.FimError):
             db.mine(D, max_itemsets=510)
+    finally:
+        db.free()
+
+
+def test_outgrown_search_is_not_tried_again():
+    """A search by levels that outgrew its arenas is repeated by the frame passes once; further mines of the database at that
+    minsup, and samples at theirs, take the frame passes at once, and mines that fit the levels again."""
+    off, items = synth.dense_bernoulli(3, 20_000, 100)
+    db = fim.build_vertical_db(off, items, 100)
+
+    def launches(call):
+        c = fim.kernel_launches()
+        r = call()
+        return fim.kernel_launches() - c, r
+
+    try:
+        mine = lambda ms: db.mine(ms, result_on_device=True).n_sets  # noqa: E731
+        low, n = launches(lambda: mine(7_600))
+        again, n2 = launches(lambda: mine(7_600))
+        below, n3 = launches(lambda: mine(7_500))
+        frames, n4 = launches(lambda: db.mine(7_600, result_on_device=True, dfs_mode=fim.FIM_DFS_FRAMES).n_sets)
+        assert n == n2 == n4 < n3
+        assert again < low and again == frames and below == frames
+        high, n5 = launches(lambda: mine(9_000))
+        assert n5 == db.mine(9_000, dfs_mode=fim.FIM_DFS_FRAMES, result_on_device=True).n_sets
+        first, e1 = launches(lambda: db.estimate_class_costs(1.0, 0.38, 5, max_sample_itemsets=0))
+        second, e2 = launches(lambda: db.estimate_class_costs(1.0, 0.38, 5, max_sample_itemsets=0))
+        assert second < first
+        db.estimate_class_costs(1.0, 0.37, 5, max_sample_itemsets=0, outputs=False)  # (deferred)
+        third, e3 = launches(db.estimate_result)
+        assert third == 0
+        for a, b in zip(e1, e2):
+            assert np.array_equal(a, b)
+    finally:
+        db.free()
+    db = fim.build_vertical_db(off, items, 100)
+    try:  # the first deferred sample of a database: completed once, by the frame passes
+        db.estimate_class_costs(1.0, 0.38, 5, max_sample_itemsets=0, outputs=False)
+        redo, e4 = launches(db.estimate_result)
+        assert 0 < redo <= second
+        for a, b in zip(e1, e4):
+            assert np.array_equal(a, b)
     finally:
         db.free()
 
