@@ -391,8 +391,8 @@ void fim_plan_free(fim_plan* plan);
  * concurrent jobs share the SMs; max_itemsets (0 = none) stops a job whose
  * output grows past it (FIM_ERR_OUTPUT_OVERFLOW from fim_server_wait).  fim_server_submit copies the host CSR
  * database (as fim_build_vertical_db) and queues the job: to the device while the budget has room for the job
- * (its footprint is then in use from the submission on), else to host memory; jobs are admitted
- * in arrival order when a slot is free and their footprint fits the budget
+ * (its footprint is then in use from the submission on), else to host memory; jobs whose copy is complete are
+ * admitted in arrival order when a slot is free and their footprint fits the budget
  * left (a job larger than the budget runs alone), then run build (prefilter =
  * minsup), the sample estimate when sample_rate > 0, and the mine; the
  * database stays resident on the device until the result is copied out.

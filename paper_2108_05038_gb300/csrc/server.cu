@@ -133,17 +133,18 @@ void worker_main(fim_server* srv, size_t slot) {
     Job* j = nullptr;
     {
       std::unique_lock<std::mutex> lock(srv->mu);
+      std::deque<Job*>::iterator next;
       srv->cv_work.wait(lock, [&] {
         if (srv->stop) return true;
-        if (srv->queue.empty()) return false;
-        const Job* h = srv->queue.front();
-        if (!h->ready) return false;
-        return h->reserved || srv->in_flight == 0 || srv->in_use + h->footprint <= srv->budget;
+        // the first job whose database has been copied (one whose submitter is still at it holds nobody up).  A job larger
+        // than the budget runs alone: with no other in flight, nor one that has its room already
+        next = std::find_if(srv->queue.begin(), srv->queue.end(), [](const Job* q) { return q->ready; });
+        if (next == srv->queue.end()) return false;
+        return (*next)->reserved || srv->in_use == 0 || srv->in_use + (*next)->footprint <= srv->budget;
       });
-      if (srv->stop && srv->queue.empty()) return;
       if (srv->stop) return;
-      j = srv->queue.front();
-      srv->queue.pop_front();
+      j = *next;
+      srv->queue.erase(next);
       if (!j->reserved) srv->in_use += j->footprint;
       srv->in_flight += 1;
       srv->peak_in_flight = std::max(srv->peak_in_flight, srv->in_flight);
@@ -304,9 +305,7 @@ fim_status fim_server_submit(fim_server* srv, const uint32_t* tx_offsets, const 
   }
   {
     std::lock_guard<std::mutex> lock(srv->mu);
-    if (up && !on_device) {
-      j->reserved = false;
-      srv->in_use -= j->footprint;
+    if (up && !on_device) {  // (it keeps its room in the budget)
       srv->uploaded -= j->csr_bytes;
       j->csr_bytes = 0;
     }

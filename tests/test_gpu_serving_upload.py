@@ -1,5 +1,8 @@
 """Submitted databases on their way to the device: uploaded by the submitter while the budget has room, copied on the host
 behind a job that waits for room or with offsets that the build refuses; the caller's arrays are free after the call."""
+import threading
+import time
+
 import numpy as np
 import pytest
 
@@ -37,6 +40,38 @@ def test_results_with_arrays_reused_after_submit(budget):
         st = srv.stats()
         assert st["in_use_bytes"] == 0 and st["queued"] == 0 and st["in_flight"] == 0
         assert st["peak_in_flight"] == 1 or budget == 0
+    finally:
+        srv.free()
+
+
+def test_a_long_copy_holds_up_no_other_job():
+    """While one thread's large database is copied on the host (no budget for an upload), another's small job, submitted
+    after it, is mined and returned."""
+    D, per = 15_000_000, 20
+    off = (np.arange(D + 1, dtype=np.int64) * per).astype(np.uint32)
+    items = (np.arange(D * per, dtype=np.uint32)) % 1_000
+    small = requests(1)[0]
+    want = odict(oracle.eclat(*small))
+    srv = fim.Server(hbm_budget_bytes=1, slots=2)
+    try:
+        srv.wait(srv.submit(*small))  # (the first job of a server allocates)
+        big = {}
+
+        def submit_big():
+            big["id"] = srv.submit(off, items, 1_000, D)  # (no frequent item)
+            big["submitted"] = time.perf_counter()
+
+        t = threading.Thread(target=submit_big)
+        t.start()
+        while srv.stats()["queued"] == 0 and t.is_alive():
+            time.sleep(0.0005)
+        res = srv.wait(srv.submit(*small))[0]
+        done = time.perf_counter()
+        assert res.as_dict() == want
+        t.join()
+        assert done < big["submitted"]
+        assert srv.wait(big["id"])[0].n_sets == 0
+        assert srv.stats()["in_use_bytes"] == 0
     finally:
         srv.free()
 
