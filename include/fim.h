@@ -349,7 +349,7 @@ fim_status fim_result_view(const fim_result* res, uint64_t* n_sets, const uint64
 /*
  * Launch-shape autotuner for the persistent DFS kernel (CTA size, 16-byte
  * loads per lane, CTAs per SM, donation, traversal mode).  Mines db at minsup_abs once per
- * candidate shape (twice, best time of the kernels by CUDA events), writes
+ * candidate shape, the automatic traversal among them (twice, best time of the kernels by CUDA events), writes
  * the fastest shape into opts (threads_per_cta, vec_per_lane, ctas_per_sm,
  * donate, dfs_mode) and its time into *best_ms (may be NULL).  Results are cached per
  * (row stride, frequent items, minsup, rows).  The output of a mine never

@@ -38,7 +38,10 @@ namespace {
 struct Shape {
   uint32_t threads, vec, cps, donate, mode;
 };
+// The automatic traversal comes first: without it a tuned mine of fewer than 1,024 rows could not take the search by
+// levels, nor one of more the small-subtree walk (dense_deep replays: 122 us by levels, 158 in frame passes).
 const Shape kShapes[] = {
+    {0, 0, 0, 0, FIM_DFS_AUTO},
     {128, 2, 0, 0, 0}, {128, 4, 0, 0, 0}, {256, 2, 0, 0, 0}, {256, 4, 0, 0, 0}, {256, 8, 0, 0, 0},
     {512, 4, 0, 0, 0}, {512, 8, 0, 0, 0}, {256, 4, 0, 1, 0}, {512, 4, 0, 1, 0},
     {512, 2, 0, 0, 0}, {128, 2, 0, 0, 1}, {128, 4, 0, 0, 1}, {256, 2, 0, 0, 1}, {256, 4, 0, 0, 1},
@@ -112,8 +115,9 @@ fim_status fim_autotune(fim_db* db, uint32_t minsup_abs, fim_mine_opts* opts, fl
     c.mode = sh.mode;
     c.collect_times = true;
     float t = 1e30f;
+    fim_mine_stats st{};
     for (int rep = 0; rep < 2; ++rep) {
-      fim_mine_stats st{};
+      st = {};
       EngineOutput eo;
       FIM_TRY(engine_mine(db, db->ws, in, c, &eo, &st));
       t = std::min(t, st.ms_device_total);
@@ -121,6 +125,10 @@ fim_status fim_autotune(fim_db* db, uint32_t minsup_abs, fim_mine_opts* opts, fl
     if (t < best_t) {
       best_t = t;
       best = sh;
+      if (!best.threads) {  // what the automatic choice ran with
+        best.threads = st.threads_per_cta;
+        best.vec = st.vec_per_lane;
+      }
     }
   }
   {

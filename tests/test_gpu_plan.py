@@ -72,6 +72,21 @@ def test_autotune_shape_is_valid_and_output_unchanged():
     db.free()
 
 
+def test_autotune_times_the_automatic_traversal_too():
+    """On a dense database of few rows the search by levels, which only the automatic choice takes, is the fastest."""
+    w = synth.make_workload("dense_deep", D=50_000)
+    ms = synth.abs_minsup(w["rel_minsup"], 50_000)
+    db = fim.build_vertical_db(w["offsets"], w["items"], w["N"])
+    try:
+        shape, best_ms = db.autotune(ms)
+        auto = min(db.mine(ms, collect_times=True).stats["ms_device_total"] for _ in range(5))
+        frames = min(db.mine(ms, collect_times=True, dfs_mode=fim.FIM_DFS_FRAMES).stats["ms_device_total"] for _ in range(5))
+        assert auto < frames
+        assert shape["dfs_mode"] == fim.FIM_DFS_AUTO and best_ms < frames
+    finally:
+        db.free()
+
+
 @pytest.mark.parametrize("mode", [None, fim.FIM_DFS_PROJECTED])
 def test_replay_without_room_is_repeated(mode):
     """Replays whose search by levels, or small-subtree walk, has no room (the sizing run has it): the first result comes
