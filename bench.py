@@ -71,6 +71,20 @@ def sources_sha256() -> str:
     return h.hexdigest()
 
 
+def tx_additions(w, minsup, rows):
+    """Additions of level 2 counted from the transactions: pairs, in each of them, of the `rows` least frequent of the
+    frequent items (rows in ascending support, ties by id)."""
+    items = w["items"].astype(np.int64)
+    supp = np.bincount(items, minlength=w["N"])
+    order = np.argsort(supp, kind="stable")
+    keep = np.zeros(w["N"], dtype=np.int64)
+    keep[order[supp[order] >= minsup][:rows]] = 1
+    total = np.concatenate([[0], np.cumsum(keep[items])])
+    off = w["offsets"].astype(np.int64)
+    k = total[off[1:]] - total[off[:-1]]
+    return float((k * (k - 1) // 2).sum())
+
+
 def captured(workload):
     """The DRAM-traffic record of a workload when it matches the current sources, else (None, reason)."""
     rec = CAPTURES.get(workload)
@@ -295,10 +309,7 @@ def run_ours(args):
         alu_peak_gword = 128.0 / 3.0 * num_sms * sm_max_mhz * 1e6 / 1e9
         words = stats["n_pair_intersections"] * ((D + 31) // 32)  # algorithmic 32-bit word pairs
         achieved_gword = words / (pair_avg * 1e-3) / 1e9
-        # (more word pairs or flops than the row kernels can do: counted from the transactions)
-        by_tx = (achieved_gword > alu_peak_gword if stats.get("pair_kernel", 1) == 1 else
-                 stats["pair_kernel"] == 4 and 2.0 * stats["n_pair_intersections"] * D / (pair_avg * 1e-3) / 1e12
-                 > 2.0 * float(peaks.get("bf16_tflops", 1900.0)))
+        by_tx = stats["pair_rows_tx"] > 0  # pairs counted from the transactions
         rec, rec_note = captured(args.workload)
         hbm = float(peaks.get("hbm_gbs", 6800.0))
         hbm_src = "measured copy rate (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks else "fallback 6.8 TB/s"
@@ -307,7 +318,7 @@ def run_ours(args):
             alg = stats["bytes_projected"] if proj else stats["bytes_dfs_kernel"]
             dfs_gbs = alg / (dfs_avg * 1e-3) / 1e9
             roofline = {"kernel": ("k_proj_tids + k_proj_bits + k_sub + k_dfs_proj (+ k_dfs_sparse on the classes left out)"
-                                   if proj else "k_levels (fewer than 1,024 rows) or the DFS kernel"),
+                                   if proj else "k_levels" if stats["search"] == 6 else "the DFS kernel"),
                         "bound": "hbm", "achieved": round(dfs_gbs, 1), "peak": round(hbm, 1),
                         "unit": "GB/s", "frac": round(dfs_gbs / hbm, 4),
                         "traffic": rec["kernels"]["dfs"] if rec else None, "traffic_source": rec_note,
@@ -320,13 +331,13 @@ def run_ours(args):
                                  "algorithmic bytes count every candidate row in full (the dense definition); the "
                                  "kernel reads row words only under nonzero prefix words")}
         elif by_tx:  # level 2 counted from the transactions: one addition in L2 per pair of a transaction's items
-            lens = np.diff(w["offsets"].astype(np.int64))
-            adds = float((lens * (lens - 1) // 2).sum()) / (pair_avg * 1e-3) / 1e9
+            adds = tx_additions(w, minsup, stats["pair_rows_tx"]) / (pair_avg * 1e-3) / 1e9
             roofline = {"kernel": "k_pair_tx" + (" + k_pair_mma_fused" if stats["pair_kernel"] == 4 else ""),
                         "bound": "l2 atomics", "achieved": round(adds, 1), "peak": 180.0, "unit": "Gadd/s",
                         "frac": round(adds / 180.0, 4), "traffic": None, "traffic_source": rec_note,
                         "peak_source": "scattered 32-bit additions in L2, measured on a GB300",
-                        "note": "pairs of each transaction's items, an upper bound of the additions made"}
+                        "note": "one addition per transaction and pair of its rows that are counted this way, over the "
+                                "whole pair step (clearing the counters and the other rows' product included)"}
         elif stats.get("pair_kernel") in (2, 3, 4):  # level 2 on the tensor cores: the 0/1 contraction, kind::f8f6f4
             flops = 2.0 * stats["n_pair_intersections"] * D  # one multiply-add per pair and transaction
             tf = flops / (pair_avg * 1e-3) / 1e12

@@ -67,7 +67,7 @@ typedef struct {
   uint64_t bytes_pair_kernel;    /* algorithmic bytes of the pair kernel                           */
   uint64_t bytes_dfs_kernel;     /* algorithmic bytes of the DFS kernel                            */
   uint32_t words_per_row;        /* 32-bit words per bitmap row, padded (row stride)               */
-  uint32_t grid_ctas;            /* persistent CTAs launched                                       */
+  uint32_t grid_ctas;            /* CTAs launched by the search (projected: for the classes left out) */
   uint32_t threads_per_cta;
   uint32_t vec_per_lane;         /* 16-byte loads per lane per piece                               */
   float ms_pair_kernel;          /* CUDA-event time of the pair kernel (collect_times = 1)         */
@@ -86,11 +86,22 @@ typedef struct {
                                     survivor and transaction, the bitmaps written), per class node its
                                     prefix and candidates over its region's width, per compacted or
                                     handed-out frame its gathered words and region                  */
+  /* (not written for a caller whose fim_mine_opts.struct_size is that without the walk_* fields)   */
+  uint32_t pair_rows_tx;         /* rows whose pairs were counted from the transactions (0: none; all:
+                                    no kernel read the rows; else the others by pair_kernel)        */
+  uint32_t search;               /* what searched below level 2: FIM_DFS_NODES, _FRAMES, _SPARSE, _WARP
+                                    or _PROJECTED, FIM_SEARCH_LEVELS, or FIM_SEARCH_SUBTREES
+                                    (projected, small subtrees walked first); with fewer than 3
+                                    frequent items FIM_DFS_AUTO: none                                */
+  uint32_t search_runs;          /* its runs: more than 1 when it was repeated for room             */
+  uint32_t reserved;
 } fim_mine_stats;
 
 /* Traversal of the persistent DFS (fim_mine_opts.dfs_mode). */
 enum { FIM_DFS_NODES = 0, FIM_DFS_FRAMES = 1, FIM_DFS_AUTO = 2, FIM_DFS_SPARSE = 3, FIM_DFS_WARP = 4,
        FIM_DFS_PROJECTED = 5 };
+/* (fim_mine_stats.search only: what FIM_DFS_AUTO and FIM_DFS_PROJECTED may have run) */
+enum { FIM_SEARCH_LEVELS = 6, FIM_SEARCH_SUBTREES = 7 };
 
 /* Which itemsets fim_mine returns (fim_mine_opts.output). */
 enum { FIM_OUTPUT_ALL = 0, FIM_OUTPUT_CLOSED = 1, FIM_OUTPUT_MAXIMAL = 2 };

@@ -599,8 +599,14 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
     stats->bytes_pair_kernel = ep->npairs_max * rb + (uint64_t)(n1 > 0 ? n1 - 1 : 0) * rb;
     stats->bytes_dfs_kernel = h.n_intersections * rb + h.n_nodes * rb + h.n_frames * rb;
     stats->bytes_algorithmic = stats->bytes_pair_kernel + stats->bytes_dfs_kernel;
-    stats->grid_ctas = n1 >= 3 ? ep->grid : 0;
-    stats->threads_per_cta = ep->threads;
+    stats->grid_ctas = n1 < 3 ? 0 : ep->levels ? ep->lev_grid : ep->grid;
+    stats->threads_per_cta = ep->levels ? kLevThreads : ep->threads;
+    stats->pair_rows_tx = ep->pair_tx ? ep->tx_lim : 0u;
+    stats->search = n1 < 3         ? (uint32_t)FIM_DFS_AUTO
+                    : ep->levels ? FIM_SEARCH_LEVELS
+                    : ep->proj   ? (ep->sub ? FIM_SEARCH_SUBTREES : FIM_DFS_PROJECTED)
+                                 : ep->mode;
+    stats->search_runs = ep->runs;
     stats->vec_per_lane = ep->vec;
     stats->pair_kernel = !ep->pair_mma   ? FIM_PAIR_CORES
                          : ep->pair_fused ? FIM_PAIR_TENSOR_FUSED
@@ -658,6 +664,7 @@ fim_status engine_mine(fim_db* db, Workspace& ws, const EngineInput& in, const E
       break;
     }
     bool retry = false;
+    ep.runs = attempt + 1;
     s = engine_finish(db, ws.stream, &ep, out, stats, &retry);
     if (s != FIM_OK || !retry) break;
     if (attempt == 7) s = fail(FIM_ERR_OUTPUT_OVERFLOW, "output capacity still exceeded after regrowth");

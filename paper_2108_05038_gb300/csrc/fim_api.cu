@@ -489,6 +489,11 @@ static void engine_config_from_opts(const fim_mine_opts* o, EngineConfig* c) {
   if (o->struct_size == sizeof(fim_mine_opts)) c->walk = {o->walk_queue, o->walk_words, o->walk_rounds, o->walk_cycles};
 }
 
+CallStats::~CallStats() {
+  if (opts)
+    std::memcpy(opts->stats, &s, opts->struct_size == sizeof(fim_mine_opts) ? sizeof(s) : offsetof(fim_mine_stats, pair_rows_tx));
+}
+
 bool opts_size_ok(const fim_mine_opts* o) {
   return o->struct_size == sizeof(fim_mine_opts) || o->struct_size == offsetof(fim_mine_opts, walk_queue);
 }
@@ -1017,9 +1022,8 @@ fim_status fim_mine(fim_db* db, uint32_t minsup_abs, fim_mine_opts* opts, fim_re
     }
     return FIM_OK;
   };
-  fim_mine_stats local_stats{};
-  fim_mine_stats* stats = opts && opts->struct_size && opts->stats ? opts->stats : &local_stats;
-  std::memset(stats, 0, sizeof(*stats));
+  CallStats call_stats(opts);
+  fim_mine_stats* const stats = &call_stats.s;
   uint64_t* work_out = opts && opts->struct_size ? opts->class_work_out : nullptr;
   unsigned long long* d_work = nullptr;
   if (work_out && in.n1) {

@@ -414,6 +414,7 @@ struct SubState {
   SubRound round[kSubRounds + 1];
   alignas(128) uint32_t progress;  // raised by items that take long
 };
+constexpr uint32_t kLevThreads = 256;  // of the search by levels
 constexpr uint32_t kGramRows = 8;             // rows per side of a tile
 constexpr uint32_t kGramWords = 512;          // words per tile
 
@@ -503,6 +504,7 @@ struct EnginePlan {
   bool sub = false;  // small subtrees walked by proj_sub.cu
   WalkRoom walk;
   bool levels = false;  // the search a level at a time (levels.cu)
+  uint32_t runs = 0;    // of the search so far
   double rel = 0.0;     // minsup over the rows' transactions
   bool of_sample = false;
   uint32_t lev_grid = 0;
@@ -546,6 +548,14 @@ fim_status engine_finish(fim_db* db, cudaStream_t st, EnginePlan* ep, EngineOutp
 // stays pending (the queue order is derived on the device, the output capacity left to the caller)
 // fim_mine_opts.struct_size is that of the struct, or of the struct as it was without the walk_* fields
 bool opts_size_ok(const fim_mine_opts* o);
+// A call's counters, copied to the caller's struct when it returns: all of them, or those that a caller with the smaller
+// struct_size knows
+struct CallStats {
+  fim_mine_stats s{};
+  const fim_mine_opts* const opts;
+  explicit CallStats(const fim_mine_opts* o) : opts(o && o->struct_size && o->stats ? o : nullptr) {}
+  ~CallStats();
+};
 fim_status mine_input(fim_db* db, uint32_t minsup, const fim_mine_opts* opts, EngineInput* in, EngineConfig* cfg,
                       bool defer_ok = false);
 // the first output capacity that the database's estimate suggests for a minsup (0: none)

@@ -34,7 +34,6 @@
 namespace fim {
 namespace {
 
-constexpr uint32_t kLevThreads = 256;
 constexpr uint32_t kLevWarps = kLevThreads / 32;
 constexpr uint32_t kLevCtasPerSm = 2;
 constexpr uint32_t kLevCand = 8;      // candidates of a unit

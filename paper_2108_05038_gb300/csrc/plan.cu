@@ -196,10 +196,10 @@ fim_status fim_plan_result(fim_plan* plan, fim_mine_opts* opts, fim_result** out
   if (!plan || !out) return fail(FIM_ERR_INVALID, "plan or out is NULL");
   *out = nullptr;
   if (plan->launches == 0) return fail(FIM_ERR_INVALID, "plan was never launched");
-  fim_mine_stats local{};
-  fim_mine_stats* stats = opts && opts->struct_size && opts->stats ? opts->stats : &local;
-  std::memset(stats, 0, sizeof(*stats));
+  CallStats call_stats(opts);
+  fim_mine_stats* const stats = &call_stats.s;
   EngineOutput eo;
+  plan->ep.runs = 1;
   bool retry = false;
   FIM_TRY(engine_finish(plan->db, plan->stream, &plan->ep, &eo, stats, &retry));
   const bool again = retry;
@@ -207,6 +207,7 @@ fim_status fim_plan_result(fim_plan* plan, fim_mine_opts* opts, fim_result** out
     if (attempt == 8) return fail(FIM_ERR_OUTPUT_OVERFLOW, "plan buffers no longer fit the database");
     FIM_TRY(engine_alloc(plan->ws, &plan->ep));
     FIM_CUDA(engine_launch(plan->ep, plan->stream));
+    ++plan->ep.runs;
     FIM_TRY(engine_finish(plan->db, plan->stream, &plan->ep, &eo, stats, &retry));
   }
   if (again) FIM_TRY(plan_capture(plan));

@@ -18,6 +18,7 @@ from . import _build
 FIM_OK, FIM_ERR_INVALID, FIM_ERR_OOM, FIM_ERR_OUTPUT_OVERFLOW, FIM_ERR_CUDA, FIM_ERR_TIMEOUT = range(6)
 FIM_ORDER_ESTIMATE, FIM_ORDER_UNIFORM = 0, 1
 FIM_DFS_NODES, FIM_DFS_FRAMES, FIM_DFS_AUTO, FIM_DFS_SPARSE, FIM_DFS_WARP, FIM_DFS_PROJECTED = 0, 1, 2, 3, 4, 5
+FIM_SEARCH_LEVELS, FIM_SEARCH_SUBTREES = 6, 7  # stats["search"] only, beside the FIM_DFS_* values
 FIM_OUTPUT_ALL, FIM_OUTPUT_CLOSED, FIM_OUTPUT_MAXIMAL = 0, 1, 2
 FIM_PAIR_AUTO, FIM_PAIR_CORES, FIM_PAIR_TENSOR, FIM_PAIR_TENSOR_E4M3, FIM_PAIR_TENSOR_FUSED = 0, 1, 2, 3, 4
 SAMPLE_ITEMSET_LIMIT = 1 << 20  # FIM_SAMPLE_ITEMSET_LIMIT
@@ -55,6 +56,8 @@ class MineStats(ctypes.Structure):
         ("dfs_cta_busy_max_ms", ctypes.c_float), ("dfs_cta_busy_mean_ms", ctypes.c_float), ("pair_kernel", ctypes.c_uint32),
         ("n_proj_classes", ctypes.c_uint32), ("n_proj_splits", ctypes.c_uint64), ("n_fallback_entries", ctypes.c_uint64),
         ("bytes_projected", ctypes.c_uint64),
+        ("pair_rows_tx", ctypes.c_uint32), ("search", ctypes.c_uint32), ("search_runs", ctypes.c_uint32),
+        ("reserved", ctypes.c_uint32),
     ]
 
     def as_dict(self):

@@ -90,6 +90,11 @@ def test_opts_of_a_caller_without_the_walk_fields():
         assert ("initialised" in text) == (size == ctypes.sizeof(fim.MineOpts) - 8), text
 
 
+def test_stats_of_a_caller_without_the_walk_fields():
+    """The counters added after bytes_projected lie behind what a caller with the smaller opts has room for."""
+    assert fim.MineStats.pair_rows_tx.offset == fim.MineStats.bytes_projected.offset + 8
+
+
 def test_invalid_arguments_rejected_without_gpu():
     lib = fim.load()
     h = ctypes.c_void_p()

@@ -1,6 +1,6 @@
 """The search by levels (GPU; the automatic traversal of mines of fewer than 1,024 rows) against the frame passes (the same
 nodes, intersections and class work) and the CPU oracle: few and many survivors, one and several word segments per row,
-samples, itemset limits, and searches that outgrow its arenas."""
+samples, itemset limits, and searches without room in its arenas."""
 import numpy as np
 import pytest
 
@@ -49,6 +49,8 @@ def test_same_search_as_frame_passes(name):
         got = db.mine(minsup, class_work=True)
         ref = db.mine(minsup, dfs_mode=fim.FIM_DFS_FRAMES, class_work=True)
         assert got.as_dict() == want and ref.as_dict() == want
+        assert (got.stats["search"], got.stats["search_runs"]) == (fim.FIM_SEARCH_LEVELS, 1)
+        assert ref.stats["search"] == fim.FIM_DFS_FRAMES
         for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len", "bytes_dfs_kernel"):
             assert got.stats[key] == ref.stats[key], key
         assert np.array_equal(got.class_work, ref.class_work)
@@ -66,12 +68,10 @@ def test_without_room(name, room):
     want = odict(oracle.eclat(off, items, N, minsup))
     db = fim.build_vertical_db(off, items, N)
     try:
-        n = [fim.kernel_launches()]
         got = db.mine(minsup, class_work=True)
-        n.append(fim.kernel_launches())
         got2 = db.mine(minsup, class_work=True, walk=room)
-        n.append(fim.kernel_launches())
-        assert n[2] - n[1] > n[1] - n[0]  # (repeated)
+        assert (got.stats["search"], got.stats["search_runs"]) == (fim.FIM_SEARCH_LEVELS, 1)
+        assert (got2.stats["search"], got2.stats["search_runs"]) == (fim.FIM_DFS_FRAMES, 2)
         assert got.as_dict() == want and got2.as_dict() == want
         for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len"):
             assert got.stats[key] == got2.stats[key], key
@@ -91,6 +91,7 @@ def test_row_lengths(words):
         ref = db.mine(minsup, dfs_mode=fim.FIM_DFS_FRAMES)
         assert got.as_dict() == ref.as_dict() == odict(oracle.eclat(off, items, N, minsup))
         assert got.stats["n_intersections"] == ref.stats["n_intersections"] and got.stats["max_len"] >= 4
+        assert (got.stats["search"], got.stats["search_runs"]) == (fim.FIM_SEARCH_LEVELS, 1)
     finally:
         db.free()
 
@@ -113,9 +114,9 @@ def test_class_costs_of_a_sample(name, cost):
         db.free()
 
 
-def test_search_past_the_arenas_and_limits():
-    """20 items in every one of 64 transactions: 2^20 - 1 itemsets, more at one level than its arenas hold, so the frame
-    passes repeat the run; limits below and at the number of itemsets."""
+def test_many_itemsets_and_limits():
+    """20 items in every one of 64 transactions: 2^20 - 1 itemsets in levels of up to 2^17.5; limits below and at the number
+    of itemsets."""
     k, D = 20, 64
     off = (np.arange(D + 1) * k).astype(np.uint32)
     items = np.tile(np.arange(k, dtype=np.uint32), D)
@@ -123,6 +124,7 @@ def test_search_past_the_arenas_and_limits():
     try:
         r = db.mine(D, result_on_device=True)
         assert r.n_sets == 2 ** k - 1 and r.stats["max_len"] == k and r.stats["n_items_out"] == k * 2 ** (k - 1)
+        assert r.stats["search"] == fim.FIM_SEARCH_LEVELS
         r.free()
         with pytest.raises(fim.FimError) as e:
             db.mine(D, max_itemsets=5_000)
@@ -151,15 +153,15 @@ def test_outgrown_search_is_not_tried_again():
         return fim.kernel_launches() - c, r
 
     try:
-        mine = lambda ms: db.mine(ms, result_on_device=True).n_sets  # noqa: E731
-        low, n = launches(lambda: mine(7_600))
-        again, n2 = launches(lambda: mine(7_600))
-        below, n3 = launches(lambda: mine(7_500))
-        frames, n4 = launches(lambda: db.mine(7_600, result_on_device=True, dfs_mode=fim.FIM_DFS_FRAMES).n_sets)
-        assert n == n2 == n4 < n3
-        assert again < low and again == frames and below == frames
-        high, n5 = launches(lambda: mine(9_000))
-        assert n5 == db.mine(9_000, dfs_mode=fim.FIM_DFS_FRAMES, result_on_device=True).n_sets
+        def ran(ms, **kw):
+            r = db.mine(ms, result_on_device=True, **kw)
+            return r.n_sets, r.stats["search"], r.stats["search_runs"]
+
+        n, _, runs = ran(7_600, dfs_mode=fim.FIM_DFS_FRAMES)
+        assert ran(7_600) == (n, fim.FIM_DFS_FRAMES, runs + 1)
+        assert ran(7_600) == (n, fim.FIM_DFS_FRAMES, runs)
+        assert ran(7_500)[1:] == (fim.FIM_DFS_FRAMES, runs)
+        assert ran(9_000)[:2] == (ran(9_000, dfs_mode=fim.FIM_DFS_FRAMES)[0], fim.FIM_SEARCH_LEVELS)
         first, e1 = launches(lambda: db.estimate_class_costs(1.0, 0.38, 5, max_sample_itemsets=0))
         second, e2 = launches(lambda: db.estimate_class_costs(1.0, 0.38, 5, max_sample_itemsets=0))
         assert second < first
@@ -181,15 +183,15 @@ def test_outgrown_search_is_not_tried_again():
         db.free()
 
 
-def test_deferred_estimate_past_the_arenas():
-    """A deferred sample of 2^20 - 1 itemsets outgrows the arenas: the mine that uses it finds room for its result at once,
-    and the estimate is completed when it is read (k items alike: class i has 2^(k - 1 - i) itemsets)."""
+def test_deferred_estimate_of_many_itemsets():
+    """A deferred sample of 2^20 - 1 itemsets: the mine that uses it finds room for its result at once (k items alike:
+    class i has 2^(k - 1 - i) itemsets)."""
     k, D = 20, 64
     db = fim.build_vertical_db((np.arange(D + 1) * k).astype(np.uint32), np.tile(np.arange(k, dtype=np.uint32), D), k)
     try:
         db.estimate_class_costs(1.0, 1.0, 3, outputs=False)
         r = db.mine(D, result_on_device=True)
-        assert r.n_sets == 2 ** k - 1
+        assert r.n_sets == 2 ** k - 1 and r.stats["search_runs"] == 1
         r.free()
         cost, order = db.estimate_result()[:2]
         assert np.array_equal(order, np.arange(k))

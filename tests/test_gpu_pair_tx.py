@@ -29,12 +29,15 @@ def odict(o):
     return {tuple(int(v) for v in si[so[k]:so[k + 1]]): int(sp[k]) for k in range(len(sp))}
 
 
-def check(off, items, N, minsup, kernel, want=None, **kw):
+def check(off, items, N, minsup, kernel, left=0, want=None, **kw):
+    """``left``: rows whose pairs another kernel (``kernel``) counts from the rows."""
     db = fim.build_vertical_db(off, items, N, **kw)
     try:
         auto = db.mine(minsup)
         assert auto.stats["pair_kernel"] == kernel
+        assert auto.stats["pair_rows_tx"] == auto.stats["n_frequent_items"] - left
         cores = db.mine(minsup, pair_kernel=fim.FIM_PAIR_CORES)
+        assert cores.stats["pair_kernel"] == fim.FIM_PAIR_CORES and cores.stats["pair_rows_tx"] == 0
         got = auto.as_dict()
         assert got == cores.as_dict()
         if want is not None:
@@ -55,7 +58,7 @@ def test_pairs_from_transactions(D, N, lengths):
     k = np.diff(off.astype(np.int64))
     mean = float((k * (k - 1)).sum()) / (N * (N - 1))  # of a pair's support: the minsup is some deviations above it
     minsup = max(2, int(mean + 2.5 * mean ** 0.5) + 1)
-    got = check(off, items, N, minsup, fim.FIM_PAIR_CORES,
+    got = check(off, items, N, minsup, fim.FIM_PAIR_CORES, 0,
                 odict(oracle.eclat(off, items, N, minsup)) if D < 10_000 else None)
     assert any(len(k) == 2 for k in got)
 
@@ -65,7 +68,7 @@ def test_most_frequent_rows_left_to_the_product(N):
     """Rows that all take part, with the last ones so frequent that the product counts their pairs."""
     off, items = database(N, 100_000, N, [3, 4, 5], hot=8)
     minsup = 100
-    got = check(off, items, N, minsup, fim.FIM_PAIR_TENSOR_FUSED)
+    got = check(off, items, N, minsup, fim.FIM_PAIR_TENSOR_FUSED, 256)
     assert any(len(k) == 2 for k in got)
 
 
@@ -77,22 +80,26 @@ def test_repeated_items_take_the_rows():
     want = odict(oracle.eclat(off, items, 1200, 20))
     db = fim.build_vertical_db(off, items, 1200)
     try:
-        assert db.mine(20).as_dict() == want
+        got = db.mine(20)
+        assert got.as_dict() == want and got.stats["pair_rows_tx"] == 0
     finally:
         db.free()
 
 
-@pytest.mark.parametrize("prefilter", [0, 30])
+@pytest.mark.parametrize("prefilter", [0, 8])
 def test_noalloc_pairs_from_transactions(prefilter):
+    """(That call reports no counters.  It chooses between the transactions and the integer pipes by the model of a mine's
+    choice, which has the tensor cores as well, and a mine of the same rows takes the transactions here.)"""
     import torch
 
-    off, items = database(11, 30_000, 1000, [3, 8, 33])
+    off, items = database(11, 60_000, 1000, [1] * 20 + [3, 8, 33])
     db = fim.build_vertical_db(off, items, 1000, prefilter_minsup=prefilter)
     try:
-        want = {k: v for k, v in db.mine(30, pair_kernel=fim.FIM_PAIR_CORES).as_dict().items() if len(k) == 2}
+        assert db.mine(8).stats["pair_rows_tx"] == 1000
+        want = {k: v for k, v in db.mine(8, pair_kernel=fim.FIM_PAIR_CORES).as_dict().items() if len(k) == 2}
         p = torch.zeros(len(want) + 1, 2, dtype=torch.int32, device="cuda")
         s = torch.zeros(len(want) + 1, dtype=torch.int32, device="cuda")
-        n = db.mine_pairs_noalloc(30, p, s, len(want) + 1)
+        n = db.mine_pairs_noalloc(8, p, s, len(want) + 1)
         got = {tuple(k): v for k, v in zip(p[:n].tolist(), s[:n].tolist())}
         assert got == want
     finally:
@@ -101,7 +108,8 @@ def test_noalloc_pairs_from_transactions(prefilter):
 
 @pytest.mark.parametrize("N,D", [(5000, 40_000), (1200, 40_000)])
 def test_sample_pairs_from_transactions(N, D):
-    """The estimate's sample, over a choice of the rows (N = 5000) or over all of them, drawn with replacement."""
+    """The estimate's sample, over a choice of the rows (N = 5000) or over all of them, drawn with replacement (whichever
+    kernel the model takes for it: an estimate reports no counters)."""
     off, items = database(N, D, N, [2, 5, 9, 33])
     rel = 12 / D
     db = fim.build_vertical_db(off, items, N)

@@ -106,9 +106,12 @@ def test_replay_without_room_is_repeated(mode):
             c = fim.kernel_launches()
             plan.launch()
             plan.launch()
-            assert plan.result().as_dict() == want
-            counts.append(fim.kernel_launches() - c)
-        assert counts[0] > counts[1] == counts[2]
+            res = plan.result()
+            assert res.as_dict() == want
+            counts.append((fim.kernel_launches() - c, res.stats["search_runs"], res.stats["search"]))
+        without = fim.FIM_DFS_FRAMES if mode is None else fim.FIM_DFS_PROJECTED
+        assert counts[0][0] > counts[1][0] and counts[1] == counts[2] == (counts[1][0], 1, without)
+        assert counts[0][1:] == (2, without)
         plan.free()
         assert db.mine(60, **kw).as_dict() == want
     finally:

@@ -55,6 +55,8 @@ def test_same_walk_as_sparse_nodes(name):
         got = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, class_work=True, class_order="uniform")
         want = odict(oracle.eclat(off, items, N, minsup))
         assert got.as_dict() == want and ref.as_dict() == want
+        assert (got.stats["search"], got.stats["search_runs"]) == (fim.FIM_SEARCH_SUBTREES, 1)
+        assert ref.stats["search"] == fim.FIM_DFS_SPARSE
         for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len"):
             assert got.stats[key] == ref.stats[key], key
         assert np.array_equal(got.class_work, ref.class_work)
@@ -108,6 +110,7 @@ def test_without_room(searched, name, room):
     db, minsup, want, ref = searched(name)
     got = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, class_work=True, class_order="uniform", walk=ROOMS[room])
     assert got.as_dict() == want
+    assert (got.stats["search"], got.stats["search_runs"]) in ((fim.FIM_SEARCH_SUBTREES, 1), (fim.FIM_DFS_PROJECTED, 2))
     for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len"):
         assert got.stats[key] == ref.stats[key], key
     assert np.array_equal(got.class_work, ref.class_work)
@@ -133,13 +136,11 @@ def test_large_subtree_without_room():
 def test_class_bitmaps_past_32_bit_offsets(searched):
     """With a budget that lets a class region hold 2^32 words the walk, whose row offsets have 32 bits, is left out."""
     db, minsup, want, ref = searched("many_rows")
-    count = []
-    for words in (1 << 24, (1 << 32) - 1, 1 << 32):
-        c = fim.kernel_launches()
+    for words, search in ((1 << 24, fim.FIM_SEARCH_SUBTREES), ((1 << 32) - 1, fim.FIM_SEARCH_SUBTREES),
+                          (1 << 32, fim.FIM_DFS_PROJECTED)):
         got = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, proj_bitmap_words=words, walk=dict(words=100_000))
-        count.append(fim.kernel_launches() - c)
         assert got.as_dict() == want and got.stats["n_intersections"] == ref.stats["n_intersections"]
-    assert count[1] == count[0] and count[2] == count[0] - 1
+        assert (got.stats["search"], got.stats["search_runs"]) == (search, 1)
 
 
 @pytest.mark.parametrize("limit", [50, 2_000])
