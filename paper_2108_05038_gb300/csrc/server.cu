@@ -10,12 +10,16 @@
 // The persistent DFS of a served job exits as soon as its queue drains (no
 // idle polling), so concurrent jobs never hold SMs for one another.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <functional>
+#include <memory>
 #include <mutex>
 #include <new>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 #include <vector>
@@ -25,6 +29,87 @@
 namespace {
 
 using Clock = std::chrono::steady_clock;
+
+// Threads that share the host's part of a submission (reading its offsets, copying it) with the submitter, a piece after the
+// other.  The caller waits only for the threads that have taken a piece, not for those that are still waking up, and they
+// look out for the next call for a moment before they sleep (submissions of a burst follow one another).
+class Crew {
+ public:
+  explicit Crew(uint32_t helpers) {
+    threads_.reserve(helpers);
+    try {
+      for (uint32_t k = 0; k < helpers; ++k) threads_.emplace_back([this] { help(); });
+    } catch (const std::system_error&) {  // (fewer than asked for)
+    }
+  }
+  ~Crew() {
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      stop_ = true;
+    }
+    cv_open_.notify_all();
+    for (auto& t : threads_) t.join();
+  }
+  // f(0) .. f(n - 1) (one caller at a time; f does not throw)
+  void run(uint64_t n, const std::function<void(uint64_t)>& f) {
+    if (n <= 2 || threads_.empty()) {
+      for (uint64_t k = 0; k < n; ++k) f(k);
+      return;
+    }
+    {
+      std::lock_guard<std::mutex> lock(mu_);
+      f_ = &f;
+      n_ = n;
+      next_ = 0;
+      open_ = true;
+      ++turn_;
+    }
+    cv_open_.notify_all();
+    pieces();
+    std::unique_lock<std::mutex> lock(mu_);
+    open_ = false;
+    cv_idle_.wait(lock, [&] { return busy_ == 0; });
+  }
+  void copy(uint8_t* dst, const uint8_t* src, uint64_t bytes) {
+    constexpr uint64_t kPiece = 128 << 10;
+    run((bytes + kPiece - 1) / kPiece,
+        [=](uint64_t k) { std::memcpy(dst + k * kPiece, src + k * kPiece, std::min(kPiece, bytes - k * kPiece)); });
+  }
+
+ private:
+  static constexpr std::chrono::microseconds kLookOut{100};
+  void pieces() {
+    for (uint64_t k; (k = next_.fetch_add(1)) < n_;) (*f_)(k);
+  }
+  void help() {
+    uint64_t seen = 0;
+    std::unique_lock<std::mutex> lock(mu_);
+    for (;;) {
+      if (!stop_ && turn_ == seen) {
+        lock.unlock();
+        const auto until = Clock::now() + kLookOut;
+        while (turn_.load() == seen && Clock::now() < until) std::this_thread::yield();
+        lock.lock();
+      }
+      cv_open_.wait(lock, [&] { return stop_ || (open_ && turn_ != seen); });
+      if (stop_) return;
+      seen = turn_;
+      ++busy_;
+      lock.unlock();
+      pieces();
+      lock.lock();
+      if (--busy_ == 0) cv_idle_.notify_one();
+    }
+  }
+  std::mutex mu_;
+  std::condition_variable cv_open_, cv_idle_;
+  const std::function<void(uint64_t)>* f_ = nullptr;
+  uint64_t n_ = 0;
+  std::atomic<uint64_t> next_{0}, turn_{0};
+  uint32_t busy_ = 0;
+  bool open_ = false, stop_ = false;
+  std::vector<std::thread> threads_;
+};
 
 struct Job {
   uint64_t id = 0;
@@ -36,6 +121,7 @@ struct Job {
   bool reserved = false;   // its footprint is part of in_use (from the submission when the submitter uploads)
   void* d_csr = nullptr;   // the uploaded database: offsets, then items (csr_items bytes further); csr_bytes in all
   uint64_t csr_items = 0, csr_bytes = 0, nnz = 0;
+  cudaEvent_t ev_csr = nullptr;  // the upload's end
   Clock::time_point t_submit, t_start, t_end;
   cudaEvent_t ev_start = nullptr, ev_end = nullptr;  // the job's device work on its slot's stream
   fim_status status = FIM_OK;
@@ -65,6 +151,10 @@ struct fim_server {
   std::vector<cudaStream_t> streams;
   std::mutex up_mu;                // one upload at a time
   cudaStream_t up_stream = nullptr;
+  std::unique_ptr<Crew> crew;  // (under up_mu)
+  uint8_t* stage[2] = {};          // pinned, kStageBytes each: uploads go through them in turn
+  cudaEvent_t stage_free[2] = {};  // the buffer's last copy is done
+  uint32_t stage_turn = 0;
   cudaEvent_t ev_origin = nullptr;  // recorded at creation: device times of jobs are measured from it
 };
 
@@ -104,7 +194,9 @@ void run_job(fim_server* srv, Job* j, cudaStream_t st) {
   fim_status s;
   if (j->d_csr) {
     uint32_t* const d_off = static_cast<uint32_t*>(j->d_csr);
-    s = fim::build_uploaded_db(d_off, d_off + j->csr_items / 4, j->nnz, j->D, j->N, 64, j->minsup, st, &db);
+    const cudaError_t e = cudaStreamWaitEvent(st, j->ev_csr, 0);
+    s = e != cudaSuccess ? fim::cuda_fail(e, "waiting for the upload")
+                         : fim::build_uploaded_db(d_off, d_off + j->csr_items / 4, j->nnz, j->D, j->N, 64, j->minsup, st, &db);
   } else {
     s = fim_build_vertical_db(j->off.data(), j->items.data(), j->D, j->N, 64, j->minsup, st, &db);
   }
@@ -156,6 +248,8 @@ void worker_main(fim_server* srv, size_t slot) {
     if (cudaEventCreate(&j->ev_end) == cudaSuccess) cudaEventRecord(j->ev_end, st);
     if (j->d_csr) cudaFreeAsync(j->d_csr, st);
     j->d_csr = nullptr;
+    if (j->ev_csr) cudaEventDestroy(j->ev_csr);
+    j->ev_csr = nullptr;
     j->t_end = Clock::now();
     {
       std::lock_guard<std::mutex> lock(srv->mu);
@@ -173,9 +267,45 @@ void worker_main(fim_server* srv, size_t slot) {
   }
 }
 
-// The submitted database copied to the device by the submitting thread, complete on return (the caller may reuse its arrays
-// then).  The copy engine reads pageable memory itself here, at 150 GB/s; one thread copies it at 13 GB/s.  False, with no
-// error left behind: no memory; the host copy takes its place.
+constexpr size_t kStageBytes = 8 << 20;
+
+bool upload_create(fim_server* srv) {
+  if (cudaStreamCreateWithFlags(&srv->up_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    srv->up_stream = nullptr;
+    return false;
+  }
+  for (uint32_t b = 0; b < 2; ++b) {
+    if (cudaMallocHost(reinterpret_cast<void**>(&srv->stage[b]), kStageBytes) != cudaSuccess) return false;
+    if (cudaEventCreateWithFlags(&srv->stage_free[b], cudaEventDisableTiming) != cudaSuccess) return false;
+  }
+  try {
+    const uint32_t cores = std::thread::hardware_concurrency();
+    srv->crew.reset(new Crew(cores > 5 ? 5 : cores > 1 ? cores - 1 : 0));
+  } catch (const std::bad_alloc&) {
+    return false;
+  }
+  return true;
+}
+
+void upload_release(fim_server* srv) {
+  srv->crew.reset();
+  if (srv->up_stream) cudaStreamSynchronize(srv->up_stream);
+  for (uint32_t b = 0; b < 2; ++b) {
+    if (srv->stage[b]) cudaFreeHost(srv->stage[b]);
+    if (srv->stage_free[b]) cudaEventDestroy(srv->stage_free[b]);
+    srv->stage[b] = nullptr;
+    srv->stage_free[b] = nullptr;
+  }
+  if (srv->up_stream) cudaStreamDestroy(srv->up_stream);
+  srv->up_stream = nullptr;
+}
+
+// The submitted database copied to the device by the submitting thread through two pinned buffers that it and the crew fill
+// in turn.  On return the caller may reuse its arrays; the job's stream waits for the last buffer's copy (ev_csr).
+// The copy engine can read pageable memory itself, at 100 to 150 GB/s, but arrays that the device has not read before may
+// take it ten times as long, and a service gets new arrays with every request: bursts of 12 jobs (71 MB) took 3 to 15 ms that
+// way, through the buffers 2.5 (2.1 and 1.9 when the same arrays come again).  One thread copies 23 GB/s, four 50.
+// False, with no error left behind: no memory; the host copy takes its place.
 bool upload(fim_server* srv, Job* j, const uint32_t* off, const uint32_t* items) {
   int dev = 0;
   // (a capture that the calling thread has open is not disturbed by calls on another stream)
@@ -188,13 +318,32 @@ bool upload(fim_server* srv, Job* j, const uint32_t* off, const uint32_t* items)
     void* p = nullptr;
     e = fim::dev_malloc_async(&p, j->csr_bytes, srv->up_stream);
     if (e == cudaSuccess) {
-      e = cudaMemcpyAsync(p, off, ((size_t)j->D + 1) * 4, cudaMemcpyHostToDevice, srv->up_stream);
-      if (e == cudaSuccess && j->nnz)
-        e = cudaMemcpyAsync(static_cast<uint8_t*>(p) + j->csr_items, items, j->nnz * 4, cudaMemcpyHostToDevice, srv->up_stream);
-      const cudaError_t done = cudaStreamSynchronize(srv->up_stream);
-      if (e == cudaSuccess) e = done;
-      if (e == cudaSuccess) j->d_csr = p;
-      else cudaFreeAsync(p, srv->up_stream);
+      // the offsets and, csr_items bytes further, the items as one run of bytes
+      const uint64_t off_bytes = ((uint64_t)j->D + 1) * 4, end = j->csr_items + j->nnz * 4;
+      for (uint64_t at = 0; at < end && e == cudaSuccess;) {
+        const uint32_t b = srv->stage_turn++ & 1u;
+        const uint64_t n = std::min<uint64_t>(kStageBytes, end - at);
+        e = cudaEventSynchronize(srv->stage_free[b]);
+        if (e != cudaSuccess) break;
+        if (at < off_bytes)
+          srv->crew->copy(srv->stage[b], reinterpret_cast<const uint8_t*>(off) + at, std::min(n, off_bytes - at));
+        if (at + n > j->csr_items) {
+          const uint64_t skip = std::max(at, j->csr_items);
+          srv->crew->copy(srv->stage[b] + (skip - at), reinterpret_cast<const uint8_t*>(items) + (skip - j->csr_items),
+                          at + n - skip);
+        }
+        e = cudaMemcpyAsync(static_cast<uint8_t*>(p) + at, srv->stage[b], n, cudaMemcpyHostToDevice, srv->up_stream);
+        if (e == cudaSuccess) e = cudaEventRecord(srv->stage_free[b], srv->up_stream);
+        at += n;
+      }
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&j->ev_csr, cudaEventDisableTiming);
+      if (e == cudaSuccess) e = cudaEventRecord(j->ev_csr, srv->up_stream);
+      if (e == cudaSuccess) {
+        j->d_csr = p;
+      } else {
+        cudaStreamSynchronize(srv->up_stream);
+        cudaFreeAsync(p, srv->up_stream);
+      }
     }
   }
   if (dev != srv->device) cudaSetDevice(dev);
@@ -240,8 +389,8 @@ fim_status fim_server_create(uint64_t hbm_budget_bytes, uint32_t slots, uint32_t
     }
     srv->streams.push_back(s);
   }
-  if (cudaStreamCreateWithFlags(&srv->up_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    srv->up_stream = nullptr;  // (every submission is copied on the host)
+  if (!upload_create(srv)) {  // (every submission is copied on the host)
+    upload_release(srv);
     cudaGetLastError();
   }
   if (cudaEventCreate(&srv->ev_origin) == cudaSuccess) cudaEventRecord(srv->ev_origin, srv->streams[0]);
@@ -265,16 +414,34 @@ fim_status fim_server_submit(fim_server* srv, const uint32_t* tx_offsets, const 
   j->sample_rate = sample_rate;
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, srv->device);
-  uint32_t max_len = 0, bad = tx_offsets[0] != 0;
-  for (uint32_t t = 0; t < D; ++t) {
-    const uint32_t a = tx_offsets[t], b = tx_offsets[t + 1], n = b > a ? b - a : 0u;
-    max_len = n > max_len ? n : max_len;
-    bad |= b < a;
+  // the longest transaction, and whether the build will refuse the offsets
+  std::atomic<uint32_t> longest{0}, refused{tx_offsets[0] != 0};
+  auto scan = [&](uint32_t t0, uint32_t t1) {
+    uint32_t m = 0, r = 0;
+    for (uint32_t t = t0; t < t1; ++t) {
+      const uint32_t a = tx_offsets[t], b = tx_offsets[t + 1], n = b > a ? b - a : 0u;
+      m = n > m ? n : m;
+      r |= b < a;
+    }
+    uint32_t seen = longest.load();
+    while (m > seen && !longest.compare_exchange_weak(seen, m)) {}
+    if (r) refused = 1;
+  };
+  {
+    constexpr uint32_t kPiece = 16384;
+    std::unique_lock<std::mutex> lock(srv->up_mu, std::defer_lock);
+    if (srv->crew && D > 2 * kPiece && lock.try_lock())
+      srv->crew->run((D + kPiece - 1) / kPiece, [&](uint64_t k) {
+        scan((uint32_t)k * kPiece, (uint32_t)std::min<uint64_t>(D, (k + 1) * kPiece));
+      });
+    else
+      scan(0, D);
   }
+  const uint32_t max_len = longest, bad = refused;
   j->footprint = job_footprint(D, N, nnz, max_len, minsup_abs, (uint32_t)nsm * srv->ctas_per_sm, srv->total_mem, nsm);
   // The submitter uploads the database when the job's footprint fits the budget now and no queued job waits for room (the
-  // jobs stay in arrival order): a burst of 12 jobs with 71 MB of databases is submitted in 1,600 us, with host copies in
-  // 5,400.  Else, and for offsets that the build will refuse, it is copied on the host, outside the budget.
+  // jobs stay in arrival order).  Else, and for offsets that the build will refuse, it is copied on the host, outside the
+  // budget (a burst of 12 jobs with 71 MB: 1.8 ms to submit with uploads, 5.4 with host copies).
   j->csr_items = (((uint64_t)D + 1) * 4 + 255) & ~255ull;
   const uint64_t csr_bytes = j->csr_items + std::max<uint64_t>(1, nnz) * 4;
   bool up = srv->up_stream && !bad && (tx_items || nnz == 0);
@@ -382,12 +549,13 @@ void fim_server_free(fim_server* srv) {
   for (auto& kv : srv->jobs) {  // (the queued jobs are among them)
     if (kv.second->d_csr) cudaFreeAsync(kv.second->d_csr, srv->up_stream);  // (never started)
     if (kv.second->result) fim_result_free(kv.second->result);
+    if (kv.second->ev_csr) cudaEventDestroy(kv.second->ev_csr);
     if (kv.second->ev_start) cudaEventDestroy(kv.second->ev_start);
     if (kv.second->ev_end) cudaEventDestroy(kv.second->ev_end);
     delete kv.second;
   }
   for (auto s : srv->streams) cudaStreamDestroy(s);
-  if (srv->up_stream) cudaStreamDestroy(srv->up_stream);
+  upload_release(srv);
   if (srv->ev_origin) cudaEventDestroy(srv->ev_origin);
   delete srv;
 }

@@ -1,4 +1,4 @@
-"""Submitted databases on their way to the device: uploaded by the submitter while the budget has room, copied on the host
+"""Submitted databases on their way to the device: uploaded through pinned buffers while the budget has room, copied on the host
 behind a job that waits for room or with offsets that the build refuses; the caller's arrays are free after the call."""
 import threading
 import time
@@ -40,6 +40,25 @@ def test_results_with_arrays_reused_after_submit(budget):
         st = srv.stats()
         assert st["in_use_bytes"] == 0 and st["queued"] == 0 and st["in_flight"] == 0
         assert st["peak_in_flight"] == 1 or budget == 0
+    finally:
+        srv.free()
+
+
+@pytest.mark.parametrize("D,per", [(1, 1), (65_537, 1), (400_001, 13), (2_500_000, 7)])
+def test_databases_of_several_pieces(D, per):
+    """Uploads of one piece and of many, of sizes that end within one: the same counts as a database built directly."""
+    rng = np.random.default_rng(D)
+    off = (np.arange(D + 1) * per).astype(np.uint32)
+    items = (rng.integers(0, 30, size=(D, per)) + 30 * np.arange(per)).astype(np.uint32).reshape(-1)
+    N, minsup = 30 * per, max(1, D // 1_000)
+    db = fim.build_vertical_db(off, items, N)
+    want = db.mine(minsup).as_dict()
+    db.free()
+    srv = fim.Server(slots=2)
+    try:
+        ids = [srv.submit(off.copy(), items.copy(), N, minsup) for _ in range(3)]
+        for jid in ids:
+            assert srv.wait(jid)[0].as_dict() == want
     finally:
         srv.free()
 
