@@ -139,7 +139,8 @@ typedef struct {
                                   cap on the CTAs per SM), else, for rows of at most 16,384 words
                                   (64 KB), a level at a time over all extendable itemsets (no cap, no
                                   donation, no diffsets; a search that outgrows its lists is repeated
-                                  as FRAMES) or frames, else SPARSE;
+                                  as FRAMES, which further mines at that minsup then take at once) or
+                                  frames, else SPARSE;
                                   FIM_DFS_WARP (4): one warp
                                   per two-item class, the
                                   prefix in its registers, no CTA-wide barrier; rows of at most 512
@@ -405,7 +406,8 @@ void fim_plan_free(fim_plan* plan);
  * (its footprint is then in use from the submission on), else to host memory; jobs whose copy is complete are
  * admitted in arrival order when a slot is free and their footprint fits the budget
  * left (a job larger than the budget runs alone), then run build (prefilter =
- * minsup), the sample estimate when sample_rate > 0, and the mine; the
+ * minsup), the sample estimate when sample_rate > 0, and the mine (at most five helper threads of the
+ * server share the submitters' copies, through 16 MB of pinned memory); the
  * database stays resident on the device until the result is copied out.
  * fim_server_wait blocks until the job is done and returns its result (owned
  * by the caller: fim_result_free), the latency from submission and the

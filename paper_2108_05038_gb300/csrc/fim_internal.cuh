@@ -122,7 +122,7 @@ enum WsSlot {
   WS_DB_BITS,
   WS_DB_SMALL,  // flags | item_rank | rank_item | supp | iota (N words each, 16-byte aligned)
   // projected DFS: per-class database parts and the warps' stacks
-  WS_PROJ_META,  // yoff (n1 u64) | toff (n1 u64) | itemoff (n1 + 1 u32) | eoffx (n1 u32)
+  WS_PROJ_META,  // yoff (n1 u64) | toff (n1 u64) | itemoff (n1 + 1 u32) | eoffx | goff (n1 u32) | tileoff (n1 + 1 u32)
   WS_PROJ_Y,     // bitmaps of every class's survivors over the class's transactions
   WS_PROJ_T,     // the transactions (tids) of every projected class
   WS_PSTACK,     // per-warp DFS stacks
@@ -135,7 +135,7 @@ enum WsSlot {
   WS_SUB_TILES,  // tiles of pairs of its later rounds
   WS_SUB_LISTS,  // row lists of its later rounds
   WS_SUB_STATE,
-  WS_LEVELS,     // arenas of the search by levels
+  WS_LEVELS,     // arenas of the search by levels (44 MB)
   WS_FILT_TABLE, // closed / maximal output: hash table and flags
   WS_FILT_OFF,   // the kept itemsets: offsets
   WS_FILT_ITEMS, // items
@@ -399,7 +399,7 @@ struct alignas(32) SubTile {
   uint32_t roff4, list, path_len, n;
   uint32_t goff, blocks, chunk, pad;  // blocks of rows (a | b << 16), words
 };
-struct alignas(32) SubUnit {  // rows j0 .. of a part's own region, over 256 words of the source region
+struct alignas(32) SubUnit {  // rows j0 .. of a part's own region, over kUnitWords (512) words of the source region
   uint32_t src4, list, path_len_cnt, j0;  // (path_len | rows << 16)
   uint32_t dst_lo, dst_hi, stride, unit;  // words of Y; unit | words << 16
 };
@@ -758,7 +758,7 @@ struct ProjLaunch {
   uint32_t* G;
   uint64_t g_cap;
   uint32_t* goff;        // n1, by class: word offset in G, or kNoGram
-  uint32_t* tileoff;     // n1 + 1, by queue position: tiles of k_gram
+  uint32_t* tileoff;     // n1 + 1, by queue position: tiles of k_sub's first round
 };
 struct SubLaunch {
   uint32_t* Y;

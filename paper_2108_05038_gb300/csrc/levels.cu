@@ -23,7 +23,7 @@
 //
 // Measured (level-2 lists, queue and search): dense_deep 107 -> 74 us, tiny 65 -> 48 us, its 738-row sample 70 -> 45 us.  What
 // bounds a level (about 8 us) is its chain of about six dependent L2 round trips: unit, rows, words, reservation, and the
-// next launch or barrier.
+// next launch or wait.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -41,9 +41,10 @@ constexpr uint32_t kLevSeg4 = 128;    // 16-byte words of a unit for one warp (5
 constexpr uint32_t kLevPath = 62;     // longest prefix (rows)
 constexpr uint32_t kLevSingles = 3;   // levels launched by themselves
 constexpr uint32_t kLevFew = 5;       // at most so many survivors: all their subsets counted at once
-// Longest rows for that with two survivors, with three to five.  One warp goes through the words, so that long rows take
-// longer than the levels they save: with no such limit dense_deep (1,568 words) takes 131 us a replay, with it 121; without
-// the pass for three to five survivors tiny (320 words) takes 270 us a step, with it 248.
+// Longest rows for that with two survivors, with three to five: one warp goes through the words, so that long rows take longer
+// than the levels they save.  Searches of 2,800 to 3,500 itemsets (75 dense items, 300 of patterns) without the pass, with it
+// for two, with it for up to five survivors, us: rows of 384 words 62, 56, 52 and 56, 56, 54; 512 words 64, 58, 58 and 56,
+// 56, 58; 640 words 62, 56, 60 and 56, 54, 62; 800 words 64, 64, 66 and 58, 60, 70; 1,184 words 72, 74, 80 and 62, 66, 88.
 constexpr uint32_t kLevPairWords = 800, kLevFewWords = 400;
 
 __device__ __forceinline__ uint32_t tri_off(uint32_t m, uint32_t n) { return m * n - m * (m + 1) / 2; }  // of (m, m + 1)
