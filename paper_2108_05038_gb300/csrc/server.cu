@@ -15,7 +15,6 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
-#include <functional>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -51,14 +50,16 @@ class Crew {
     for (auto& t : threads_) t.join();
   }
   // f(0) .. f(n - 1) (one caller at a time; f does not throw)
-  void run(uint64_t n, const std::function<void(uint64_t)>& f) {
+  template <typename F>
+  void run(uint64_t n, const F& f) {
     if (n <= 2 || threads_.empty()) {
       for (uint64_t k = 0; k < n; ++k) f(k);
       return;
     }
     {
       std::lock_guard<std::mutex> lock(mu_);
-      f_ = &f;
+      ctx_ = &f;
+      call_ = [](const void* ctx, uint64_t k) { (*static_cast<const F*>(ctx))(k); };
       n_ = n;
       next_ = 0;
       open_ = true;
@@ -79,7 +80,7 @@ class Crew {
  private:
   static constexpr std::chrono::microseconds kLookOut{100};
   void pieces() {
-    for (uint64_t k; (k = next_.fetch_add(1)) < n_;) (*f_)(k);
+    for (uint64_t k; (k = next_.fetch_add(1)) < n_;) call_(ctx_, k);
   }
   void help() {
     uint64_t seen = 0;
@@ -103,7 +104,8 @@ class Crew {
   }
   std::mutex mu_;
   std::condition_variable cv_open_, cv_idle_;
-  const std::function<void(uint64_t)>* f_ = nullptr;
+  const void* ctx_ = nullptr;
+  void (*call_)(const void*, uint64_t) = nullptr;
   uint64_t n_ = 0;
   std::atomic<uint64_t> next_{0}, turn_{0};
   uint32_t busy_ = 0;
