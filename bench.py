@@ -47,12 +47,12 @@ L2_FLUSH_BYTES = 512 << 20
 # pair kernel; "dfs": the mine's DFS stage (projection + DFS + fallback, or the one DFS launch); "step": the
 # build, estimate and mine launches (the closed/maximal flags pass of --mode once excluded).
 CAPTURES = {
-    "large_sparse": {"sources_sha256": "af555861c67a57ddcd59e6285bd6a6136fb737133666872cf46f7fc5ea750a44",
+    "large_sparse": {"sources_sha256": "ae6993276334fa731f05dcd4bdfc3ff0c5567981330f3809c5d9bdaf6336a68f",
                      "date": "2026-12-05", "summary": "profiles/launches_large_sparse.md",
-                     "kernels": {"pair": 615785984, "dfs": 854484224}, "step": 2371895552},
-    "sparse_mid": {"sources_sha256": "af555861c67a57ddcd59e6285bd6a6136fb737133666872cf46f7fc5ea750a44",
+                     "kernels": {"pair": 615863040, "dfs": 853720320}, "step": 2365527296},
+    "sparse_mid": {"sources_sha256": "ae6993276334fa731f05dcd4bdfc3ff0c5567981330f3809c5d9bdaf6336a68f",
                    "date": "2026-12-05", "summary": "profiles/launches_sparse_mid.md",
-                   "kernels": {"pair": 6446336, "dfs": 8173056}, "step": 38259200},
+                   "kernels": {"pair": 6446592, "dfs": 8175616}, "step": 38249216},
 }
 MAX_ITEMSETS_PER_JOB = 4_000_000  # serving: jobs whose output passes this are stopped and counted as rejected
 
@@ -328,8 +328,9 @@ def run_ours(args):
                                  "per survivor and transaction, bitmaps written) and per class node its prefix and "
                                  "candidates over its region's width; the regions (tens of MB) stay in the 129 MB L2"
                                  if proj else
-                                 "algorithmic bytes count every candidate row in full (the dense definition); the "
-                                 "kernel reads row words only under nonzero prefix words")}
+                                 "algorithmic bytes count every candidate row in full (the dense definition)" +
+                                 ("" if stats["search"] == 6 else
+                                  "; the kernel reads row words only under nonzero prefix words"))}
         elif by_tx:  # level 2 counted from the transactions: one addition in L2 per pair of a transaction's items
             adds = tx_additions(w, minsup, stats["pair_rows_tx"]) / (pair_avg * 1e-3) / 1e9
             roofline = {"kernel": "k_pair_tx" + (" + k_pair_mma_fused" if stats["pair_kernel"] == 4 else ""),

@@ -233,9 +233,9 @@ struct fim_db {
   std::vector<uint32_t> rank_item, supp;
   std::vector<int32_t> item_rank;
 
-  // A served job's: without the search by levels and the small-subtree walk, whose arenas (44 and 97 MB) its short-lived
-  // database would need as well (2,000 served requests, four slots: p50 2.7 ms with them in the samples' mines, 1.3 without;
-  // p99 136 and 141).
+  // A served job's: its sample without the search by levels and the small-subtree walk, whose arenas (44 and 97 MB) are not
+  // in the footprint that the server's budget reckons with.  (2,000 requests, four slots: p50 0.58, p99 134 ms; with them
+  // 0.57 and 126.)
   bool served = false;
 
   // searches by levels that outgrew their arenas (of the whole database; of samples): such a search is not tried
