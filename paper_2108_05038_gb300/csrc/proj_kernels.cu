@@ -699,6 +699,7 @@ __global__ void __launch_bounds__(kProjThreads, kProjCtasPerSm) k_dfs_proj(const
         if (off + size > p.arena_words) off = ~0ull;
       }
       const bool fits = off != ~0ull;
+      if (!fits) off = 0;  // (an item's region is never ~0, which tells a warp that nothing is left)
       if (fits) build_region(Yar + off, V, pre, list, n, xlen, supp, tmp);
       __threadfence();
       __syncwarp();

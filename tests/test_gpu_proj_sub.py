@@ -133,6 +133,20 @@ def test_large_subtree_without_room():
         db.free()
 
 
+@pytest.mark.parametrize("words", [3_000, 20_000, 100_000])
+@pytest.mark.parametrize("name", ["many_rows", "deep"])
+def test_hand_out_without_room(searched, name, words):
+    """Frames that the projected DFS would hand to other warps (all of three survivors or more) where the arena has no room
+    for their database parts: the warps keep them, and the slots reserved for them are passed over."""
+    db, minsup, want, ref = searched(name)
+    got = db.mine(minsup, dfs_mode=fim.FIM_DFS_PROJECTED, class_work=True, class_order="uniform", proj_split_words=1,
+                  proj_bitmap_words=words, walk=dict(words=1))
+    assert got.as_dict() == want and got.stats["search"] == fim.FIM_DFS_PROJECTED and got.stats["n_proj_classes"] > 0
+    for key in ("n_intersections", "n_classes", "n_queue_entries", "n_frequent", "n_items_out", "max_len"):
+        assert got.stats[key] == ref.stats[key], key
+    assert np.array_equal(got.class_work, ref.class_work)
+
+
 def test_class_bitmaps_past_32_bit_offsets(searched):
     """With a budget that lets a class region hold 2^32 words the walk, whose row offsets have 32 bits, is left out."""
     db, minsup, want, ref = searched("many_rows")
