@@ -47,12 +47,12 @@ L2_FLUSH_BYTES = 512 << 20
 # pair kernel; "dfs": the mine's DFS stage (projection + DFS + fallback, or the one DFS launch); "step": the
 # build, estimate and mine launches (the closed/maximal flags pass of --mode once excluded).
 CAPTURES = {
-    "large_sparse": {"sources_sha256": "ae6993276334fa731f05dcd4bdfc3ff0c5567981330f3809c5d9bdaf6336a68f",
+    "large_sparse": {"sources_sha256": "584dd6c85534981765a59b4b60c4d38ffed9305c5c30bd22611972716ec1f7ac",
                      "date": "2026-12-05", "summary": "profiles/launches_large_sparse.md",
-                     "kernels": {"pair": 615863040, "dfs": 853720320}, "step": 2365527296},
-    "sparse_mid": {"sources_sha256": "ae6993276334fa731f05dcd4bdfc3ff0c5567981330f3809c5d9bdaf6336a68f",
+                     "kernels": {"pair": 615792896, "dfs": 854352896}, "step": 2371365888},
+    "sparse_mid": {"sources_sha256": "584dd6c85534981765a59b4b60c4d38ffed9305c5c30bd22611972716ec1f7ac",
                    "date": "2026-12-05", "summary": "profiles/launches_sparse_mid.md",
-                   "kernels": {"pair": 6446592, "dfs": 8175616}, "step": 38249216},
+                   "kernels": {"pair": 6449408, "dfs": 8173056}, "step": 38248192},
 }
 MAX_ITEMSETS_PER_JOB = 4_000_000  # serving: jobs whose output passes this are stopped and counted as rejected
 
